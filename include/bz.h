@@ -237,8 +237,9 @@ bz_status bz_step_rk(bz_plan *plan, void *fhat, int dtype, double *t, double dt,
 bz_status bz_moments(bz_plan *plan, const void *fhat, int dtype, double out[5], void *stream);
 
 /* F(k, r_i, qhat_j) in FP64 for `count` entries (device arrays): k_idx[3e..3e+2] array
- * indices in [0, N), term[e] in [0, P); out[2e], out[2e+1] = re, im.  Uses the same
- * device code as the plan's table (before the FP32 store).  Synchronous. */
+ * indices in [0, N), term[e] in [0, P); out[2e], out[2e+1] = re, im.  Sums the theta rule
+ * of the radial node directly; in 3D the plan's table takes the same rule through a Legendre
+ * series (they agree to FP64 rounding before the table's FP32 store).  Synchronous. */
 bz_status bz_ftable_entries(bz_plan *plan, int count, const int *k_idx, const int *term,
                             double *out);
 

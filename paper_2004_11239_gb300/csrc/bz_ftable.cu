@@ -6,8 +6,20 @@
 //     + 2 pi sum_n W_n [ (exp(i x c_n) - 1) J0(y s_n) + (J0(y s_n) - 1) ]   (part II, [eps, pi])
 // with c_n = 1 - cos t_n, s_n = sin t_n, W_n = w_n g(t_n) from the host rule of the
 // radial node.  The table stores alpha_p(k) = c_p F / N^3 in FP32 (the N^-3 of the
-// forward transform folded in).  J0 is CUDA's double-precision j0; J0 - 1 uses its
-// power series for small arguments to avoid cancellation.
+// forward transform folded in).
+//
+// Two evaluations of part II:
+//   * single entries (bz_ftable_entries) sum the rule as written above, with CUDA's
+//     double-precision j0; J0 - 1 uses its power series for small arguments.
+//   * the plan's table takes the same sum through the addition theorem (Funk-Hecke): with
+//     z = a |k|, chi the angle between k and qhat and exp(-i z khat.sigma) =
+//     sum_l (2l + 1) (-i)^l j_l(z) P_l(khat.sigma),
+//       part II = exp(i x) sum_{l >= 1} (2l + 1) (-i)^l j_l(z) mu_l P_l(cos chi),
+//       mu_l = 2 pi sum_n W_n (P_l(cos t_n) - 1).
+//     The rule enters through the mu_l only (one short sum per l on the host), j_l(z) depends on
+//     (r_i, |k|^2) only (k_legendre_coef, one row per radial node and |k|^2), and an entry is a
+//     Legendre series of about z + 25 terms of three FP64 operations, against a few hundred rule
+//     nodes of some hundred operations each.
 #include <cmath>
 #include <vector>
 
@@ -55,23 +67,89 @@ struct TableArgs {
     const double *rule;      // concatenated omc | sn | W per radial node
     const int *rule_off;     // [N_rho + 1]
     float2 *alpha;           // [P][N^3]
+    // 3D: the Legendre coefficients of radial nodes i0 .. (k_legendre_coef)
+    int i0, g0, nkk, stride; // node of blockIdx.z = 0, term group of blockIdx.y = 0
+    const double *coef;
+    const int *cut;
 };
 
-// grid: x over N^3 / blockDim, y over terms p0 + blockIdx.y
-__global__ void ftable_kernel(TableArgs a) {
-    extern __shared__ double sm[];
-    const int p = a.p0 + blockIdx.y;
-    const int i = p / a.M;
-    const int off = a.rule_off[i];
-    const int n = a.rule_off[i + 1] - off;
-    double *omc = sm, *sn = sm + n, *W = sm + 2 * n;
-    const double *src = a.rule + 3 * (size_t)off;
-    for (int t = threadIdx.x; t < 3 * n; t += blockDim.x) sm[t] = src[t];
+// Coefficients of the Legendre series: row (radial node i, m = |k|^2) holds
+// coef[l] = mu'_l j_l(z), z = pi r_i sqrt(m) / (2L), l = 0 .. cut - 1, where mu'_l carries (2l + 1), the
+// sign of (-i)^l and the scale of the recurrence's polynomials; cut (even) drops the tail below
+// 2^-60 of the row's largest.  j_l by downward recurrence from lmax (where |j_l| < 1e-22 for the
+// largest z, or from the l where that holds for this z), normalised by sum (2l + 1) j_l^2 = 1 with
+// the sign of j_0 = sin z / z or j_1.  One thread per row; the work is a few percent of the table's.
+struct CoefArgs {
+    int i0, ni, nkk, stride, lmax;
+    double L;
+    const double *r;         // [N_rho] radial nodes
+    const double *mu;        // [lmax + 1]
+    double *coef;            // [ni][nkk][stride]
+    int *cut;                // [ni][nkk]
+};
+
+__global__ void __launch_bounds__(64) k_legendre_coef(CoefArgs a) {
+    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (m >= a.nkk) return;
+    const size_t row = (size_t)blockIdx.y * a.nkk + m;
+    const double z = M_PI * a.r[a.i0 + blockIdx.y] * sqrt((double)m) / (2.0 * a.L);
+    double *c = a.coef + row * a.stride;
+    if (!(z > 0.0)) {                                     // k = 0: F = 0
+        a.cut[row] = 0;
+        return;
+    }
+    // |j_l(z)| <= z^l / (2l + 1)!!: the first l where this is below 1e-22 of j_1's scale
+    int top = 1;
+    const double lz = log(z);
+    for (double lb = 0.0; top < a.lmax; ++top) {
+        lb += lz - log(2.0 * top + 3.0);
+        if (top > z && lb < -50.7) break;
+    }
+    const double iz = 1.0 / z;
+    double f2 = 0.0, f1 = 1e-30, norm = 0.0;              // f_{l+1}, f_l
+    for (int l = top; l >= 0; --l) {
+        if (l < a.stride) c[l] = f1;
+        norm += (2.0 * l + 1.0) * f1 * f1;
+        const double f0 = (2.0 * l + 1.0) * iz * f1 - f2;
+        f2 = f1;
+        f1 = f0;
+    }
+    double sz, cz;
+    sincos(z, &sz, &cz);
+    const double j0 = sz * iz, j1 = z < 0.1 ? z / 3.0 : (j0 - cz) * iz;
+    const double g0 = c[0], g1 = c[1];
+    double sc = 1.0 / sqrt(norm);
+    if (fabs(j0) > fabs(j1) ? (j0 < 0.0) != (g0 < 0.0) : (j1 < 0.0) != (g1 < 0.0)) sc = -sc;
+    double big = 0.0;
+    c[0] = 0.0;
+    for (int l = 1; l <= top; ++l) {
+        const double v = a.mu[l] * sc * c[l];
+        c[l] = v;
+        big = fmax(big, fabs(v));
+    }
+    int n = top;
+    while (n > 1 && fabs(c[n]) < 0x1p-60 * big) --n;
+    if ((n & 1) == 0) c[n + 1] = 0.0;                     // pairs (even, odd); stride >= lmax + 2
+    a.cut[row] = (n | 1) + 1;
+}
+
+// Thread: one mode k (of each pair k, -k) and up to kLegTerms terms of one radial node, sharing the
+// coefficient row.  The polynomials are 2^l times the monic Legendre ones, q_{l+1} = 2c q_l -
+// g_l q_{l-1}, g_l = 4 l^2 / (4 l^2 - 1): two FP64 operations a step and a third for the sum; no
+// over- or underflow for any l.  FP64 bound (this part runs about two FP64 lanes per clock and SM).
+// Measured at N = 32, P = 384 (R = 6, s = 1/2): 4.6 ms, and 0.19 ms for the rows; the direct sum over
+// the rule took 578 ms (plan creation 582 -> 8.0 ms).
+constexpr int kLegTerms = 4;
+
+__global__ void __launch_bounds__(128) ftable_kernel(TableArgs a) {
+    extern __shared__ double sg[];                        // g_l, l = 0 .. lmax + 1
+    for (int t = threadIdx.x; t < a.stride; t += blockDim.x) sg[t] = 4.0 * t * t / (4.0 * t * t - 1.0);
     __syncthreads();
-    const int n3 = a.N * a.N * a.N;
+    const int N = a.N, n3 = N * N * N;
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= n3) return;
-    const int N = a.N;
+    const int il = blockIdx.z, j0 = (a.g0 + blockIdx.y) * kLegTerms;
+    const int p0 = (a.i0 + il) * a.M + j0, np = min(kLegTerms, a.M - j0);
     int i1 = idx / (N * N), i2 = (idx / N) % N, i3 = idx % N;
     int k1 = i1 < N / 2 ? i1 : i1 - N;
     int k2 = i2 < N / 2 ? i2 : i2 - N;
@@ -90,23 +168,51 @@ __global__ void ftable_kernel(TableArgs a) {
     const bool in_k = a.nin == 0 || (k1 >= -h && k1 < h && k2 >= -h && k2 < h && k3 >= -h && k3 < h);
     const bool in_m = midx >= 0 && (a.nin == 0 || (-k1 >= -h && -k1 < h && -k2 >= -h && -k2 < h && -k3 >= -h && -k3 < h));
     if (!in_k && !in_m) {
-        a.alpha[(size_t)p * n3 + idx] = make_float2(0.f, 0.f);
-        if (midx > idx) a.alpha[(size_t)p * n3 + midx] = make_float2(0.f, 0.f);
+        for (int u = 0; u < np; ++u) {
+            a.alpha[(size_t)(p0 + u) * n3 + idx] = make_float2(0.f, 0.f);
+            if (midx > idx) a.alpha[(size_t)(p0 + u) * n3 + midx] = make_float2(0.f, 0.f);
+        }
         return;
     }
-    const double *tp = a.term + 5 * (size_t)p;
-    double r = tp[0];
-    double kap = k1 * tp[1] + k2 * tp[2] + k3 * tp[3];
-    double kk = (double)k1 * k1 + (double)k2 * k2 + (double)k3 * k3;
-    double kp2 = kk - kap * kap;
-    double kp = kp2 > 0.0 ? sqrt(kp2) : 0.0;
-    double aa = M_PI * r / (2.0 * a.L);
-    double A[3] = {a.A0, a.A1, a.A2};
-    double2 F = f_value(aa * kap, aa * kp, A, n, omc, sn, W);
-    double sc = tp[4] * a.inv_n3;
-    a.alpha[(size_t)p * n3 + idx] = in_k ? make_float2((float)(sc * F.x), (float)(sc * F.y)) : make_float2(0.f, 0.f);
-    if (midx > idx)
-        a.alpha[(size_t)p * n3 + midx] = in_m ? make_float2((float)(sc * F.x), (float)(-sc * F.y)) : make_float2(0.f, 0.f);
+    const int kk = k1 * k1 + k2 * k2 + k3 * k3;
+    const double ik = kk > 0 ? 1.0 / sqrt((double)kk) : 0.0;
+    double kap[kLegTerms], c2[kLegTerms], q0[kLegTerms], q1[kLegTerms], sr[kLegTerms], si[kLegTerms];
+    #pragma unroll
+    for (int u = 0; u < kLegTerms; ++u) {
+        const double *tp = a.term + 5 * (size_t)(p0 + (u < np ? u : 0));
+        kap[u] = k1 * tp[1] + k2 * tp[2] + k3 * tp[3];
+        c2[u] = 2.0 * fmin(1.0, fmax(-1.0, kap[u] * ik));
+        q0[u] = 1.0;                                      // q_0
+        q1[u] = c2[u];                                    // q_1 = 2 c
+        sr[u] = si[u] = 0.0;
+    }
+    const size_t row = (size_t)il * a.nkk + kk;
+    const double2 *c = (const double2 *)(a.coef + row * a.stride);
+    const int cut = a.cut[row];
+    for (int l = 0; l < cut; l += 2) {
+        const double2 cl = c[l / 2];
+        const double ga = sg[l + 1], gb = sg[l + 2];
+        #pragma unroll
+        for (int u = 0; u < kLegTerms; ++u) {
+            sr[u] = fma(cl.x, q0[u], sr[u]);
+            si[u] = fma(cl.y, q1[u], si[u]);
+            q0[u] = fma(c2[u], q1[u], -ga * q0[u]);
+            q1[u] = fma(c2[u], q0[u], -gb * q1[u]);
+        }
+    }
+    for (int u = 0; u < np; ++u) {
+        const double *tp = a.term + 5 * (size_t)(p0 + u);
+        const double aa = M_PI * tp[0] / (2.0 * a.L);
+        const double x = aa * kap[u], y2 = aa * aa * fmax((double)kk - kap[u] * kap[u], 0.0);
+        double sx, cx;
+        sincos(x, &sx, &cx);
+        const double sc = tp[4] * a.inv_n3;
+        const double fr = sc * (2.0 * M_PI * (-0.5 * x * x * a.A1 - 0.25 * y2 * a.A2) + (cx * sr[u] - sx * si[u]));
+        const double fi = sc * (2.0 * M_PI * x * a.A0 + (cx * si[u] + sx * sr[u]));
+        float2 *al = a.alpha + (size_t)(p0 + u) * n3;
+        al[idx] = in_k ? make_float2((float)fr, (float)fi) : make_float2(0.f, 0.f);
+        if (midx > idx) al[midx] = in_m ? make_float2((float)fr, (float)(-fi)) : make_float2(0.f, 0.f);
+    }
 }
 
 // 2D (Sec. 4.1 (i)): with x = a k.qhat, y = a k.qperp the odd terms cancel between parts I and
@@ -203,6 +309,89 @@ __global__ void fentries_kernel(EntryArgs a) {
 
 }  // namespace
 
+namespace {
+
+// The 3D table: mu_l on the host, then per group of radial nodes the coefficient rows and the
+// table entries.  A group's rows take at most kCoefBytes (at least one node).
+constexpr size_t kCoefBytes = (size_t)64 << 20;
+
+bz_status table3(Plan &pl, TableArgs a) {
+    const int N = pl.N, nkk = 3 * (N / 2) * (N / 2) + 1;
+    double rmax = 0.0;
+    std::vector<double> r(pl.N_rho);
+    for (int i = 0; i < pl.N_rho; ++i) {
+        r[i] = pl.terms.r[(size_t)i * pl.M];
+        rmax = r[i] > rmax ? r[i] : rmax;
+    }
+    // lmax: |j_l(z)| <= z^l / (2l + 1)!! < 1e-22 beyond it for every z of the plan
+    const double zmax = M_PI * rmax * std::sqrt((double)(nkk - 1)) / (2.0 * pl.L);
+    int lmax = 1;
+    for (double lb = 0.0; !(lmax > zmax && lb < -50.7); ++lmax) lb += std::log(zmax) - std::log(2.0 * lmax + 3.0);
+    const int stride = (lmax + 4) & ~1;
+    // mu'_l = 2 pi sum_n W_n (P_l(cos t_n) - 1) times (2l + 1), the sign of (-i)^l (the sum over odd l
+    // is the imaginary part) and P_l / q_l; D_l = P_l - 1 by its own recurrence (no cancellation at
+    // small angles), on the rule with the most nodes
+    const ThetaRule *R = &pl.rules[0];
+    for (const ThetaRule &q : pl.rules)
+        if (q.W.size() > R->W.size()) R = &q;
+    std::vector<double> mu(lmax + 1, 0.0);
+    for (size_t n = 0; n < R->W.size(); ++n) {
+        const double omc = R->omc[n], c = 1.0 - omc;
+        double d0 = 0.0, d1 = -omc;                        // D_0, D_1
+        for (int l = 1; l <= lmax; ++l) {
+            mu[l] += R->W[n] * d1;
+            const double d2 = ((2.0 * l + 1.0) * (c * d1 - omc) - l * d0) / (l + 1.0);
+            d0 = d1;
+            d1 = d2;
+        }
+    }
+    double lead = 1.0;                                     // P_l / q_l = (2l)! / (4^l l!^2)
+    for (int l = 1; l <= lmax; ++l) {
+        lead *= (2.0 * l - 1.0) / (2.0 * l);
+        const double sign = (l & 3) == 0 || (l & 3) == 3 ? 1.0 : -1.0;   // (-i)^l: -i, -1, i, 1
+        mu[l] *= 2.0 * M_PI * (2.0 * l + 1.0) * sign * lead;
+    }
+    const size_t row = (size_t)nkk * stride * sizeof(double);
+    int ni = (int)(kCoefBytes / row);
+    const int groups = (pl.M + kLegTerms - 1) / kLegTerms;
+    if (ni > 65535) ni = 65535;                            // gridDim limit
+    if (ni < 1) ni = 1;
+    if (ni > pl.N_rho) ni = pl.N_rho;
+    const size_t gsm = (size_t)stride * sizeof(double);
+    if (gsm > 48 * 1024)
+        BZ_CUDA_TRY(cudaFuncSetAttribute(ftable_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm));
+    double *buf = nullptr;                                 // coefficient rows, r, mu, row lengths
+    const size_t head = r.size() + mu.size();
+    if (cudaMalloc(&buf, ni * row + head * sizeof(double) + (size_t)ni * nkk * sizeof(int)) != cudaSuccess) {
+        cudaGetLastError();
+        return BZ_ERR_OOM;
+    }
+    double *coef = buf, *r_dev = coef + ni * row / sizeof(double), *mu_dev = r_dev + r.size();
+    int *cut = (int *)(mu_dev + mu.size());
+    cudaError_t e = cudaMemcpy(r_dev, r.data(), r.size() * sizeof(double), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(mu_dev, mu.data(), mu.size() * sizeof(double), cudaMemcpyHostToDevice);
+    CoefArgs ca;
+    ca.nkk = nkk; ca.stride = stride; ca.lmax = lmax; ca.L = pl.L; ca.r = r_dev; ca.mu = mu_dev; ca.coef = coef;
+    ca.cut = cut;
+    a.nkk = nkk; a.stride = stride; a.coef = coef; a.cut = cut;
+    for (int i0 = 0; e == cudaSuccess && i0 < pl.N_rho; i0 += ni) {
+        const int n = pl.N_rho - i0 < ni ? pl.N_rho - i0 : ni;
+        ca.i0 = a.i0 = i0;
+        ca.ni = n;
+        k_legendre_coef<<<dim3((nkk + 63) / 64, n), 64>>>(ca);
+        for (a.g0 = 0; a.g0 < groups; a.g0 += 65535) {
+            const int ng = groups - a.g0 < 65535 ? groups - a.g0 : 65535;
+            ftable_kernel<<<dim3((N * N * N + 127) / 128, ng, n), 128, gsm>>>(a);
+        }
+        e = cudaGetLastError();
+    }
+    const cudaError_t es = cudaDeviceSynchronize();
+    cudaFree(buf);
+    return e == cudaSuccess && es == cudaSuccess ? BZ_OK : BZ_ERR_CUDA;
+}
+
+}  // namespace
+
 // Uploads terms and theta rules; fills pl.alpha with c_p F / N^3 (FP32).
 bz_status ftable_build(Plan &pl) {
     const int P = pl.P, N = pl.N;
@@ -233,22 +422,20 @@ bz_status ftable_build(Plan &pl) {
 
     const size_t smem = 3 * (size_t)pl.rule_max * sizeof(double);
     if (smem > 200 * 1024) return BZ_ERR_UNSUPPORTED;
-    if (smem > 48 * 1024) {
-        BZ_CUDA_TRY(cudaFuncSetAttribute(ftable_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        BZ_CUDA_TRY(cudaFuncSetAttribute(ftable2d_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    }
-    TableArgs a;
+    TableArgs a = {};
     a.N = N; a.M = pl.M; a.P = P; a.L = pl.L; a.nin = pl.Nin;
     a.inv_n3 = 1.0 / (double)modes(pl);      // the forward transform's N^-d
     a.A0 = pl.A[0]; a.A1 = pl.A[1]; a.A2 = pl.A[2];
     a.term = pl.term_dev; a.rule = pl.rule_buf; a.rule_off = pl.rule_off; a.alpha = pl.alpha;
+    if (pl.dim != 2) return table3(pl, a);
+    if (smem > 48 * 1024)
+        BZ_CUDA_TRY(cudaFuncSetAttribute(ftable2d_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int n3 = (int)modes(pl), bs = 128;
     const int ychunk = 32768;   // gridDim.y limit
     for (int p0 = 0; p0 < P; p0 += ychunk) {
         a.p0 = p0;
         dim3 grid((n3 + bs - 1) / bs, (P - p0) < ychunk ? (P - p0) : ychunk);
-        if (pl.dim == 2) ftable2d_kernel<<<grid, bs, smem>>>(a);
-        else ftable_kernel<<<grid, bs, smem>>>(a);
+        ftable2d_kernel<<<grid, bs, smem>>>(a);
         BZ_CUDA_TRY(cudaGetLastError());
     }
     BZ_CUDA_TRY(cudaDeviceSynchronize());
