@@ -142,7 +142,8 @@ typedef struct {
     int chunk_terms;  /* terms per pipeline chunk; <= 0 selects automatically          */
     int pipeline;     /* BZ_PIPE_*; BZ_ERR_UNSUPPORTED if FUSED cannot run for this N     */
     int cluster;      /* FUSED: CTAs per cluster (N=16: 1|2, 24: 2|3, 32: 4|8); <= 0 times the
-                         compiled sizes at creation and keeps the fastest                   */
+                         compiled sizes at creation and keeps the fastest (BZ_DATA_REAL at N = 32:
+                         see ctas_per_sm)                                                   */
     int h_precision;  /* BZ_H_*                                                            */
     int conv;         /* BZ_CONV_*                                                         */
     int dim;          /* 3 (or 0): the 3D operator; 2: the 2D operator of Sec. 4.1 (i) and Sec. 5.2 on
@@ -158,8 +159,9 @@ typedef struct {
     int ctas_per_sm;  /* fused pipeline, BZ_DATA_REAL at N = 32: 2 runs k_fused, 3 the three-CTA-
                          per-SM pair kernel k_pair3 (sum over pairs and fhat column in tensor
                          memory; with BZ_H_FP32 its h comes from one FP32 plane pass and one
-                         pencil pass); <= 0 times both at creation and keeps the faster.  Any
-                         other plan: must be <= 0 or 2, else BZ_ERR_UNSUPPORTED.              */
+                         pencil pass); <= 0 (and cluster <= 0) runs k_col32, one term per SM;
+                         <= 0 with a cluster size times that size's kernels and keeps the
+                         faster.  Any other plan: must be <= 0 or 2, else BZ_ERR_UNSUPPORTED. */
 } bz_plan_desc;
 
 /* Creates a plan: quadrature terms, the FP64 F table (computed on the device, stored
@@ -181,9 +183,9 @@ bz_status bz_plan_info(const bz_plan *plan, int *P, size_t *alpha_bytes, size_t 
  * *tuned_ms = the timed collide that selected the cluster size.  Any pointer may be NULL. */
 bz_status bz_plan_pipeline(const bz_plan *plan, int *pipeline, int *cluster, int *clusters, float *tuned_ms);
 
-/* Name of the kernel that carries the plan's per-term work: "k_fused", "k_pair3" (the
- * three-CTA-per-SM pair kernel of a BZ_DATA_REAL plan at N = 32), "k_mixed", "k_collide_2d"
- * or "chunked"; NULL for a NULL plan.  The string is static. */
+/* Name of the kernel that carries the plan's per-term work: "k_fused", "k_col32" (a
+ * BZ_DATA_REAL plan at N = 32), "k_pair3" (the same on request, ctas_per_sm = 3), "k_mixed",
+ * "k_collide_2d" or "chunked"; NULL for a NULL plan.  The string is static. */
 const char *bz_plan_kernel(const bz_plan *plan);
 
 /* Copies the term list to host arrays of length P (any may be NULL):

@@ -31,6 +31,8 @@ void free_plan(bz::Plan &p) {
     cudaFree(p.term_dev); cudaFree(p.S); cudaFree(p.h); cudaFree(p.fin); cudaFree(p.acc);
     cudaFree(p.rk); cudaFree(p.mom); cudaFree(p.part); cudaFree(p.fin64); cudaFree(p.scr64);
     cudaFree(p.wimg); cudaFree(p.dev_err); cudaFree(p.apair); cudaFree(p.fsym); cudaFree(p.fsym64);
+    cudaFree(p.acol); cudaFree(p.fcol); cudaFree(p.hcol);
+    p.acol = nullptr; p.fcol = nullptr; p.hcol = nullptr;
     cudaFree(p.cpair); cudaFree(p.part_s); cudaFree(p.S_s); cudaFree(p.acc_s);
     for (int e = 0; e < bz::kExtraStreams; ++e) {
         cudaFree(p.xS[e]); cudaFree(p.xS_s[e]); cudaFree(p.xacc[e]); cudaFree(p.xacc_s[e]);
@@ -71,6 +73,30 @@ std::vector<float2> make_twiddles(const bz::Plan &pl) {
                 tw[((size_t)p * 3 + d) * N + i] = make_float2((float)std::cos(ph), (float)std::sin(ph));
             }
     return tw;
+}
+
+// k_col32's plan: one CTA per SM, nothing to select.  tuned_ms is one timed collide of a zero field.
+bz_status setup_col32(bz::Plan &pl) {
+    int G = 0;
+    if (bz::col32_setup(&G) != cudaSuccess || G <= 0) return BZ_ERR_CUDA;
+    const size_t part = (size_t)G * bz::kCol32Part * sizeof(float2);
+    if (dmalloc(&pl.part, part) != BZ_OK) return BZ_ERR_OOM;
+    pl.use_fused = 1; pl.fused_C = 1; pl.fused_G = G;
+    pl.ws_bytes += part;
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    bz_status s = cudaMemset(pl.fin, 0, (size_t)pl.N * pl.N * pl.N * sizeof(float2)) == cudaSuccess ? BZ_OK : BZ_ERR_CUDA;
+    if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) s = BZ_ERR_CUDA;
+    if (s == BZ_OK) s = bz::collide_fused(pl, 0, pl.P, nullptr, nullptr);     // warm-up
+    if (s == BZ_OK) {
+        cudaEventRecord(e0);
+        s = bz::collide_fused(pl, 0, pl.P, nullptr, nullptr);
+        cudaEventRecord(e1);
+        if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&pl.fused_ms, e0, e1) != cudaSuccess)
+            s = BZ_ERR_CUDA;
+    }
+    if (e0) cudaEventDestroy(e0);
+    if (e1) cudaEventDestroy(e1);
+    return s;
 }
 
 // Times one full collide of a zero field for each compiled cluster size (or only `forced`)
@@ -222,7 +248,16 @@ bz_status create(bz_plan **out, const bz_plan_desc *d) {
         return BZ_ERR_CUDA;
     }
     s = bz::ftable_build(pl);
-    if (s == BZ_OK && pl.real) {
+    // real data at N = 32: k_col32, unless a cluster size or a pair kernel is asked for.  RK4 at
+    // P = 1024 took 191 us a collide with the faster of k_fused and k_pair3 (timed here until then).
+    pl.col32 = pl.real && N == 32 && d->pipeline != BZ_PIPE_CHUNKED && d->cluster <= 0 && d->ctas_per_sm <= 0;
+    if (s == BZ_OK && pl.col32) {
+        if ((s = dmalloc(&pl.acol, (size_t)pl.P * bz::kCol32Part * sizeof(float2))) == BZ_OK &&
+            (s = dmalloc(&pl.fcol, field)) == BZ_OK && (s = dmalloc(&pl.hcol, n3 * sizeof(float))) == BZ_OK &&
+            (s = dmalloc(&pl.fsym, field)) == BZ_OK && (s = dmalloc(&pl.fsym64, n3 * sizeof(double2))) == BZ_OK)
+            s = bz::col32_table(pl);
+        pl.ws_bytes += 2 * field + n3 * (sizeof(float) + sizeof(double2));
+    } else if (s == BZ_OK && pl.real) {
         // term pairs (2q, 2q + 1) share a radial node (M even) and one pair of transforms
         const size_t ns = (size_t)3 * N * N;
         if ((s = dmalloc(&pl.apair, (size_t)(pl.P / 2) * field)) == BZ_OK &&
@@ -258,8 +293,17 @@ bz_status create(bz_plan **out, const bz_plan_desc *d) {
     if (d->pipeline != BZ_PIPE_CHUNKED && N <= 32) {
         if (dmalloc(&pl.fin64, n3 * sizeof(double2)) == BZ_OK && dmalloc(&pl.scr64, n3 * sizeof(double2)) == BZ_OK) {
             pl.ws_bytes += 2 * n3 * sizeof(double2);
-            if (select_fused(pl, d->cluster, d->ctas_per_sm) != BZ_OK) cudaGetLastError();
+            if (pl.col32) s = setup_col32(pl);
+            else if (select_fused(pl, d->cluster, d->ctas_per_sm) != BZ_OK) cudaGetLastError();
+        } else if (pl.col32) {
+            s = BZ_ERR_OOM;
         }
+    }
+    if (s != BZ_OK) {                         // k_col32's plan has no other pipeline's tables
+        cudaGetLastError();
+        free_plan(pl);
+        delete h;
+        return s;
     }
     if ((d->pipeline == BZ_PIPE_FUSED || pl.precision == BZ_PREC_BF16X3) && !pl.use_fused) {
         free_plan(pl);
@@ -317,7 +361,7 @@ bz_status bz_plan_info(const bz_plan *plan, int *P, size_t *alpha_bytes, size_t 
     size_t n3 = bz::modes(p);
     if (P) *P = p.P;
     if (alpha_bytes)
-        *alpha_bytes = ((size_t)p.P * n3 + (p.real ? (size_t)(p.P / 2) * (n3 + 3 * (size_t)p.N * p.N) : 0)) *
+        *alpha_bytes = ((size_t)p.P * n3 + (p.col32 ? (size_t)p.P * bz::kCol32Part : p.real ? (size_t)(p.P / 2) * (n3 + 3 * (size_t)p.N * p.N) : 0)) *
                        sizeof(float2);
     if (workspace_bytes) *workspace_bytes = p.ws_bytes;
     return BZ_OK;
@@ -329,7 +373,7 @@ const char *bz_plan_kernel(const bz_plan *plan) {
     if (p.dim == 2) return "k_collide_2d";
     if (!p.use_fused) return "chunked";
     if (p.precision == BZ_PREC_BF16X3) return "k_mixed";
-    return p.pair3 ? "k_pair3" : "k_fused";
+    return p.col32 ? "k_col32" : p.pair3 ? "k_pair3" : "k_fused";
 }
 
 bz_status bz_plan_pipeline(const bz_plan *plan, int *pipeline, int *cluster, int *clusters, float *tuned_ms) {

@@ -258,6 +258,78 @@ __global__ void k_batch_rk_out(const double2 *f0, const int *slots, const int *c
     }
 }
 
+// k_col32's items (part [nblk][18][32][32], bz_col32.cu): block (k1, instance) sums the planes k1
+// and -k1 of the half spectrum and turns them around in shared memory, so that the sums are read
+// and the natural-order modes (k1, k2, k3) of `sink` written in runs of 32.
+template <class Sink>
+__device__ __forceinline__ void col_modes_of(const float2 *part, int nblk, int slot, int k1, Sink sink) {
+    constexpr int N = 32, N2 = N * N, H = N / 2;
+    __shared__ double2 s1[H + 1][N + 1], s2[H][N + 1];    // [k3][k2] of k1; of the modes whose conjugates
+                                                           // are (k1, -k2, -k3)
+    const int m1 = (N - k1) % N;
+    const float2 *base = part + (size_t)slot * nblk * kCol32Part;
+    for (int e = threadIdx.x; e < (2 * H + 1) * N; e += blockDim.x) {
+        const int r = e / N, v = e % N, k3 = r <= H ? r : r - H;
+        size_t at = (size_t)k3 * N2 + (r <= H ? k1 : m1) * N + v;
+        if (r > H && k1 == H) at = (size_t)17 * N2 + k3 * N + v;
+        else if (r > H && v == H) at = (size_t)17 * N2 + (H + k3) * N + m1;
+        if (r > H && k3 >= H) continue;
+        const double2 q = sum_blocks(base + at, 0, nblk, (int)kCol32Part, 0);
+        if (r <= H) s1[k3][v] = q;
+        else s2[k3][v] = q;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < N2; e += blockDim.x) {
+        const int k2 = e / N, k3 = e % N;
+        double2 q;
+        if (k3 <= H) {
+            q = s1[k3][k2];
+        } else {
+            q = s2[N - k3][(N - k2) % N];
+            q.y = -q.y;
+        }
+        sink((size_t)slot * N * N2 + (size_t)k1 * N2 + e, q);
+    }
+}
+
+__global__ void __launch_bounds__(512) k_batch_out_col(const float2 *part, int nblk, const int *slots,
+                                                       const int *count_dev, void *Qhat, int dtype, int *flag) {
+    if ((int)blockIdx.y >= *count_dev) return;
+    col_modes_of(part, nblk, slots[blockIdx.y], blockIdx.x, [&](size_t idx, double2 q) {
+        if (dtype == BZ_C128) {
+            ((double2 *)Qhat)[idx] = q;
+            note_finite(q, flag);
+        } else {
+            const float2 w = make_float2((float)q.x, (float)q.y);
+            ((float2 *)Qhat)[idx] = w;
+            note_finite(w, flag);
+        }
+    });
+}
+
+__global__ void __launch_bounds__(512) k_batch_rk_stage_col(const float2 *part, int nblk, const int *slots,
+                                                            const int *count_dev, double2 *f0, double2 *fsum,
+                                                            float2 *fin, double2 *fin64, int stage, double dt) {
+    if ((int)blockIdx.y >= *count_dev) return;
+    col_modes_of(part, nblk, slots[blockIdx.y], blockIdx.x, [&](size_t idx, double2 q) {
+        rk_stage_mode(idx, q, f0, fsum, fin, fin64, stage, dt);
+    });
+}
+
+// Terms per item for k_col32: the items of a full batch run on G CTAs in waves; an item costs its
+// terms and about one more (h and the sums in, the sums out and added up).  Fewest term times.
+int col_terms(int P, int capacity, int G) {
+    int best = P;
+    double cost = 1e300;
+    for (int nblk = 1; nblk <= P && nblk <= 256; ++nblk) {
+        const int tb = (P + nblk - 1) / nblk;
+        const double waves = std::ceil((double)capacity * ((P + tb - 1) / tb) / G);
+        const double c = waves * (tb + 1.0);
+        if (c < cost) { cost = c; best = tb; }
+    }
+    return best;
+}
+
 ItemArgs item_args(const bz_batch &B) {
     const Plan &pl = *B.pl;
     ItemArgs a;
@@ -267,6 +339,7 @@ ItemArgs item_args(const bz_batch &B) {
     a.p0 = 0; a.p1 = B.units; a.TB = B.TB; a.nblk = B.nblk; a.M = pl.M; a.N_rho = pl.N_rho;
     if (pl.real) {                                   // units are term pairs
         a.real = 1; a.fin = B.fsym; a.alpha = pl.apair; a.cpair = pl.cpair; a.part_s = B.part_s;
+        if (pl.col32) a.alpha = pl.acol;             // (units are terms)
     }
     return a;
 }
@@ -463,7 +536,7 @@ bz_status bz_batch_create(bz_batch **out, const bz_plan *plan, int capacity, int
     bz_batch *B = new (std::nothrow) bz_batch();
     if (!B) return BZ_ERR_OOM;
     B->pl = pl;
-    B->units = pl->real ? pl->P / 2 : pl->P;
+    B->units = pl->real && !pl->col32 ? pl->P / 2 : pl->P;
     B->capacity = capacity;
     B->gamma.assign(capacity, pl->gamma);
     const size_t n3 = (size_t)pl->N * pl->N * pl->N;
@@ -500,7 +573,8 @@ bz_status bz_batch_create(bz_batch **out, const bz_plan *plan, int capacity, int
         return fail(BZ_ERR_OOM);
     }
     if (upload_gsc(*B) != BZ_OK) return fail(BZ_ERR_CUDA);
-    int tb = pl->real && terms_per_item > 0 ? (terms_per_item + 1) / 2 : terms_per_item;   // in units
+    int tb = pl->real && !pl->col32 && terms_per_item > 0 ? (terms_per_item + 1) / 2 : terms_per_item;   // in units
+    if (tb <= 0 && pl->col32) tb = col_terms(pl->P, capacity, pl->fused_G);
     if (tb <= 0) {
         // autotune on a trial of up to 4 instances per resident cluster
         int trial = capacity < 4 * pl->fused_G ? capacity : 4 * pl->fused_G;
@@ -524,8 +598,8 @@ bz_status bz_batch_create(bz_batch **out, const bz_plan *plan, int capacity, int
     }
     B->TB = tb < B->units ? tb : B->units;
     B->nblk = (B->units + B->TB - 1) / B->TB;
-    if (cudaMalloc(&B->part, (size_t)capacity * B->nblk * field) != cudaSuccess ||
-        (pl->real && cudaMalloc(&B->part_s, (size_t)capacity * B->nblk * 3 * pl->N * pl->N * sizeof(float2)) !=
+    if (cudaMalloc(&B->part, (size_t)capacity * B->nblk * (pl->col32 ? kCol32Part * sizeof(float2) : field)) != cudaSuccess ||
+        (pl->real && !pl->col32 && cudaMalloc(&B->part_s, (size_t)capacity * B->nblk * 3 * pl->N * pl->N * sizeof(float2)) !=
                          cudaSuccess)) {
         cudaGetLastError();
         return fail(BZ_ERR_OOM);
@@ -549,7 +623,7 @@ bz_status bz_batch_info(const bz_batch *batch, int *capacity, int *terms_per_ite
     if (!batch) return BZ_ERR_ARG;
     const size_t n3 = (size_t)batch->pl->N * batch->pl->N * batch->pl->N;
     if (capacity) *capacity = batch->capacity;
-    if (terms_per_item) *terms_per_item = batch->TB * (batch->pl->real ? 2 : 1);
+    if (terms_per_item) *terms_per_item = batch->TB * (batch->pl->real && !batch->pl->col32 ? 2 : 1);
     if (workspace_bytes)
         *workspace_bytes = (size_t)batch->capacity * n3 * (sizeof(float2) * (1 + batch->nblk) + 2 * sizeof(double2));
     return BZ_OK;
@@ -568,12 +642,16 @@ bz_status bz_batch_collide(bz_batch *batch, int count, const int *slots, const v
     if (!B.pl->real)
         k_batch_load<<<grid_for(B), 256, 0, st>>>(fhat, dtype, B.slots_dev, B.count_dev, n3, B.fin);
     if (B.pl->h_fp64) {                                   // (the real-data form's inputs come from the first pass)
-        s = h64_launch(B.pl->N, fhat, dtype, B.slots_dev, B.count_dev, B.capacity, B.scr64, B.h, st, B.fsym);
+        s = h64_launch(B.pl->N, fhat, dtype, B.slots_dev, B.count_dev, B.capacity, B.scr64, B.h, st, B.fsym,
+                       B.pl->col32 != 0);
         if (s != BZ_OK) return s;
     }
     s = launch_fused(*B.pl, item_args(B), st);
     if (s != BZ_OK) return s;
-    if (B.pl->real)
+    if (B.pl->col32)
+        k_batch_out_col<<<dim3(32, B.capacity), 512, 0, st>>>(B.part, B.nblk, B.slots_dev, B.count_dev, Qhat, dtype,
+                                                             nonfinite_flag(*B.pl));
+    else if (B.pl->real)
         k_batch_out_real<<<grid_for(B), 256, 0, st>>>(B.part, B.part_s, B.nblk, B.slots_dev, B.count_dev, B.pl->N,
                                                      Qhat, dtype, nonfinite_flag(*B.pl));
     else
@@ -603,9 +681,13 @@ bz_status bz_batch_step_rk(bz_batch *batch, int count, const int *slots, void *f
         for (int stage = 1; stage <= 4 && cs == BZ_OK; ++stage) {
             if (B.pl->h_fp64)
                 cs = h64_launch(B.pl->N, B.fin64, BZ_C128, B.slots_dev, B.count_dev, B.capacity, B.scr64, B.h,
-                                B.cap_stream, B.fsym);
+                                B.cap_stream, B.fsym, B.pl->col32 != 0);
             if (cs == BZ_OK) cs = launch_fused(*B.pl, item_args(B), B.cap_stream);
-            if (B.pl->real)
+            if (B.pl->col32)
+                k_batch_rk_stage_col<<<dim3(32, B.capacity), 512, 0, B.cap_stream>>>(B.part, B.nblk, B.slots_dev,
+                                                                                    B.count_dev, B.f0, B.fsum, B.fin,
+                                                                                    B.fin64, stage, dt);
+            else if (B.pl->real)
                 k_batch_rk_stage_real<<<grid_for(B), 256, 0, B.cap_stream>>>(B.part, B.part_s, B.nblk, B.slots_dev,
                                                                             B.count_dev, B.pl->N, B.f0, B.fsum,
                                                                             B.fin, B.fin64, stage, dt);

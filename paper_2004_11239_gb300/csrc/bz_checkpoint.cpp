@@ -52,7 +52,7 @@ void fill(const bz::Plan &pl, Header &h) {
     h.f[F_HPREC] = pl.h_fp64 ? BZ_H_FP64 : BZ_H_FP32;
     // 2D plans have one pipeline and split-BF16 plans one cluster size: left to the plan
     h.f[F_PIPE] = pl.dim == 2 ? BZ_PIPE_AUTO : (pl.use_fused ? BZ_PIPE_FUSED : BZ_PIPE_CHUNKED);
-    h.f[F_CLUSTER] = pl.use_fused && pl.dim == 3 && pl.precision == BZ_PREC_FP32 ? pl.fused_C : 0;
+    h.f[F_CLUSTER] = pl.use_fused && pl.dim == 3 && pl.precision == BZ_PREC_FP32 && !pl.col32 ? pl.fused_C : 0;   // 0: k_col32
     h.f[F_CTAS] = pl.pair3 ? 3 : 0;
     h.f[F_CHUNK] = pl.chunk;
     h.d[D_L] = pl.L;
@@ -130,7 +130,9 @@ bz_status bz_checkpoint_plan_desc(const char *path, bz_plan_desc *desc, double *
     desc->h_precision = h.f[F_HPREC];
     desc->pipeline = h.f[F_PIPE];
     desc->cluster = h.f[F_CLUSTER];
-    desc->ctas_per_sm = h.f[F_CTAS] ? h.f[F_CTAS] : (h.f[F_DATA] == BZ_DATA_REAL && h.f[F_PIPE] == BZ_PIPE_FUSED ? 2 : 0);
+    // real data on the fused pipeline: cluster 0 is k_col32 (the default), else a cluster kernel
+    desc->ctas_per_sm = h.f[F_CTAS] ? h.f[F_CTAS]
+                        : (h.f[F_DATA] == BZ_DATA_REAL && h.f[F_PIPE] == BZ_PIPE_FUSED && h.f[F_CLUSTER] > 0 ? 2 : 0);
     desc->chunk_terms = h.f[F_CHUNK];
     desc->L = h.d[D_L];
     desc->R = h.d[D_R];

@@ -63,7 +63,7 @@ template <int N> __device__ __forceinline__ int bitrev_n(int l) {
 template <int N, int AXIS>
 __global__ void __launch_bounds__(256)
 k_h64_warp(const void *f, int dtype, const int *slots, const int *count_dev, double2 *scr, float2 *h,
-           float2 *fsym) {
+           float2 *fsym, int col) {
     constexpr int N2 = N * N, LPW = 32 / N, LINES = 8 * LPW;     // lines per warp, per CTA
     const int b = blockIdx.y;
     if (count_dev && b >= *count_dev) return;
@@ -111,8 +111,12 @@ k_h64_warp(const void *f, int dtype, const int *slots, const int *count_dev, dou
         else v = cadd(v, p);
     }
     const size_t o = base + (size_t)bitrev_n<N>(l) * stride;
-    if (AXIS == 1) h[o] = make_float2((float)v.x, (float)v.y);
-    else scr[o] = v;
+    if (AXIS == 1) {
+        if (col) ((float *)(h + vol))[((line % N) * N + bitrev_n<N>(l)) * N + line / N] = (float)v.x;   // [j3][j1][j2]
+        else h[o] = make_float2((float)v.x, (float)v.y);
+    } else {
+        scr[o] = v;
+    }
 }
 
 // One line transform of length 32 across the lanes of a warp (radix-2 decimation in frequency,
@@ -137,7 +141,7 @@ __device__ __forceinline__ double2 warp_fft32(double2 v, int l) {
 // j3 = 8r .. 8r + 7, gathering each line from the four CTAs (DSMEM), into scr for the k1 pass.
 // fsym: as k_h64_warp<N, 3>.  Grid (32 planes x 4, instances).
 __global__ void __launch_bounds__(256) k_h64_plane32(const void *f, int dtype, const int *slots, const int *count_dev,
-                                                    double2 *scr, float2 *fsym) {
+                                                    double2 *scr, float2 *fsym, int col) {
     constexpr int N = 32, N2 = N * N;
     __shared__ double2 rows[8][N];                           // [k2 - 8r][j3]
     const int b = blockIdx.y;
@@ -160,7 +164,9 @@ __global__ void __launch_bounds__(256) k_h64_plane32(const void *f, int dtype, c
                 const double2 c = load_c(f, dtype, vol + ((size_t)((N - k1) % N) * N + (N - k2) % N) * N + (N - l) % N);
                 v = make_double2(0.5 * (a.x + c.x), 0.5 * (a.y - c.y));
             }
-            fsym[base + l] = make_float2((float)v.x, (float)v.y);
+            const float2 fs = make_float2((float)v.x, (float)v.y);
+            if (!col) fsym[base + l] = fs;
+            else if (l < h2) fsym[vol + ((size_t)l * N + k1) * N + k2] = fs;   // [k3][k1][k2]
         }
         rows[w][bitrev_n<N>(l)] = warp_fft32(v, l);
     }
@@ -178,7 +184,7 @@ __global__ void __launch_bounds__(256) k_h64_plane32(const void *f, int dtype, c
 
 template <int N>
 static bz_status h64_n(const void *f, int dtype, const int *slots, const int *count_dev, int count, double2 *scr,
-                       float2 *h, float2 *fsym, cudaStream_t st) {
+                       float2 *h, float2 *fsym, bool col, cudaStream_t st) {
     if constexpr ((N & (N - 1)) == 0) {
         constexpr int LINES = 8 * (32 / N);
         const dim3 grid((N * N + LINES - 1) / LINES, count);
@@ -195,12 +201,12 @@ static bz_status h64_n(const void *f, int dtype, const int *slots, const int *co
             cfg.stream = st;
             cfg.attrs = attr;
             cfg.numAttrs = 1;
-            BZ_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_h64_plane32, f, dtype, slots, count_dev, scr, fsym));
+            BZ_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_h64_plane32, f, dtype, slots, count_dev, scr, fsym, (int)col));
         } else {
-            k_h64_warp<N, 3><<<grid, 256, 0, st>>>(f, dtype, slots, count_dev, scr, h, fsym);
-            k_h64_warp<N, 2><<<grid, 256, 0, st>>>(f, dtype, slots, count_dev, scr, h, nullptr);
+            k_h64_warp<N, 3><<<grid, 256, 0, st>>>(f, dtype, slots, count_dev, scr, h, fsym, 0);
+            k_h64_warp<N, 2><<<grid, 256, 0, st>>>(f, dtype, slots, count_dev, scr, h, nullptr, 0);
         }
-        k_h64_warp<N, 1><<<grid, 256, 0, st>>>(f, dtype, slots, count_dev, scr, h, nullptr);
+        k_h64_warp<N, 1><<<grid, 256, 0, st>>>(f, dtype, slots, count_dev, scr, h, nullptr, (int)col);
     } else {
         if (fsym) return BZ_ERR_UNSUPPORTED;
         const dim3 grid((N * N + kH64Lines - 1) / kH64Lines, count);
@@ -213,13 +219,14 @@ static bz_status h64_n(const void *f, int dtype, const int *slots, const int *co
 }
 
 bz_status h64_launch(int N, const void *f, int dtype, const int *slots, const int *count_dev, int count,
-                     double2 *scr, float2 *h, cudaStream_t st, float2 *fsym) {
+                     double2 *scr, float2 *h, cudaStream_t st, float2 *fsym, bool col) {
     if (count <= 0) return BZ_OK;
+    if (col && N != 32) return BZ_ERR_UNSUPPORTED;
     switch (N) {
-        case 8: return h64_n<8>(f, dtype, slots, count_dev, count, scr, h, fsym, st);
-        case 16: return h64_n<16>(f, dtype, slots, count_dev, count, scr, h, fsym, st);
-        case 24: return h64_n<24>(f, dtype, slots, count_dev, count, scr, h, fsym, st);
-        case 32: return h64_n<32>(f, dtype, slots, count_dev, count, scr, h, fsym, st);
+        case 8: return h64_n<8>(f, dtype, slots, count_dev, count, scr, h, fsym, col, st);
+        case 16: return h64_n<16>(f, dtype, slots, count_dev, count, scr, h, fsym, col, st);
+        case 24: return h64_n<24>(f, dtype, slots, count_dev, count, scr, h, fsym, col, st);
+        case 32: return h64_n<32>(f, dtype, slots, count_dev, count, scr, h, fsym, col, st);
     }
     return BZ_ERR_UNSUPPORTED;
 }
@@ -381,6 +388,7 @@ template <int N, int C> static bz_status launch_sc(const Plan &pl, const ItemArg
 bz_status launch_fused(const Plan &pl, const ItemArgs &a, cudaStream_t st) {
     const int N = pl.N, C = pl.fused_C;
     if (pl.precision == BZ_PREC_BF16X3) return a.real ? BZ_ERR_UNSUPPORTED : launch_mixed(pl, a, st);
+    if (pl.col32) return launch_col32(pl, a, st);
     if (pl.pair3 && a.real) return launch_pair3(pl, a, st);
     if (N == 8 && C == 1) return launch_sc<8, 1>(pl, a, st);
     if (N == 16 && C == 1) return launch_sc<16, 1>(pl, a, st);
@@ -422,24 +430,31 @@ bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches
         }
         a.fin = pl.fsym; a.alpha = pl.apair; a.real = 1; a.cpair = pl.cpair; a.part_s = pl.part_s;
         a.p0 = p0 / 2; a.p1 = p1 / 2;
+        if (pl.col32) {
+            a.fin = pl.fcol; a.alpha = pl.acol; a.hg = (const float2 *)pl.hcol;
+            a.p0 = p0; a.p1 = p1;                         // one term at a time
+        }
     }
     const int nt = a.p1 - a.p0;
     a.TB = nt > 0 ? (nt + pl.fused_G - 1) / pl.fused_G : 1;
     a.nblk = nt > 0 ? (nt + a.TB - 1) / a.TB : 0;
     if (pl.h_fp64 || pl.precision == BZ_PREC_BF16X3) {
         tm_begin(pl, st);
-        s = h64_launch(pl.N, src, src_dtype, nullptr, nullptr, 1, pl.scr64, pl.h, st, pl.real ? pl.fsym : nullptr);
+        s = h64_launch(pl.N, src, src_dtype, nullptr, nullptr, 1, pl.scr64,
+                       pl.col32 ? (float2 *)pl.hcol : pl.h, st, pl.col32 ? pl.fcol : (pl.real ? pl.fsym : nullptr),
+                       pl.col32 != 0);
         if (s != BZ_OK) return s;
         tm_end(pl, st, TK_OTHER);
         nl += h64_launches(pl.N);
-    } else if (pl.pair3) {
-        // the pair kernel reads h: formed in FP32 from the symmetrised input by one plane pass
+    } else if (pl.pair3 || pl.col32) {
+        // these kernels read h: formed in FP32 from the symmetrised input by one plane pass
         // and one pencil pass of the chunked pipeline
         tm_begin(pl, st);
         s = h_fp32(pl, pl.fsym, st);
+        if (s == BZ_OK && pl.col32) s = col32_inputs(pl, st);
         if (s != BZ_OK) return s;
         tm_end(pl, st, TK_OTHER);
-        nl += 2;
+        nl += pl.col32 ? 3 : 2;
     } else {
         a.hg = nullptr;                                   // h formed in FP32 in the item prologue
     }
@@ -449,7 +464,7 @@ bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches
     tm_end(pl, st, TK_FUSED);
     tm_begin(pl, st);
     if (pl.real) {
-        s = reduce_sym(pl, a.nblk, st);                   // sums of the blocks, symmetrised
+        s = pl.col32 ? reduce_col(pl, a.nblk, st) : reduce_sym(pl, a.nblk, st);   // sums of the blocks, symmetrised
         if (s != BZ_OK) return s;
     } else {
         k_reduce_parts<<<(n3 + 31) / 32, 256, 0, st>>>(pl.part, a.nblk, n3, pl.acc);

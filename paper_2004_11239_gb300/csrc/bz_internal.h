@@ -81,7 +81,11 @@ struct Plan {
     uint4 *wimg = nullptr;          // BZ_PREC_BF16X3: split DFT matrix (tensor-core B operand)
     // BZ_DATA_REAL: terms 2q and 2q + 1 share one pair of transforms
     int real = 0;
-    int pair3 = 0;                  // N = 32: the three-CTA-per-SM pair kernel (k_pair3) instead of k_fused
+    int col32 = 0;                  // N = 32: one term per SM (k_col32): the default of the fused pipeline
+    float2 *acol = nullptr;         // its table [P][18][32][32] (bz_col32.cu)
+    float2 *fcol = nullptr;         // its input [k3 < 16][k1][k2] (N^3 allocated)
+    float *hcol = nullptr;          // its h [j3][j1][j2], packed floats
+    int pair3 = 0;                  // N = 32, on request: the three-CTA-per-SM pair kernel (k_pair3) instead of k_fused
     float2 *apair = nullptr;        // [P / 2][N^3] A = (alpha_2q - i alpha_2q+1) / 2
     float2 *cpair = nullptr;        // [P / 2][3][N][N] C = conj B(-k), B = (alpha_2q + i alpha_2q+1) / 2, on the
                                     // Nyquist planes (families k1 = -N/2, k2 = -N/2, k3 = -N/2), 0 elsewhere
@@ -177,9 +181,10 @@ bz_status launch_fused(const Plan &pl, const ItemArgs &a, cudaStream_t st);
 // Kernel launches of one h64_launch: three line passes (N = 32: the k3 and k2 passes as one).
 inline int h64_launches(int N) { return N == 32 ? 2 : 3; }
 // fsym (BZ_DATA_REAL, N a power of two): transform the Hermitian, Nyquist-free part of f and
-// store that part in FP32 to fsym.
+// store that part in FP32 to fsym; col (N = 32): in k_col32's layouts ([k3 < 16][k1][k2], and h as
+// packed floats [j3][j1][j2]; the same stride of N^3 float2 per slot).
 bz_status h64_launch(int N, const void *f, int dtype, const int *slots, const int *count_dev, int count,
-                     double2 *scr, float2 *h, cudaStream_t st, float2 *fsym = nullptr);
+                     double2 *scr, float2 *h, cudaStream_t st, float2 *fsym = nullptr, bool col = false);
 bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches);
 // bz_real.cu (BZ_DATA_REAL): the pair table from alpha (after ftable_build); pl.fsym and
 // pl.fsym64 from a c64 / c128 array
@@ -193,6 +198,15 @@ bz_status sym_output(Plan &pl, cudaStream_t st);
 // bz_pair3.cu (BZ_DATA_REAL, N = 32, FP64 h): resident clusters and launch of k_pair3
 cudaError_t pair3_setup(int *G);
 bz_status launch_pair3(const Plan &pl, const ItemArgs &a, cudaStream_t st);
+
+// bz_col32.cu (BZ_DATA_REAL, N = 32): one CTA per SM; items count terms.  The table from pl.alpha;
+// inputs from pl.fsym and pl.h (FP32 h); pl.acc <- the sum of nblk items
+constexpr size_t kCol32Part = (size_t)18 * 32 * 32;     // float2 per item's sums
+cudaError_t col32_setup(int *G);
+bz_status launch_col32(const Plan &pl, const ItemArgs &a, cudaStream_t st);
+bz_status col32_table(Plan &pl);
+bz_status col32_inputs(Plan &pl, cudaStream_t st);
+bz_status reduce_col(Plan &pl, int nblk, cudaStream_t st);
 
 // bz_mixed.cu (BZ_PREC_BF16X3, N = 32)
 cudaError_t mixed_setup(int N, int *G);

@@ -16,6 +16,7 @@
 #include "bz_cluster.cuh"
 #include "bz_fft.cuh"
 #include "bz_internal.h"
+#include "bz_tmem.cuh"
 
 namespace bz {
 
@@ -32,31 +33,6 @@ constexpr uint32_t P_TMEM_COLS = 128;          // acc (64 columns) + fhat column
 constexpr uint32_t TM_ACC = 0, TM_FH = 64;
 static_assert(3 * (P_SMEM + 1024) <= 228 * 1024, "three CTAs per SM");
 static_assert(4 * (P_SMEM + 1024) > 228 * 1024 || 4 * P_TMEM_COLS <= 512, "tensor memory never oversubscribed");
-
-__device__ __forceinline__ void tfence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
-__device__ __forceinline__ void tfence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
-__device__ __forceinline__ void t_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory"); }
-__device__ __forceinline__ void t_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
-
-// 16 consecutive 32-bit columns of the thread's own lane.
-__device__ __forceinline__ void t_ld16(uint32_t ta, float *v) {
-    uint32_t r[16];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-                 : "r"(ta) : "memory");
-    #pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-__device__ __forceinline__ void t_st16(uint32_t ta, const float *v) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};\n"
-                 ::"r"(ta), "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
-                   "r"(__float_as_uint(v[3])), "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])),
-                   "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7])), "r"(__float_as_uint(v[8])),
-                   "r"(__float_as_uint(v[9])), "r"(__float_as_uint(v[10])), "r"(__float_as_uint(v[11])),
-                   "r"(__float_as_uint(v[12])), "r"(__float_as_uint(v[13])), "r"(__float_as_uint(v[14])),
-                   "r"(__float_as_uint(v[15])) : "memory");
-}
 
 template <bool SCALED>
 __global__ void __launch_bounds__(PT, 3) k_pair3(ItemArgs a) {
