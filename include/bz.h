@@ -99,9 +99,11 @@ enum { BZ_PIPE_AUTO = 0, BZ_PIPE_FUSED = 1, BZ_PIPE_CHUNKED = 2 };
 
 /* Precision of h = IFFT(fhat) on the fused pipeline.  FP32 transforms leave a noise floor of
  * about eps max|h| over the grid, which the product h g_p turns into error where g_p is large
- * and h small; forming h in FP64 (from the caller's FP64 coefficients) removes that half of
- * the rounding error, at the cost of three short FP64 passes per collide.  FP32 forms h
- * inside the fused kernel.  AUTO = FP64. */
+ * and h small; forming h in extended precision (from the caller's FP64 coefficients) removes that
+ * half of the rounding error, at the cost of one or two short launches per collide.  BZ_H_FP64
+ * computes in double-float arithmetic (pairs of FP32, about 47 bits): the stored FP32 h has the
+ * error of its rounding, as with FP64 arithmetic.  FP32 forms h inside the fused kernel.
+ * AUTO = FP64. */
 enum { BZ_H_AUTO = 0, BZ_H_FP64 = 1, BZ_H_FP32 = 2 };
 
 /* Data of the operator (Sec. 2: f is a real distribution function, so fhat is Hermitian).
@@ -265,7 +267,7 @@ const char *bz_status_str(bz_status s);
  * nothing is allocated or freed.  The plan must have been created beforehand on the
  * current device.
  *   - Size limit: the array holds the FP32 input copy and h (8 N^3 bytes each), the FP64
- *     accumulator (16 N^3), the FP64 h pass's scratch where h is formed in FP64 (16 N^3) and at
+ *     accumulator (16 N^3), the h pass's scratch where the plan asks for BZ_H_FP64 (16 N^3) and at
  *     least one term of 8 N^3 (each rounded up to 256-byte blocks).  N <= 48 fits (N = 48: five
  *     terms per chunk); N = 64 does not and returns BZ_ERR_ARG without touching Qhat.
  *   - Each call looks up the array's device address (cudaGetSymbolAddress) with the current

@@ -642,7 +642,7 @@ bz_status bz_batch_collide(bz_batch *batch, int count, const int *slots, const v
     if (!B.pl->real)
         k_batch_load<<<grid_for(B), 256, 0, st>>>(fhat, dtype, B.slots_dev, B.count_dev, n3, B.fin);
     if (B.pl->h_fp64) {                                   // (the real-data form's inputs come from the first pass)
-        s = h64_launch(B.pl->N, fhat, dtype, B.slots_dev, B.count_dev, B.capacity, B.scr64, B.h, st, B.fsym,
+        s = hff_launch(B.pl->N, fhat, dtype, B.slots_dev, B.count_dev, B.capacity, B.scr64, B.h, st, B.fsym,
                        B.pl->col32 != 0);
         if (s != BZ_OK) return s;
     }
@@ -658,7 +658,7 @@ bz_status bz_batch_collide(bz_batch *batch, int count, const int *slots, const v
         k_batch_out<<<grid_for(B), 256, 0, st>>>(B.part, B.nblk, B.slots_dev, B.count_dev, n3, Qhat, dtype,
                                                 nonfinite_flag(*B.pl));
     BZ_CUDA_TRY(cudaGetLastError());
-    B.last_launches = (B.pl->real ? 2 : 3) + (B.pl->h_fp64 ? h64_launches(B.pl->N) : 0);
+    B.last_launches = (B.pl->real ? 2 : 3) + (B.pl->h_fp64 ? hff_launches(B.pl->N) : 0);
     return BZ_OK;
 }
 
@@ -680,7 +680,7 @@ bz_status bz_batch_step_rk(bz_batch *batch, int count, const int *slots, void *f
         bz_status cs = BZ_OK;
         for (int stage = 1; stage <= 4 && cs == BZ_OK; ++stage) {
             if (B.pl->h_fp64)
-                cs = h64_launch(B.pl->N, B.fin64, BZ_C128, B.slots_dev, B.count_dev, B.capacity, B.scr64, B.h,
+                cs = hff_launch(B.pl->N, B.fin64, BZ_C128, B.slots_dev, B.count_dev, B.capacity, B.scr64, B.h,
                                 B.cap_stream, B.fsym, B.pl->col32 != 0);
             if (cs == BZ_OK) cs = launch_fused(*B.pl, item_args(B), B.cap_stream);
             if (B.pl->col32)
@@ -711,7 +711,7 @@ bz_status bz_batch_step_rk(bz_batch *batch, int count, const int *slots, void *f
     for (int step = 0; step < nsteps; ++step) BZ_CUDA_TRY(cudaGraphLaunch(it->second, st));
     k_batch_rk_out<<<grid_for(B), 256, 0, st>>>(B.f0, B.slots_dev, B.count_dev, n3, fhat, dtype, nonfinite_flag(*B.pl));
     BZ_CUDA_TRY(cudaGetLastError());
-    B.last_launches = 2 + 4 * (2 + (B.pl->h_fp64 ? h64_launches(B.pl->N) : 0)) * nsteps;
+    B.last_launches = 2 + 4 * (2 + (B.pl->h_fp64 ? hff_launches(B.pl->N) : 0)) * nsteps;
     return BZ_OK;
 }
 

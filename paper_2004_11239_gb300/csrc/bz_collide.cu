@@ -564,7 +564,7 @@ bz_status load_input(Plan &pl, const void *fhat, int dtype, cudaStream_t st, int
     const int n3 = (int)modes(pl);
     if (dtype != BZ_C64 && dtype != BZ_C128) return BZ_ERR_ARG;
     if (pl.Nin) {
-        // padded: embed into the 2N grid, in FP32 and (where the FP64 h pass reads it) FP64
+        // padded: embed into the 2N grid, in FP32 and (where the h pass reads it) FP64
         k_embed<<<(n3 + 255) / 256, 256, 0, st>>>(fhat, dtype, pl.Nin, pl.N, pl.fin, pl.fin64);
         BZ_CUDA_TRY(cudaGetLastError());
         pl.src = pl.fin64;
@@ -681,7 +681,7 @@ bz_status run_noalloc(const Plan &pl, const void *fhat, void *Qhat, int dtype, u
     }
     if (h64) {
         // as bz_collide on this plan: h from the caller's coefficients in FP64, stored FP32
-        const bz_status s = h64_launch(N, fhat, dtype, nullptr, nullptr, 1, scr64, h, st);
+        const bz_status s = hff_launch(N, fhat, dtype, nullptr, nullptr, 1, scr64, h, st);
         if (s != BZ_OK) return s;
     } else {
         k_plane_inv<N><<<dim3(N / PPC, 1), Cfg<N>::THREADS, Cfg<N>::SMEM, st>>>(fin, pl.tw, S, 0, 0);

@@ -1,235 +1,9 @@
-// The fused per-term pipeline (N <= 32): launch configuration, cluster-size setup, the FP64
-// h passes and the fixed-order reduction of the items' partial sums.  The kernel itself is in
+// The fused per-term pipeline (N <= 32): launch configuration, cluster-size setup and the
+// fixed-order reduction of the items' partial sums.  The kernel itself is in
 // bz_fused_kernel.cuh.
 #include "bz_fused_kernel.cuh"
 
 namespace bz {
-
-// h = IFFT(fhat) in FP64 (stored FP32) for the fused path.  FP32 transforms leave a noise
-// floor of about eps max|h| over the whole grid, and the product h g_p turns that floor into
-// errors where g_p is large and h is small; forming h in FP64 removes that half of the
-// rounding error (the per-term g_p stay FP32).  FP64 throughput per SM is low on this GPU,
-// so the transform runs as three line passes (axis 3, 2, 1) with eight lines per CTA: the
-// N^2 lines of a pass spread over (nearly) every SM.
-constexpr int kH64Lines = 8;
-
-__device__ __forceinline__ double2 load_c(const void *f, int dtype, size_t i) {
-    if (dtype == BZ_C128) return ((const double2 *)f)[i];
-    float2 v = ((const float2 *)f)[i];
-    return make_double2(v.x, v.y);
-}
-
-// AXIS 3: line (k1, k2) contiguous, from f into scr; AXIS 2: line (k1, k3) with stride N in
-// scr; AXIS 1: line (j2, j3) with stride N^2, from scr into h (FP32).
-template <int N, int AXIS>
-__global__ void __launch_bounds__(kH64Lines)
-k_h64_pass(const void *f, int dtype, const int *slots, const int *count_dev, double2 *scr, float2 *h) {
-    constexpr int N2 = N * N;
-    const int b = blockIdx.y;
-    if (count_dev && b >= *count_dev) return;
-    const int slot = slots ? slots[b] : b;
-    const int line = blockIdx.x * kH64Lines + threadIdx.x;
-    if (line >= N2) return;
-    const size_t vol = (size_t)slot * N * N2;
-    size_t base, stride;
-    if (AXIS == 3) { base = vol + (size_t)line * N; stride = 1; }
-    else if (AXIS == 2) { base = vol + (size_t)(line / N) * N2 + (line % N); stride = N; }
-    else { base = vol + line; stride = N2; }
-    double2 x[N];
-    #pragma unroll
-    for (int k = 0; k < N; ++k)
-        x[k] = AXIS == 3 ? load_c(f, dtype, base + k * stride) : scr[base + k * stride];
-    fft_inplace<N, +1>(x);
-    if (AXIS == 1) {
-        #pragma unroll
-        for (int j = 0; j < N; ++j) h[base + j * stride] = make_float2((float)x[j].x, (float)x[j].y);
-    } else {
-        #pragma unroll
-        for (int j = 0; j < N; ++j) scr[base + j * stride] = x[j];
-    }
-}
-
-// Power-of-two N: one warp (N <= 16: a lane segment) per line, radix-2 decimation in
-// frequency across lanes with shuffles, lane l ends with frequency bitrev(l).  Each lane's
-// twiddles for the log2 N stages are read once.  32 lanes per line keep many more FP64
-// operations in flight than one thread per line.
-template <int N> __device__ __forceinline__ int bitrev_n(int l) {
-    int r = 0;
-    #pragma unroll
-    for (int b = 1; b < N; b <<= 1) r = (r << 1) | ((l & b) ? 1 : 0);
-    return r;
-}
-
-template <int N, int AXIS>
-__global__ void __launch_bounds__(256)
-k_h64_warp(const void *f, int dtype, const int *slots, const int *count_dev, double2 *scr, float2 *h,
-           float2 *fsym, int col) {
-    constexpr int N2 = N * N, LPW = 32 / N, LINES = 8 * LPW;     // lines per warp, per CTA
-    const int b = blockIdx.y;
-    if (count_dev && b >= *count_dev) return;
-    const int slot = slots ? slots[b] : b;
-    const int lane = threadIdx.x & 31, l = lane % N;
-    const int line = blockIdx.x * LINES + (threadIdx.x >> 5) * LPW + lane / N;
-    if (line >= N2) return;                                   // whole segments exit together
-    // twiddle of this lane at each stage (half-size hs): exp(+2 pi i (l mod hs) / (2 hs))
-    double2 tw[16];
-    int st = 0;
-    #pragma unroll
-    for (int hs = N / 2; hs >= 1; hs >>= 1, ++st) {
-        const int j = (l % hs) * (N / (2 * hs));              // index into the length-N roots
-        tw[st] = c_twd.v[tw_off<N>() + j];
-    }
-    const size_t vol = (size_t)slot * N * N2;
-    size_t base, stride;
-    if (AXIS == 3) { base = vol + (size_t)line * N; stride = 1; }
-    else if (AXIS == 2) { base = vol + (size_t)(line / N) * N2 + (line % N); stride = N; }
-    else { base = vol + line; stride = N2; }
-    double2 v;
-    if (AXIS != 3) {
-        v = scr[base + (size_t)l * stride];
-    } else if (!fsym) {
-        v = load_c(f, dtype, base + (size_t)l * stride);
-    } else {
-        // BZ_DATA_REAL: the Hermitian part (fhat_k + conj fhat_{-k}) / 2, zero where an index is
-        // N/2; its FP32 copy is the fused kernel's input
-        const int k1 = line / N, k2 = line % N, h2 = N / 2;
-        v = make_double2(0.0, 0.0);
-        if (k1 != h2 && k2 != h2 && l != h2) {
-            const double2 a = load_c(f, dtype, base + l);
-            const double2 c = load_c(f, dtype, vol + ((size_t)((N - k1) % N) * N + (N - k2) % N) * N + (N - l) % N);
-            v = make_double2(0.5 * (a.x + c.x), 0.5 * (a.y - c.y));
-        }
-        fsym[base + l] = make_float2((float)v.x, (float)v.y);
-    }
-    st = 0;
-    #pragma unroll
-    for (int hs = N / 2; hs >= 1; hs >>= 1, ++st) {
-        double2 p;
-        p.x = __shfl_xor_sync(0xffffffffu, v.x, hs);
-        p.y = __shfl_xor_sync(0xffffffffu, v.y, hs);
-        if (l & hs) v = cmul(csub(p, v), tw[st]);
-        else v = cadd(v, p);
-    }
-    const size_t o = base + (size_t)bitrev_n<N>(l) * stride;
-    if (AXIS == 1) {
-        if (col) ((float *)(h + vol))[((line % N) * N + bitrev_n<N>(l)) * N + line / N] = (float)v.x;   // [j3][j1][j2]
-        else h[o] = make_float2((float)v.x, (float)v.y);
-    } else {
-        scr[o] = v;
-    }
-}
-
-// One line transform of length 32 across the lanes of a warp (radix-2 decimation in frequency,
-// as k_h64_warp): lane l holds x_l on entry and X_bitrev(l) on return.
-__device__ __forceinline__ double2 warp_fft32(double2 v, int l) {
-    int st = 0;
-    #pragma unroll
-    for (int hs = 16; hs >= 1; hs >>= 1, ++st) {
-        const double2 tw = c_twd.v[tw_off<32>() + (l % hs) * (32 / (2 * hs))];
-        double2 p;
-        p.x = __shfl_xor_sync(0xffffffffu, v.x, hs);
-        p.y = __shfl_xor_sync(0xffffffffu, v.y, hs);
-        if (l & hs) v = cmul(csub(p, v), tw);
-        else v = cadd(v, p);
-    }
-    return v;
-}
-
-// N = 32: the first two FP64 passes (axes k3 and k2, both inside a plane k1) in one kernel.  A
-// cluster of 4 CTAs holds one plane: CTA r transforms the k3 lines of rows k2 = 8r .. 8r + 7 (one
-// warp per line) into its shared memory, and after a cluster barrier the k2 lines of columns
-// j3 = 8r .. 8r + 7, gathering each line from the four CTAs (DSMEM), into scr for the k1 pass.
-// fsym: as k_h64_warp<N, 3>.  Grid (32 planes x 4, instances).
-__global__ void __launch_bounds__(256) k_h64_plane32(const void *f, int dtype, const int *slots, const int *count_dev,
-                                                    double2 *scr, float2 *fsym, int col) {
-    constexpr int N = 32, N2 = N * N;
-    __shared__ double2 rows[8][N];                           // [k2 - 8r][j3]
-    const int b = blockIdx.y;
-    if (count_dev && b >= *count_dev) return;               // uniform over the cluster
-    const int slot = slots ? slots[b] : b;
-    const int r = (int)cooperative_groups::this_cluster().block_rank();
-    const int k1 = blockIdx.x / 4, w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    const size_t vol = (size_t)slot * N * N2;
-    {                                                        // k3 line of row k2 = 8r + w
-        const int k2 = 8 * r + w;
-        const size_t base = vol + ((size_t)k1 * N + k2) * N;
-        double2 v;
-        if (!fsym) {
-            v = load_c(f, dtype, base + l);
-        } else {
-            const int h2 = N / 2;
-            v = make_double2(0.0, 0.0);
-            if (k1 != h2 && k2 != h2 && l != h2) {
-                const double2 a = load_c(f, dtype, base + l);
-                const double2 c = load_c(f, dtype, vol + ((size_t)((N - k1) % N) * N + (N - k2) % N) * N + (N - l) % N);
-                v = make_double2(0.5 * (a.x + c.x), 0.5 * (a.y - c.y));
-            }
-            const float2 fs = make_float2((float)v.x, (float)v.y);
-            if (!col) fsym[base + l] = fs;
-            else if (l < h2) fsym[vol + ((size_t)l * N + k1) * N + k2] = fs;   // [k3][k1][k2]
-        }
-        rows[w][bitrev_n<N>(l)] = warp_fft32(v, l);
-    }
-    cooperative_groups::this_cluster().sync();
-    {                                                        // k2 line of column j3 = 8r + w
-        const int j3 = 8 * r + w;
-        const uint32_t src = dsmem_addr(&rows[l % 8][j3], (uint32_t)(l / 8));   // element (k2 = l, j3)
-        double2 v;
-        asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];\n" : "=d"(v.x), "=d"(v.y) : "r"(src) : "memory");
-        v = warp_fft32(v, l);
-        scr[vol + ((size_t)k1 * N + bitrev_n<N>(l)) * N + j3] = v;
-    }
-    cooperative_groups::this_cluster().sync();               // no CTA leaves while its rows are read
-}
-
-template <int N>
-static bz_status h64_n(const void *f, int dtype, const int *slots, const int *count_dev, int count, double2 *scr,
-                       float2 *h, float2 *fsym, bool col, cudaStream_t st) {
-    if constexpr ((N & (N - 1)) == 0) {
-        constexpr int LINES = 8 * (32 / N);
-        const dim3 grid((N * N + LINES - 1) / LINES, count);
-        if constexpr (N == 32) {
-            // axes k3 and k2 in one clustered pass, then the k1 pass
-            cudaLaunchConfig_t cfg = {};
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = 4;
-            attr[0].val.clusterDim.y = 1;
-            attr[0].val.clusterDim.z = 1;
-            cfg.gridDim = dim3(4 * N, count);
-            cfg.blockDim = dim3(256);
-            cfg.stream = st;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
-            BZ_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_h64_plane32, f, dtype, slots, count_dev, scr, fsym, (int)col));
-        } else {
-            k_h64_warp<N, 3><<<grid, 256, 0, st>>>(f, dtype, slots, count_dev, scr, h, fsym, 0);
-            k_h64_warp<N, 2><<<grid, 256, 0, st>>>(f, dtype, slots, count_dev, scr, h, nullptr, 0);
-        }
-        k_h64_warp<N, 1><<<grid, 256, 0, st>>>(f, dtype, slots, count_dev, scr, h, nullptr, (int)col);
-    } else {
-        if (fsym) return BZ_ERR_UNSUPPORTED;
-        const dim3 grid((N * N + kH64Lines - 1) / kH64Lines, count);
-        k_h64_pass<N, 3><<<grid, kH64Lines, 0, st>>>(f, dtype, slots, count_dev, scr, h);
-        k_h64_pass<N, 2><<<grid, kH64Lines, 0, st>>>(f, dtype, slots, count_dev, scr, h);
-        k_h64_pass<N, 1><<<grid, kH64Lines, 0, st>>>(f, dtype, slots, count_dev, scr, h);
-    }
-    BZ_CUDA_TRY(cudaGetLastError());
-    return BZ_OK;
-}
-
-bz_status h64_launch(int N, const void *f, int dtype, const int *slots, const int *count_dev, int count,
-                     double2 *scr, float2 *h, cudaStream_t st, float2 *fsym, bool col) {
-    if (count <= 0) return BZ_OK;
-    if (col && N != 32) return BZ_ERR_UNSUPPORTED;
-    switch (N) {
-        case 8: return h64_n<8>(f, dtype, slots, count_dev, count, scr, h, fsym, col, st);
-        case 16: return h64_n<16>(f, dtype, slots, count_dev, count, scr, h, fsym, col, st);
-        case 24: return h64_n<24>(f, dtype, slots, count_dev, count, scr, h, fsym, col, st);
-        case 32: return h64_n<32>(f, dtype, slots, count_dev, count, scr, h, fsym, col, st);
-    }
-    return BZ_ERR_UNSUPPORTED;
-}
 
 // acc[k] = sum over g of part[g][k] with a fixed shape: thread (kk, s) of a 32 x 8 block sums
 // g = s, s + 8, ... for mode k = 32 blockIdx.x + kk with Kahan compensation in FP32, then the
@@ -421,7 +195,7 @@ bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches
     if (pl.real) {
         if ((p0 | p1) & 1) return BZ_ERR_ARG;
         if (!(pl.h_fp64 || pl.precision == BZ_PREC_BF16X3)) {
-            // h formed in FP32 in the kernel from the symmetrised copy (the FP64 pass writes it otherwise)
+            // h formed in FP32 in the kernel from the symmetrised copy (the h pass writes it otherwise)
             tm_begin(pl, st);
             s = sym_input(pl, src, src_dtype, st);
             if (s != BZ_OK) return s;
@@ -440,12 +214,12 @@ bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches
     a.nblk = nt > 0 ? (nt + a.TB - 1) / a.TB : 0;
     if (pl.h_fp64 || pl.precision == BZ_PREC_BF16X3) {
         tm_begin(pl, st);
-        s = h64_launch(pl.N, src, src_dtype, nullptr, nullptr, 1, pl.scr64,
+        s = hff_launch(pl.N, src, src_dtype, nullptr, nullptr, 1, pl.scr64,
                        pl.col32 ? (float2 *)pl.hcol : pl.h, st, pl.col32 ? pl.fcol : (pl.real ? pl.fsym : nullptr),
                        pl.col32 != 0);
         if (s != BZ_OK) return s;
         tm_end(pl, st, TK_OTHER);
-        nl += h64_launches(pl.N);
+        nl += hff_launches(pl.N);
     } else if (pl.pair3 || pl.col32) {
         // these kernels read h: formed in FP32 from the symmetrised input by one plane pass
         // and one pencil pass of the chunked pipeline

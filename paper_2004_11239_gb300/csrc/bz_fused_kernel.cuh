@@ -12,7 +12,7 @@
 //   -- cluster barrier --
 //   C  planes (own k1):   FFT over j3 (rows), FFT over j2 (registers), times alpha_p (tile
 //                         prefetched by cp.async during A and B), accumulate in registers
-// h = IFFT(fhat) is formed beforehand in FP64 (k_h64_*) and each item's prologue loads the
+// h = IFFT(fhat) is formed beforehand (bz_hff.cu) and each item's prologue loads the
 // slice of h for the CTA's pencils into shared memory.  DSMEM is reached
 // with ld/st.shared::cluster on mapa addresses.  Each CTA ends with its plane slab of the
 // cluster's partial sum (FP32 over the cluster's terms); a second kernel adds the G

@@ -1,0 +1,380 @@
+// h = IFFT(fhat) in double-float arithmetic, stored FP32: the shared inverse transform of the fused
+// pipelines (N = 8, 16, 24, 32) and of the 2D operator (N = 8, 16, 32, 64).
+//
+// FP32 transforms leave a noise floor of about eps max|h| over the whole grid, and the product
+// h g_p turns that floor into errors where g_p is large and h is small; forming h with more bits
+// removes that half of the rounding error (the per-term g_p stay FP32).  A number here is an
+// unevaluated sum hi + lo of two floats (Dekker 1971; Knuth's TwoSum, FMA-based TwoProduct), about
+// 47 significant bits on the FP32 pipes.  This part runs an FP64 instruction of a warp in 68
+// clocks of its scheduler: an FP64 addition costs what 64 FP32 operations do, a double-float one 11.
+// The stored h has the error of its rounding to FP32 either way (relative 2-norm 2.0e-8 .. 3.8e-8 at
+// N = 8 .. 64, equal to the rounded FP64 transform's in every digit printed).
+// Bound by latency for one instance, by FP32 issue in a batch.  Measured, all launches of one h, against
+// the FP64 kernels before: N = 16 4.5 us (12.0), N = 24 6.3 us (39), N = 32 real 9 - 10 us (14.4); 251
+// instances of N = 16 27 us (202), 16 of N = 32 real 22 us (138).
+//
+// A line of N = 8 R points takes 8 lanes with R points each (x[l + 8 m] in lane l): an R-point
+// transform over m in registers, the twiddle W_N^(l r), and an 8-point transform over the lanes
+// (radix 2 by shuffles, bit-reversed lanes), which leaves X[r + R q] in the lane of q = bitrev(l).
+//   N = 24, 32: one CTA per plane k1 (axes 3 and 2 through shared memory), then lines along axis 1;
+//   N = 8, 16:  a cluster of 8 CTAs per instance, R planes each; axis 1 gathers from the cluster;
+//   2D:         a cluster of 8 CTAs, R rows each; axis 1 gathers from the cluster.
+#include <cooperative_groups.h>
+
+#include "bz_cluster.cuh"
+#include "bz_fft.cuh"
+#include "bz_internal.h"
+
+namespace bz {
+
+namespace {
+
+struct ff { float h, l; };
+struct ffc { ff x, y; };
+
+struct alignas(16) RootFF { float xh, xl, yh, yl; };
+struct RootTable { RootFF v[192]; };
+constexpr RootTable make_roots() {
+    RootTable t{};
+    for (int j = 0; j < 192; ++j) {
+        const TwCS c = unit_root(j, 192);
+        t.v[j].xh = (float)c.c;
+        t.v[j].xl = (float)(c.c - (double)(float)c.c);
+        t.v[j].yh = (float)c.s;
+        t.v[j].yl = (float)(c.s - (double)(float)c.s);
+    }
+    return t;
+}
+static __device__ const RootTable g_roots = make_roots();
+
+// exp(+2 pi i j / N)
+template <int N> __device__ __forceinline__ ffc root(int j) {
+    const float4 v = __ldg((const float4 *)g_roots.v + (j % N) * (192 / N));
+    return {{v.x, v.y}, {v.z, v.w}};
+}
+
+// The _rn intrinsics keep the compiler from contracting or reordering the error-free steps.
+__device__ __forceinline__ ff fadd(ff a, ff b) {
+    const float s = __fadd_rn(a.h, b.h), t = __fsub_rn(s, a.h);
+    float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(b.h, t));
+    e = __fadd_rn(e, __fadd_rn(a.l, b.l));
+    const float h = __fadd_rn(s, e);
+    return {h, __fsub_rn(e, __fsub_rn(h, s))};
+}
+__device__ __forceinline__ ff fneg(ff a) { return {-a.h, -a.l}; }
+// a b + sign c d, sign = +-1
+template <int SIGN> __device__ __forceinline__ ff fdot(ff a, ff b, ff c, ff d) {
+    const float p = __fmul_rn(a.h, b.h), q0 = __fmul_rn(c.h, d.h), q = SIGN > 0 ? q0 : -q0;
+    float pe = __fmaf_rn(a.h, b.h, -p), qe = __fmaf_rn(c.h, d.h, -q0);
+    pe = __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, pe));
+    qe = __fmaf_rn(c.h, d.l, __fmaf_rn(c.l, d.h, qe));
+    const float s = __fadd_rn(p, q), t = __fsub_rn(s, p);
+    float e = __fadd_rn(__fsub_rn(p, __fsub_rn(s, t)), __fsub_rn(q, t));
+    e = __fadd_rn(e, SIGN > 0 ? __fadd_rn(pe, qe) : __fsub_rn(pe, qe));
+    const float h = __fadd_rn(s, e);
+    return {h, __fsub_rn(e, __fsub_rn(h, s))};
+}
+__device__ __forceinline__ ffc add(ffc a, ffc b) { return {fadd(a.x, b.x), fadd(a.y, b.y)}; }
+__device__ __forceinline__ ffc neg(ffc a) { return {fneg(a.x), fneg(a.y)}; }
+__device__ __forceinline__ ffc sub(ffc a, ffc b) { return add(a, neg(b)); }
+__device__ __forceinline__ ffc mul(ffc a, ffc w) { return {fdot<-1>(a.x, w.x, a.y, w.y), fdot<1>(a.x, w.y, a.y, w.x)}; }
+__device__ __forceinline__ ffc times_i(ffc a) { return {fneg(a.y), a.x}; }
+__device__ __forceinline__ ffc half(ffc a) { return {{0.5f * a.x.h, 0.5f * a.x.l}, {0.5f * a.y.h, 0.5f * a.y.l}}; }
+__device__ __forceinline__ float4 pack(ffc a) { return make_float4(a.x.h, a.x.l, a.y.h, a.y.l); }
+__device__ __forceinline__ ffc unpack(float4 v) { return {{v.x, v.y}, {v.z, v.w}}; }
+__device__ __forceinline__ float2 round2(ffc a) { return make_float2(a.x.h, a.y.h); }   // |lo| <= ulp(hi) / 2
+
+// A double as hi + lo by its bits (no FP64 instruction): hi the leading 24 bits of the mantissa, lo the
+// other 29.  Below the FP32 range 0, above it and for Inf / NaN the FP32 infinity or NaN.
+__device__ __forceinline__ ff split(double d) {
+    const unsigned hw = (unsigned)__double2hiint(d), lw = (unsigned)__double2loint(d);
+    const unsigned e = (hw >> 20) & 0x7ffu, sign = hw & 0x80000000u;
+    if (e <= 1023u - 127u) return {__uint_as_float(sign), 0.f};
+    if (e >= 1023u + 128u)
+        return {__uint_as_float(sign | 0x7f800000u | (e == 0x7ffu && ((hw & 0xfffffu) | lw) ? 0x400000u : 0u)), 0.f};
+    const unsigned ef = (e - 896u) << 23;
+    const float h = __uint_as_float(sign | ef | ((hw & 0xfffffu) << 3) | (lw >> 29));
+    const float l = __fmul_rn((float)(lw & 0x1fffffffu) * 0x1p-52f, __uint_as_float(sign | ef));
+    const float s = __fadd_rn(h, l);                      // |lo| <= ulp(hi) / 2
+    return {s, __fsub_rn(l, __fsub_rn(s, h))};
+}
+__device__ __forceinline__ ffc load_ff(const void *f, int dtype, size_t i) {
+    if (dtype == BZ_C128) {
+        const double2 v = ((const double2 *)f)[i];
+        return {split(v.x), split(v.y)};
+    }
+    const float2 v = ((const float2 *)f)[i];
+    return {{v.x, 0.f}, {v.y, 0.f}};
+}
+
+// R-point transform in registers (sign +), natural order.
+template <int R> __device__ __forceinline__ void dft_reg(ffc (&v)[R]) {
+    if constexpr (R == 2) {
+        const ffc a = v[0];
+        v[0] = add(a, v[1]);
+        v[1] = sub(a, v[1]);
+    } else if constexpr (R == 3) {
+        // -1/2 and sqrt(3)/2 from the roots' table (exactly -1/2; sqrt(3)/2 to 48 bits)
+        const ff s3 = root<3>(1).y;
+        const ffc t = add(v[1], v[2]), d = sub(v[1], v[2]), m = sub(v[0], half(t));
+        const ff z = {0.f, 0.f};
+        const ffc r = times_i({fdot<1>(d.x, s3, z, z), fdot<1>(d.y, s3, z, z)});
+        v[0] = add(v[0], t);
+        v[1] = add(m, r);
+        v[2] = sub(m, r);
+    } else if constexpr (R == 4) {
+        const ffc s0 = add(v[0], v[2]), d0 = sub(v[0], v[2]), s1 = add(v[1], v[3]), d1 = times_i(sub(v[1], v[3]));
+        v[0] = add(s0, s1);
+        v[2] = sub(s0, s1);
+        v[1] = add(d0, d1);
+        v[3] = sub(d0, d1);
+    } else if constexpr (R == 8) {
+        ffc e[4] = {v[0], v[2], v[4], v[6]}, o[4] = {v[1], v[3], v[5], v[7]};
+        dft_reg<4>(e);
+        dft_reg<4>(o);
+        o[1] = mul(o[1], root<8>(1));
+        o[2] = times_i(o[2]);
+        o[3] = mul(o[3], root<8>(3));
+        #pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            v[k] = add(e[k], o[k]);
+            v[k + 4] = sub(e[k], o[k]);
+        }
+    }
+}
+
+__device__ __forceinline__ ffc lane_xor(ffc a, int m) {
+    return {{__shfl_xor_sync(0xffffffffu, a.x.h, m), __shfl_xor_sync(0xffffffffu, a.x.l, m)},
+            {__shfl_xor_sync(0xffffffffu, a.y.h, m), __shfl_xor_sync(0xffffffffu, a.y.l, m)}};
+}
+// 8-point transform over 8 lanes (sign +): lane l ends with q = bitrev(l); w8 = W8^(l mod 4) where l >= 4,
+// else 1.
+__device__ __forceinline__ ffc dft_lanes(ffc v, int l, ffc w8) {
+    v = mul(add(lane_xor(v, 4), l & 4 ? neg(v) : v), w8);
+    v = add(lane_xor(v, 2), l & 2 ? neg(v) : v);
+    if ((l & 3) == 3) v = times_i(v);
+    return add(lane_xor(v, 1), l & 1 ? neg(v) : v);
+}
+
+// The lane's twiddles, and one line: x[l + 8 m] in v[m] -> X[r + R q] in v[r].  Every lane of the warp takes part.
+template <int N> struct LineFF {
+    static constexpr int R = N / 8;
+    ffc w[R], w8;
+    int l, q;
+    __device__ __forceinline__ LineFF(int lane8) : l(lane8) {
+        q = ((l & 1) << 2) | (l & 2) | (l >> 2);
+        #pragma unroll
+        for (int r = 1; r < R; ++r) w[r] = root<N>(l * r);
+        w8 = root<8>(l & 4 ? l & 3 : 0);
+    }
+    __device__ __forceinline__ void operator()(ffc (&v)[R]) const {
+        dft_reg<R>(v);
+        #pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = dft_lanes(r ? mul(v[r], w[r]) : v[r], l, w8);
+    }
+};
+
+struct HArgs {
+    const void *f;             // [slots][N^3] (c64 / c128)
+    int dtype;
+    const int *slots, *count_dev;
+    float4 *scr;               // [slots][N^3] between the two launches (N = 24, 32)
+    float2 *h;                 // [slots][N^3]
+    float2 *fout;              // real data: the Hermitian, Nyquist-free part in FP32, or null
+    int col;                   // k_col32's layouts: fout [k3 < 16][k1][k2], h packed floats [j3][j1][j2]
+};
+
+// fhat(k) of the instance, or (fout) its Hermitian part, zero where an index is N / 2, which is also
+// stored.
+template <int N> __device__ __forceinline__ ffc input(const HArgs &a, size_t vol, int k1, int k2, int k3) {
+    const size_t i = vol + ((size_t)k1 * N + k2) * N + k3;
+    if (!a.fout) return load_ff(a.f, a.dtype, i);
+    constexpr int H = N / 2;
+    ffc v = {{0.f, 0.f}, {0.f, 0.f}};
+    if (k1 != H && k2 != H && k3 != H) {
+        ffc c = load_ff(a.f, a.dtype, vol + ((size_t)((N - k1) % N) * N + (N - k2) % N) * N + (N - k3) % N);
+        c.y = fneg(c.y);
+        v = half(add(load_ff(a.f, a.dtype, i), c));
+    }
+    if (!a.col) a.fout[i] = round2(v);
+    else if (k3 < H) a.fout[vol + ((size_t)k3 * N + k1) * N + k2] = round2(v);
+    return v;
+}
+
+// Axes 3 and 2 of the R planes k1 = k10 .. into s[R][N][N + 1] ([k1][j2][j3]); 8 N threads a plane.
+template <int N, int P>
+__device__ __forceinline__ void planes_ff(const HArgs &a, const LineFF<N> &F, size_t vol, int k10, float4 *s) {
+    constexpr int R = N / 8, LD = N + 1;
+    const int pl = threadIdx.x / (8 * N), line = threadIdx.x / 8 % N;
+    float4 *sp = s + pl * N * LD;
+    ffc v[R];
+    #pragma unroll
+    for (int m = 0; m < R; ++m) v[m] = input<N>(a, vol, k10 + pl, line, F.l + 8 * m);
+    F(v);                                                 // k3 -> j3 of row k2 = line
+    #pragma unroll
+    for (int r = 0; r < R; ++r) sp[line * LD + r + R * F.q] = pack(v[r]);
+    __syncthreads();
+    #pragma unroll
+    for (int m = 0; m < R; ++m) v[m] = unpack(sp[(F.l + 8 * m) * LD + line]);
+    F(v);                                                 // k2 -> j2 of column j3 = line
+    __syncthreads();
+    #pragma unroll
+    for (int r = 0; r < R; ++r) sp[(r + R * F.q) * LD + line] = pack(v[r]);
+    __syncthreads();
+}
+
+// N = 24, 32: the plane k1 = blockIdx.x of instance blockIdx.y to scr ([k1][j2][j3]; col: [k1][j3][j2]).
+template <int N> __global__ void __launch_bounds__(8 * N) k_hff_plane(HArgs a) {
+    __shared__ float4 s[N * (N + 1)];
+    if (a.count_dev && (int)blockIdx.y >= *a.count_dev) return;
+    const size_t vol = (size_t)(a.slots ? a.slots[blockIdx.y] : blockIdx.y) * N * N * N;
+    const int k1 = blockIdx.x;
+    planes_ff<N, 1>(a, LineFF<N>(threadIdx.x & 7), vol, k1, s);
+    float4 *o = a.scr + vol + (size_t)k1 * N * N;
+    for (int e = threadIdx.x; e < N * N; e += 8 * N)
+        o[e] = a.col ? s[(e % N) * (N + 1) + e / N] : s[(e / N) * (N + 1) + e % N];
+}
+// The lines along axis 1: (u, v) = (j2, j3), or (j3, j2) for col; u = blockIdx.x.
+template <int N> __global__ void __launch_bounds__(8 * N) k_hff_line(HArgs a) {
+    constexpr int R = N / 8;
+    if (a.count_dev && (int)blockIdx.y >= *a.count_dev) return;
+    const size_t vol = (size_t)(a.slots ? a.slots[blockIdx.y] : blockIdx.y) * N * N * N;
+    // four adjacent lines of a warp, eight lanes each
+    const int w = threadIdx.x >> 5, u = blockIdx.x, v0 = 4 * w + (threadIdx.x & 3);
+    // lanes of a line are 4 apart so that its four neighbours' elements are adjacent in memory; the
+    // shuffles want them in one group of 8: transposed on the way in and out by a shuffle
+    const int lane = threadIdx.x & 31, l8 = lane >> 2, src = (lane & 7) * 4 + (lane >> 3), back = (lane & 3) * 8 + l8;
+    const LineFF<N> F(lane & 7);
+    const float4 *in = a.scr + vol + (size_t)u * N + v0;
+    ffc v[R];
+    #pragma unroll
+    for (int m = 0; m < R; ++m) {
+        const float4 t = in[(size_t)(l8 + 8 * m) * N * N];
+        v[m] = {{__shfl_sync(0xffffffffu, t.x, src), __shfl_sync(0xffffffffu, t.y, src)},
+                {__shfl_sync(0xffffffffu, t.z, src), __shfl_sync(0xffffffffu, t.w, src)}};
+    }
+    F(v);
+    const int q = ((l8 & 1) << 2) | (l8 & 2) | (l8 >> 2);  // of the lane that wrote this thread's value
+    #pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const float2 o = round2(v[r]);
+        const float2 t = make_float2(__shfl_sync(0xffffffffu, o.x, back), __shfl_sync(0xffffffffu, o.y, back));
+        const int j1 = r + R * q;
+        if (a.col) ((float *)(a.h + vol))[((size_t)u * N + j1) * N + v0] = t.x;
+        else a.h[vol + ((size_t)j1 * N + u) * N + v0] = t;
+    }
+}
+
+// N = 8, 16: one cluster of 8 CTAs per instance.
+template <int N> __global__ void __launch_bounds__(N * N) k_hff_cube(HArgs a) {
+    constexpr int R = N / 8, LD = N + 1;
+    __shared__ float4 s[R * N * LD];
+    if (a.count_dev && (int)blockIdx.y >= *a.count_dev) return;          // uniform over the cluster
+    const size_t vol = (size_t)(a.slots ? a.slots[blockIdx.y] : blockIdx.y) * N * N * N;
+    const int c = (int)cooperative_groups::this_cluster().block_rank();
+    const LineFF<N> F(threadIdx.x & 7);
+    planes_ff<N, R>(a, F, vol, R * c, s);
+    cooperative_groups::this_cluster().sync();
+    // lines (j2, j3), j2 = R c .. R c + R - 1
+    const int j2 = R * c + threadIdx.x / (8 * N), j3 = threadIdx.x / 8 % N;
+    ffc v[R];
+    #pragma unroll
+    for (int m = 0; m < R; ++m) {
+        const int k1 = F.l + 8 * m;
+        const uint32_t ad = dsmem_addr(&s[(k1 % R) * N * LD + j2 * LD + j3], (uint32_t)(k1 / R));
+        float4 t;
+        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];\n"
+                     : "=f"(t.x), "=f"(t.y), "=f"(t.z), "=f"(t.w) : "r"(ad) : "memory");
+        v[m] = unpack(t);
+    }
+    F(v);
+    #pragma unroll
+    for (int r = 0; r < R; ++r) a.h[vol + ((size_t)(r + R * F.q) * N + j2) * N + j3] = round2(v[r]);
+    cooperative_groups::this_cluster().sync();               // no CTA leaves while its planes are read
+}
+
+// 2D: one cluster of 8 CTAs, rows k1 = R c ..
+template <int N> __global__ void __launch_bounds__(N < 32 ? 32 : N) k_hff_2d(const void *f, int dtype, float2 *h) {
+    constexpr int R = N / 8, LD = N + 1;
+    __shared__ float4 s[R * LD];
+    const int c = (int)cooperative_groups::this_cluster().block_rank();
+    const LineFF<N> F(threadIdx.x & 7);
+    const int i = threadIdx.x / 8 < R ? threadIdx.x / 8 : R - 1;         // spare lanes repeat the last line
+    ffc v[R];
+    #pragma unroll
+    for (int m = 0; m < R; ++m) v[m] = load_ff(f, dtype, (size_t)(R * c + i) * N + F.l + 8 * m);
+    F(v);                                                    // k2 -> j2
+    #pragma unroll
+    for (int r = 0; r < R; ++r) s[i * LD + r + R * F.q] = pack(v[r]);
+    cooperative_groups::this_cluster().sync();
+    #pragma unroll
+    for (int m = 0; m < R; ++m) {
+        const int k1 = F.l + 8 * m;
+        const uint32_t ad = dsmem_addr(&s[(k1 % R) * LD + R * c + i], (uint32_t)(k1 / R));
+        float4 t;
+        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];\n"
+                     : "=f"(t.x), "=f"(t.y), "=f"(t.z), "=f"(t.w) : "r"(ad) : "memory");
+        v[m] = unpack(t);
+    }
+    F(v);                                                    // k1 -> j1 of column j2 = R c + i
+    #pragma unroll
+    for (int r = 0; r < R; ++r) h[(size_t)(r + R * F.q) * N + R * c + i] = round2(v[r]);
+    cooperative_groups::this_cluster().sync();
+}
+
+template <class... P, class... A>
+cudaError_t launch8(void (*k)(P...), dim3 grid, int threads, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 8;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, args...);
+}
+
+}  // namespace
+
+bz_status hff_launch(int N, const void *f, int dtype, const int *slots, const int *count_dev, int count,
+                     double2 *scr, float2 *h, cudaStream_t st, float2 *fsym, bool col) {
+    if (count <= 0) return BZ_OK;
+    if ((col && N != 32) || (fsym && N == 24)) return BZ_ERR_UNSUPPORTED;
+    HArgs a = {f, dtype, slots, count_dev, (float4 *)scr, h, fsym, col};
+    cudaError_t e = cudaSuccess;
+    switch (N) {
+        case 8: e = launch8(k_hff_cube<8>, dim3(8, count), 64, st, a); break;
+        case 16: e = launch8(k_hff_cube<16>, dim3(8, count), 256, st, a); break;
+        case 24:
+            k_hff_plane<24><<<dim3(24, count), 192, 0, st>>>(a);
+            k_hff_line<24><<<dim3(24, count), 192, 0, st>>>(a);
+            break;
+        case 32:
+            k_hff_plane<32><<<dim3(32, count), 256, 0, st>>>(a);
+            k_hff_line<32><<<dim3(32, count), 256, 0, st>>>(a);
+            break;
+        default: return BZ_ERR_UNSUPPORTED;
+    }
+    BZ_CUDA_TRY(e);
+    BZ_CUDA_TRY(cudaGetLastError());
+    return BZ_OK;
+}
+
+bz_status hff_launch_2d(int N, const void *f, int dtype, float2 *h, cudaStream_t st) {
+    cudaError_t e = cudaSuccess;
+    switch (N) {
+        case 8: e = launch8(k_hff_2d<8>, dim3(8), 32, st, f, dtype, h); break;
+        case 16: e = launch8(k_hff_2d<16>, dim3(8), 32, st, f, dtype, h); break;
+        case 32: e = launch8(k_hff_2d<32>, dim3(8), 32, st, f, dtype, h); break;
+        case 64: e = launch8(k_hff_2d<64>, dim3(8), 64, st, f, dtype, h); break;
+        default: return BZ_ERR_UNSUPPORTED;
+    }
+    BZ_CUDA_TRY(e);
+    return BZ_OK;
+}
+
+}  // namespace bz

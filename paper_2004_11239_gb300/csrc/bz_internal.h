@@ -72,9 +72,9 @@ struct Plan {
     int fused_C = 0;                // CTAs per cluster
     int fused_G = 0;                // resident clusters (persistent grid)
     float fused_ms = 0.f;           // timed collide of the selected cluster size
-    int h_fp64 = 1;                 // fused path: h formed in FP64 (1) or in FP32 in-kernel (0)
-    double2 *fin64 = nullptr;       // [N^3] FP64 stage input (RK4) for the FP64 h pass
-    double2 *scr64 = nullptr;       // [N^3] FP64 scratch of the h pass
+    int h_fp64 = 1;                 // fused path: h formed in double-float (1) or in FP32 in-kernel (0)
+    double2 *fin64 = nullptr;       // [N^3] FP64 stage input (RK4) for the h pass
+    double2 *scr64 = nullptr;       // [N^3] scratch of the h pass (16 bytes per mode)
     const void *src = nullptr;      // FP64-capable source of h for the next fused collide
     int src_dtype = BZ_C128;
     float2 *part = nullptr;         // [fused_G][N^3] per-cluster partial sums
@@ -177,14 +177,16 @@ struct ItemArgs {
 int fused_candidates(int N, int *cs);
 cudaError_t fused_setup(int N, int C, int *G, bool real);
 bz_status launch_fused(const Plan &pl, const ItemArgs &a, cudaStream_t st);
-// h[slot] = IFFT(f[slot]) computed in FP64 and stored FP32 for the active slots (N <= 32).
-// Kernel launches of one h64_launch: three line passes (N = 32: the k3 and k2 passes as one).
-inline int h64_launches(int N) { return N == 32 ? 2 : 3; }
+// bz_hff.cu: h[slot] = IFFT(f[slot]) in double-float arithmetic (about 47 bits), stored FP32, for the
+// active slots (N <= 32).  Kernel launches of one hff_launch:
+inline int hff_launches(int N) { return N <= 16 ? 1 : 2; }
 // fsym (BZ_DATA_REAL, N a power of two): transform the Hermitian, Nyquist-free part of f and
 // store that part in FP32 to fsym; col (N = 32): in k_col32's layouts ([k3 < 16][k1][k2], and h as
-// packed floats [j3][j1][j2]; the same stride of N^3 float2 per slot).
-bz_status h64_launch(int N, const void *f, int dtype, const int *slots, const int *count_dev, int count,
+// packed floats [j3][j1][j2]; the same stride of N^3 float2 per slot).  scr: 16 N^3 bytes per slot
+// (N = 24, 32).
+bz_status hff_launch(int N, const void *f, int dtype, const int *slots, const int *count_dev, int count,
                      double2 *scr, float2 *h, cudaStream_t st, float2 *fsym = nullptr, bool col = false);
+bz_status hff_launch_2d(int N, const void *f, int dtype, float2 *h, cudaStream_t st);
 bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches);
 // bz_real.cu (BZ_DATA_REAL): the pair table from alpha (after ftable_build); pl.fsym and
 // pl.fsym64 from a c64 / c128 array
@@ -195,7 +197,7 @@ bz_status reduce_sym(Plan &pl, int nblk, cudaStream_t st);
 // chunked pipeline: pl.acc (V, FP64) <- Q in place, with pl.acc_s (X)
 bz_status sym_output(Plan &pl, cudaStream_t st);
 
-// bz_pair3.cu (BZ_DATA_REAL, N = 32, FP64 h): resident clusters and launch of k_pair3
+// bz_pair3.cu (BZ_DATA_REAL, N = 32): resident clusters and launch of k_pair3
 cudaError_t pair3_setup(int *G);
 bz_status launch_pair3(const Plan &pl, const ItemArgs &a, cudaStream_t st);
 

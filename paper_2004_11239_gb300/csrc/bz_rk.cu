@@ -105,7 +105,7 @@ bz_status rk4_steps(Plan &pl, void *fhat, int dtype, double dt, int nsteps, cuda
     const int bs = 256, gs = (n + bs - 1) / bs;
     double2 *f0 = pl.rk, *fsum = pl.rk + n;
     k_rk_init<<<gs, bs, 0, st>>>(fhat, dtype, f0, pl.fin, pl.fin64, n);
-    pl.src = pl.fin64;             // stage inputs for the FP64 h pass (fused plans)
+    pl.src = pl.fin64;             // stage inputs for the h pass (fused plans)
     pl.src_dtype = BZ_C128;
     int nl = 1;
     for (int step = 0; step < nsteps; ++step) {
