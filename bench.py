@@ -110,7 +110,7 @@ _PROFILES = {
     "mixed": ("mixed_rk4_n32.md", ("bz_mixed.cu", "bz_fft.cuh", "bz_cluster.cuh")),
     "fused_real": ("fused_real_rk4_n32.md", ("bz_fused_kernel.cuh", "bz_fft.cuh", "bz_cluster.cuh")),
     "pair3": ("pair3_rk4_n32.md", ("bz_pair3.cu", "bz_fft.cuh", "bz_cluster.cuh")),
-    "n64:pipeline": ("chunked_single_n64.md", ("bz_collide.cu", "bz_chunk64.cu", "bz_fft.cuh")),
+    "n64:pipeline": ("chunked_single_n64.md", ("bz_lines.cu", "bz_fft.cuh")),
 }
 
 
@@ -681,7 +681,7 @@ def _pipeline_roofline(w, ms_per_collide, peaks, src, traffic_key=None):
     for r in (alu, hbm):
         r["frac"] = r["achieved"] / r["peak"]
     roof, other = (alu, hbm) if alu["frac"] >= hbm["frac"] else (hbm, alu)
-    roof.update({"kernel": "chunked pipeline (plane, pencil, plane, reduce on two streams)",
+    roof.update({"kernel": "chunked pipeline (lines, planes, lines on two streams)",
                  "traffic": _profiled_traffic(traffic_key) if traffic_key else None,
                  "peak_source": alu_src if roof is alu else src, "sm_count": sms,
                  "avg_launch_us": ms_per_collide * 1e3, "unit_of_work": f"one collide of {P} terms",

@@ -93,7 +93,7 @@ enum { BZ_CONV_CIRCULAR = 0, BZ_CONV_PADDED = 1 };
 
 /* Collide pipelines.  FUSED: one thread-block cluster per term keeps the whole field in
  * (distributed) shared memory from twiddle to weighted accumulation (N <= 32).  CHUNKED:
- * four kernels per chunk of terms over an L2-sized scratch buffer (every N).  AUTO picks
+ * kernels over chunks of terms in an L2-sized scratch buffer (every N).  AUTO picks
  * FUSED where it applies. */
 enum { BZ_PIPE_AUTO = 0, BZ_PIPE_FUSED = 1, BZ_PIPE_CHUNKED = 2 };
 
@@ -417,7 +417,8 @@ bz_status bz_server_stats(bz_server *server, long *completed, long *steps, size_
 /* Stops the worker after its current iteration and frees everything. */
 void bz_server_destroy(bz_server *server);
 
-/* Kernel kinds reported by bz_plan_timing. */
+/* Kernel kinds reported by bz_plan_timing.  On the chunked pipeline at N = 48 and 64: PENCIL the first
+ * line pass, PLANE_INV the plane pass (both directions), REDUCE the accumulating line pass. */
 enum { BZ_K_PLANE_INV = 0, BZ_K_PENCIL = 1, BZ_K_PLANE_FWD = 2, BZ_K_REDUCE = 3, BZ_K_OTHER = 4,
        BZ_K_FUSED = 5 };
 

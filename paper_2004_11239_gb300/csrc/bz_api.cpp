@@ -30,7 +30,9 @@ void free_plan(bz::Plan &p) {
     cudaFree(p.alpha); cudaFree(p.tw); cudaFree(p.rule_buf); cudaFree(p.rule_off);
     cudaFree(p.term_dev); cudaFree(p.S); cudaFree(p.h); cudaFree(p.fin); cudaFree(p.acc);
     cudaFree(p.rk); cudaFree(p.mom); cudaFree(p.part); cudaFree(p.fin64); cudaFree(p.scr64);
-    cudaFree(p.wimg); cudaFree(p.dev_err); cudaFree(p.apair); cudaFree(p.fsym); cudaFree(p.fsym64);
+    cudaFree(p.wimg); cudaFree(p.dev_err); cudaFree(p.apair); cudaFree(p.fsym);
+    cudaFree(p.lstate); cudaFree(p.xs);
+    p.lstate = nullptr; p.xs = nullptr;
     cudaFree(p.acol); cudaFree(p.fcol); cudaFree(p.hcol);
     p.acol = nullptr; p.fcol = nullptr; p.hcol = nullptr;
     cudaFree(p.cpair); cudaFree(p.part_s); cudaFree(p.S_s); cudaFree(p.acc_s);
@@ -44,7 +46,7 @@ void free_plan(bz::Plan &p) {
     if (p.ev_fork) cudaEventDestroy(p.ev_fork);
     p.ev_fork = nullptr;
     p.xn = 0;
-    p.wimg = nullptr; p.dev_err = nullptr; p.apair = nullptr; p.fsym = nullptr; p.fsym64 = nullptr;
+    p.wimg = nullptr; p.dev_err = nullptr; p.apair = nullptr; p.fsym = nullptr;
     p.cpair = nullptr; p.part_s = nullptr; p.S_s = nullptr; p.acc_s = nullptr;
     p.part = nullptr; p.fin64 = nullptr; p.scr64 = nullptr; p.src = nullptr;
     p.alpha = nullptr; p.tw = nullptr; p.rule_buf = nullptr; p.rule_off = nullptr;
@@ -217,8 +219,8 @@ bz_status create(bz_plan **out, const bz_plan_desc *d) {
     if (chunk <= 0) {
         // two waves of plane CTAs, within an L2-sized scratch; one wave per stream on two streams
         if (bz::collide_set_attributes(N) != cudaSuccess) { delete h; return BZ_ERR_CUDA; }
-        chunk = bz::chunk_terms_for(N);
-        if (two_streams && chunk > 1) chunk = (chunk + bz::kExtraStreams) / (1 + bz::kExtraStreams);
+        chunk = bz::lines_N(N) ? bz::lines_chunk(N) : bz::chunk_terms_for(N);
+        if (!bz::lines_N(N) && two_streams && chunk > 1) chunk = (chunk + bz::kExtraStreams) / (1 + bz::kExtraStreams);
     }
     if (chunk > pl.P) chunk = pl.P;
     if (chunk > 65535) chunk = 65535;
@@ -254,9 +256,9 @@ bz_status create(bz_plan **out, const bz_plan_desc *d) {
     if (s == BZ_OK && pl.col32) {
         if ((s = dmalloc(&pl.acol, (size_t)pl.P * bz::kCol32Part * sizeof(float2))) == BZ_OK &&
             (s = dmalloc(&pl.fcol, field)) == BZ_OK && (s = dmalloc(&pl.hcol, n3 * sizeof(float))) == BZ_OK &&
-            (s = dmalloc(&pl.fsym, field)) == BZ_OK && (s = dmalloc(&pl.fsym64, n3 * sizeof(double2))) == BZ_OK)
+            (s = dmalloc(&pl.fsym, field)) == BZ_OK)
             s = bz::col32_table(pl);
-        pl.ws_bytes += 2 * field + n3 * (sizeof(float) + sizeof(double2));
+        pl.ws_bytes += 2 * field + n3 * sizeof(float);
     } else if (s == BZ_OK && pl.real) {
         // term pairs (2q, 2q + 1) share a radial node (M even) and one pair of transforms
         const size_t ns = (size_t)3 * N * N;
@@ -264,9 +266,9 @@ bz_status create(bz_plan **out, const bz_plan_desc *d) {
             (s = dmalloc(&pl.cpair, (size_t)(pl.P / 2) * ns * sizeof(float2))) == BZ_OK &&
             (s = dmalloc(&pl.S_s, (size_t)pl.chunk * ns * sizeof(float2))) == BZ_OK &&
             (s = dmalloc(&pl.acc_s, ns * sizeof(double2))) == BZ_OK &&
-            (s = dmalloc(&pl.fsym, field)) == BZ_OK && (s = dmalloc(&pl.fsym64, n3 * sizeof(double2))) == BZ_OK)
+            (s = dmalloc(&pl.fsym, field)) == BZ_OK)
             s = bz::build_pair_table(pl);
-        pl.ws_bytes += field + n3 * sizeof(double2) + (size_t)pl.chunk * ns * sizeof(float2) + ns * sizeof(double2);
+        pl.ws_bytes += field + (size_t)pl.chunk * ns * sizeof(float2) + ns * sizeof(double2);
     }
     if (s != BZ_OK) {
         free_plan(pl);
@@ -309,22 +311,37 @@ bz_status create(bz_plan **out, const bz_plan_desc *d) {
         delete h;
         return BZ_ERR_UNSUPPORTED;
     }
+    if (bz::lines_N(N) && dim == 3) {
+        const size_t states = (size_t)(1 + bz::kExtraStreams) * bz::lines_splits(N);
+        if ((s = bz::lines_set_attributes(N) == cudaSuccess ? BZ_OK : BZ_ERR_CUDA) != BZ_OK ||
+            (s = dmalloc(&pl.lstate, states * n3 * sizeof(float4))) != BZ_OK ||
+            (pl.real && (s = dmalloc(&pl.xs, (size_t)(pl.P / 2) * 3 * N * N * sizeof(float2))) != BZ_OK)) {
+            cudaGetLastError();
+            free_plan(pl);
+            delete h;
+            return s;
+        }
+        pl.ws_bytes += states * n3 * sizeof(float4) + (pl.real ? (size_t)(pl.P / 2) * 3 * N * N * sizeof(float2) : 0);
+    }
     if (two_streams && !pl.use_fused) {
         // the other lanes' scratch and accumulators; without them the chunks stay on one stream
         const size_t ns = (size_t)3 * N * N;
         bool ok = cudaEventCreateWithFlags(&pl.ev_fork, cudaEventDisableTiming) == cudaSuccess;
         for (int e = 0; ok && e < bz::kExtraStreams; ++e) {
+            const bool acc = !bz::lines_N(N);   // bz_lines.cu keeps every lane's sums in pl.lstate
             ok = dmalloc(&pl.xS[e], (size_t)pl.chunk * field) == BZ_OK &&
-                 dmalloc(&pl.xacc[e], n3 * sizeof(double2)) == BZ_OK;
-            if (ok && pl.real)
+                 (!acc || dmalloc(&pl.xacc[e], n3 * sizeof(double2)) == BZ_OK);
+            if (ok && pl.real && acc)
                 ok = dmalloc(&pl.xS_s[e], (size_t)pl.chunk * ns * sizeof(float2)) == BZ_OK &&
                      dmalloc(&pl.xacc_s[e], ns * sizeof(double2)) == BZ_OK;
             ok = ok && cudaStreamCreateWithFlags(&pl.xst[e], cudaStreamNonBlocking) == cudaSuccess &&
                  cudaEventCreateWithFlags(&pl.xev_join[e], cudaEventDisableTiming) == cudaSuccess;
             if (ok) {
                 pl.xn = e + 1;
-                pl.ws_bytes += (size_t)pl.chunk * field + n3 * sizeof(double2) +
-                               (pl.real ? (size_t)pl.chunk * ns * sizeof(float2) + ns * sizeof(double2) : 0);
+                pl.ws_bytes += (size_t)pl.chunk * field;
+                if (acc)
+                    pl.ws_bytes += n3 * sizeof(double2) +
+                                   (pl.real ? (size_t)pl.chunk * ns * sizeof(float2) + ns * sizeof(double2) : 0);
             }
         }
         if (!ok) cudaGetLastError();   // the lanes that were set up stay in use

@@ -5,7 +5,7 @@
 // stream's scratch and accumulator, overlapping the others; the sums are added at the end):
 //   plane_inv  (planes k1):  S = IFFT_{axes 3,2}( beta_p(m) fhat_m )       twiddle + 2 axes
 //   pencil     (lines k1):   S = FFT_1( h . IFFT_1(S) )                     product in registers
-// (at N = 64 the plane and pencil passes are the radix-8 x 8 kernels of bz_chunk64.cu)
+// (N = 48 and 64 have kernels and an order of passes of their own: bz_lines.cu)
 //   plane_fwd  (planes k1):  S = alpha_p . FFT_{axes 3,2}(S)                 weight in the epilogue
 //   reduce     (modes k):    acc += sum_t S[t]  (compensated FP32 over every term, FP64 at the end)
 // h = IFFT(fhat) is formed once per call by plane_inv without twiddles plus an
@@ -19,13 +19,12 @@
 namespace bz {
 
 template <int N> struct Cfg {
-    // planes per CTA; N = 64 takes two so that three CTAs (12 warps) share an SM
-    static constexpr int PPC = N <= 8 ? 8 : (N <= 16 ? 16 : (N <= 32 ? 8 : (N <= 48 ? 4 : 2)));
+    static constexpr int PPC = N <= 8 ? 8 : (N <= 16 ? 16 : (N <= 32 ? 8 : 4));   // planes per CTA
     static constexpr int LD = N + 1;                                              // padded row
     static constexpr int THREADS = PPC * N;
     static constexpr size_t SMEM = ((size_t)PPC * N * LD + 6 * N) * sizeof(float2);   // planes + a pair's twiddles
     // resident CTAs per SM the register budget is held to (shared memory allows as many)
-    static constexpr int MINB = N == 64 ? 3 : (N == 48 ? 2 : 1);
+    static constexpr int MINB = N == 48 ? 2 : 1;
 };
 
 // ---------------------------------------------------------------------------------------
@@ -200,7 +199,7 @@ struct Kahan4 {
 // (zero bytes are the empty sum), and k_kahan_fold turns them into FP64 once at the end.  The
 // per-chunk pass thus runs no FP64 arithmetic, whose rate on this part is a small fraction of
 // FP32's.  S2 / n2 / acc2 (or null): a second field summed the same way (the Nyquist sums).
-__global__ void __launch_bounds__(256, 4)        // <= 64 registers: a launch at N = 64 fits one wave
+__global__ void __launch_bounds__(256, 4)
 k_reduce(const float2 *__restrict__ S, int T, int n3, double2 *__restrict__ acc,
          const float2 *__restrict__ S2 = nullptr, int n2 = 0, double2 *__restrict__ acc2 = nullptr) {
     int k2 = blockIdx.x * blockDim.x + threadIdx.x;          // mode pair index
@@ -336,10 +335,6 @@ int supported_N(int N) {
 }
 
 template <int N> static cudaError_t set_attrs() {
-    if constexpr (N == 64) {
-        const cudaError_t e = chunk64_set_attributes();
-        if (e != cudaSuccess) return e;
-    }
     const void *ks[4] = {(const void *)k_plane_inv<N, false>, (const void *)k_plane_inv<N, true>,
                          (const void *)k_plane_fwd<N, false>, (const void *)k_plane_fwd<N, true>};
     for (const void *k : ks) {
@@ -351,8 +346,7 @@ template <int N> static cudaError_t set_attrs() {
 
 // Terms per chunk: two waves of plane CTAs (resident CTAs / CTAs per term, twice), so that
 // the second wave's loads overlap the first wave's arithmetic, capped by a scratch of 64 MB
-// that stays in L2 (measured at N = 64, P = 1024, real data: 2.56 ms per collide with one
-// wave of 14 pairs, 2.18 ms with two).
+// that stays in L2.
 template <int N> static int chunk_for() {
     int per_sm = 0, dev = 0, sms = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_plane_inv<N, false>, Cfg<N>::THREADS, Cfg<N>::SMEM) !=
@@ -374,8 +368,6 @@ int chunk_terms_for(int N) {
         case 16: return chunk_for<16>();
         case 24: return chunk_for<24>();
         case 32: return chunk_for<32>();
-        case 48: return chunk_for<48>();
-        case 64: return chunk_for<64>();
     }
     return 1;
 }
@@ -387,31 +379,26 @@ cudaError_t collide_set_attributes(int N) {
         case 24: return set_attrs<24>();
         case 32: return set_attrs<32>();
         case 48: return set_attrs<48>();
-        case 64: return set_attrs<64>();
+        case 64: return cudaSuccess;                      // (bz_lines.cu)
     }
     return cudaErrorInvalidValue;
 }
 
-// Plane passes of a chunk: at N = 64 the radix-8 one-plane-per-CTA kernels, else the generic ones.
+// The passes of a chunk of T terms (pairs).
 template <int N, bool PAIR>
 static void plane_inv(const float2 *fin, const float2 *tw, float2 *S, int p0, int T, int use_tw, cudaStream_t st) {
-    constexpr int PPC = Cfg<N>::PPC;
-    if constexpr (N == 64) plane_inv64(fin, tw, S, p0, T, use_tw, PAIR, st);
-    else k_plane_inv<N, PAIR><<<dim3(N / PPC, T), Cfg<N>::THREADS, Cfg<N>::SMEM, st>>>(fin, tw, S, p0, use_tw);
+    k_plane_inv<N, PAIR><<<dim3(N / Cfg<N>::PPC, T), Cfg<N>::THREADS, Cfg<N>::SMEM, st>>>(fin, tw, S, p0, use_tw);
 }
 
 template <int N, bool PAIR>
 static void plane_fwd(float2 *S, const float2 *alpha, int p0, int T, const float2 *cpair, float2 *Ss, const float *gsc,
                       int M, cudaStream_t st) {
-    constexpr int PPC = Cfg<N>::PPC;
-    if constexpr (N == 64) plane_fwd64(S, alpha, p0, T, cpair, Ss, gsc, M, PAIR, st);
-    else k_plane_fwd<N, PAIR><<<dim3(N / PPC, T), Cfg<N>::THREADS, Cfg<N>::SMEM, st>>>(S, alpha, p0, cpair, Ss, gsc, M);
+    k_plane_fwd<N, PAIR><<<dim3(N / Cfg<N>::PPC, T), Cfg<N>::THREADS, Cfg<N>::SMEM, st>>>(S, alpha, p0, cpair, Ss, gsc, M);
 }
 
 template <int N, int MODE>
 static void pencil(float2 *S, const float2 *h, float2 *out, int T, cudaStream_t st) {
-    if constexpr (N == 64) pencil64(S, h, out, T, MODE, st);
-    else k_pencil<N, MODE><<<dim3((N * N + 127) / 128, T), 128, 0, st>>>(S, h, out);
+    k_pencil<N, MODE><<<dim3((N * N + 127) / 128, T), 128, 0, st>>>(S, h, out);
 }
 
 // BZ_DATA_REAL: the Hermitian part of the input (sym_input) feeds h and the pair passes; the
@@ -427,9 +414,7 @@ static bz_status run_chunks_real(Plan &pl, int p0, int p1, cudaStream_t st, int 
     bz_status s = sym_input(pl, pl.src ? pl.src : (const void *)pl.fin, pl.src ? pl.src_dtype : BZ_C64, st);
     if (s != BZ_OK) return s;
     plane_inv<N, false>(pl.fsym, pl.tw, pl.S, 0, 1, 0, st);
-    // h is real: at N = 64 it is stored as N^3 packed floats (half the bytes the pair pencils read)
-    if constexpr (N == 64) pencil64(pl.S, nullptr, pl.h, 1, 3, st);
-    else pencil<N, 0>(pl.S, nullptr, pl.h, 1, st);
+    pencil<N, 0>(pl.S, nullptr, pl.h, 1, st);
     BZ_CUDA_TRY(cudaMemsetAsync(pl.acc, 0, (size_t)n3 * sizeof(double2), st));
     BZ_CUDA_TRY(cudaMemsetAsync(pl.acc_s, 0, (size_t)ns * sizeof(double2), st));
     tm_end(pl, st, TK_OTHER);
@@ -595,8 +580,8 @@ bz_status collide_core(Plan &pl, int p0, int p1, cudaStream_t st, int *launches)
         case 16: return run_chunks<16>(pl, p0, p1, st, launches);
         case 24: return run_chunks<24>(pl, p0, p1, st, launches);
         case 32: return run_chunks<32>(pl, p0, p1, st, launches);
-        case 48: return run_chunks<48>(pl, p0, p1, st, launches);
-        case 64: return run_chunks<64>(pl, p0, p1, st, launches);
+        case 48:
+        case 64: return collide_lines(pl, p0, p1, st, launches);
     }
     return BZ_ERR_ARG;
 }
@@ -739,7 +724,6 @@ extern "C" bz_status bz_collide_noalloc(const bz_plan *plan, const void *fhat, v
         case 24: return run_noalloc<24>(pl, fhat, Qhat, dtype, base, h64, T, st);
         case 32: return run_noalloc<32>(pl, fhat, Qhat, dtype, base, h64, T, st);
         case 48: return run_noalloc<48>(pl, fhat, Qhat, dtype, base, h64, T, st);
-        case 64: return run_noalloc<64>(pl, fhat, Qhat, dtype, base, h64, T, st);
     }
     return BZ_ERR_ARG;
 }

@@ -102,8 +102,11 @@ struct Plan {
     float2 *xS_s[kExtraStreams] = {};                // [chunk][3][N][N] (BZ_DATA_REAL)
     double2 *xacc[kExtraStreams] = {};               // [N^3]
     double2 *xacc_s[kExtraStreams] = {};             // [3][N][N] (BZ_DATA_REAL)
+    // N = 48, 64 (bz_lines.cu): running sums per lane and split [lanes][splits][N^3], and the term
+    // pairs' products [P / 2][3][N][N] on the Nyquist planes (BZ_DATA_REAL)
+    float4 *lstate = nullptr;
+    float2 *xs = nullptr;
     float2 *fsym = nullptr;         // [N^3] Hermitian part of fhat, Nyquist planes zero (FP32)
-    double2 *fsym64 = nullptr;      // [N^3] the same in FP64 (source of h)
     const float *gsc_cur = nullptr; // chunked pipeline inside a batch call: the slot's radial scale
                                     // r_i^(gamma_slot - gamma) per radial node (null: none)
     int *dev_err = nullptr;         // device flags: [0] a bounded wait of a kernel gave up,
@@ -188,8 +191,8 @@ bz_status hff_launch(int N, const void *f, int dtype, const int *slots, const in
                      double2 *scr, float2 *h, cudaStream_t st, float2 *fsym = nullptr, bool col = false);
 bz_status hff_launch_2d(int N, const void *f, int dtype, float2 *h, cudaStream_t st);
 bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches);
-// bz_real.cu (BZ_DATA_REAL): the pair table from alpha (after ftable_build); pl.fsym and
-// pl.fsym64 from a c64 / c128 array
+// bz_real.cu (BZ_DATA_REAL): the pair table from alpha (after ftable_build); pl.fsym from a
+// c64 / c128 array
 bz_status build_pair_table(Plan &pl);
 bz_status sym_input(Plan &pl, const void *f, int dtype, cudaStream_t st);
 // pl.acc <- Q from the nblk item sums of pl.part (V) and pl.part_s (X): one kernel
@@ -217,18 +220,16 @@ bz_status launch_mixed(const Plan &pl, const ItemArgs &a, cudaStream_t st);
 // one bounded wait that nothing completes, giving up after `limit` clocks (bz_plan_wait_selftest)
 bz_status wait_selftest(const Plan &pl, long long limit, cudaStream_t st);
 cudaError_t collide_set_attributes(int N);
-// bz_chunk64.cu: the plane and pencil passes of the chunked pipeline at N = 64 (radix 8 x 8)
-cudaError_t chunk64_set_attributes();
-void plane_inv64(const float2 *fin, const float2 *tw, float2 *S, int p0, int T, int use_tw, bool pair,
-                 cudaStream_t st);
-void plane_fwd64(float2 *S, const float2 *alpha, int p0, int T, const float2 *cpair, float2 *Ss, const float *gsc,
-                 int M, bool pair, cudaStream_t st);
-// pencil pass (axis 1) over T terms: mode 0 out = IFFT_1(S); 1 S = FFT_1(h . IFFT_1(S)); 2 as 1 with
-// h real (N^3 packed floats); 3 out = Re IFFT_1(S) as N^3 packed floats
-void pencil64(float2 *S, const float2 *h, float2 *out, int T, int mode, cudaStream_t st);
 void reduce_parts(const float2 *part, int nblk, int n, double2 *acc, cudaStream_t st);
 int chunk_terms_for(int N);          // after collide_set_attributes(N)
 int supported_N(int N);
+
+// bz_lines.cu: the chunked pipeline at N = 48 and 64; terms (pairs) of a chunk, running sums of a lane
+int lines_chunk(int N);
+int lines_splits(int N);
+inline bool lines_N(int N) { return N == 48 || N == 64; }
+cudaError_t lines_set_attributes(int N);
+bz_status collide_lines(Plan &pl, int p0, int p1, cudaStream_t st, int *launches);
 
 // bz_2d.cu (dim = 2)
 cudaError_t setup_2d(Plan &pl);                       // persistent grid size (pl.fused_G)

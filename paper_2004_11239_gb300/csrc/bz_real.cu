@@ -20,9 +20,8 @@ namespace bz {
 
 namespace {
 
-// fs (FP32 and FP64) from the caller's array (c64 or c128).
-__global__ void k_sym_in(const void *__restrict__ f, int dtype, int N, float2 *__restrict__ fs,
-                         double2 *__restrict__ fs64) {
+// fs (FP32) from the caller's array (c64 or c128).
+__global__ void k_sym_in(const void *__restrict__ f, int dtype, int N, float2 *__restrict__ fs) {
     const int n3 = N * N * N;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n3) return;
@@ -42,7 +41,6 @@ __global__ void k_sym_in(const void *__restrict__ f, int dtype, int N, float2 *_
         v = make_double2(0.5 * (a.x + b.x), 0.5 * (a.y - b.y));
     }
     fs[k] = make_float2((float)v.x, (float)v.y);
-    fs64[k] = v;
 }
 
 // Kahan-compensated FP32 sum.
@@ -190,7 +188,7 @@ bz_status build_pair_table(Plan &pl) {
 
 bz_status sym_input(Plan &pl, const void *f, int dtype, cudaStream_t st) {
     const int n3 = (int)modes(pl);
-    k_sym_in<<<(n3 + 255) / 256, 256, 0, st>>>(f, dtype, pl.N, pl.fsym, pl.fsym64);
+    k_sym_in<<<(n3 + 255) / 256, 256, 0, st>>>(f, dtype, pl.N, pl.fsym);
     BZ_CUDA_TRY(cudaGetLastError());
     return BZ_OK;
 }
