@@ -106,7 +106,7 @@ bz_status setup_col32(bz::Plan &pl) {
 bz_status select_fused(bz::Plan &pl, int forced, int ctas) {
     int cs[4];
     const bool mixed = pl.precision == BZ_PREC_BF16X3;
-    int nc = mixed ? 1 : bz::fused_candidates(pl.N, cs);
+    int nc = mixed ? 1 : bz::fused_candidates(pl.N, cs, forced);
     if (mixed) cs[0] = 8;
     // the real-data form at N = 32 also times the three-CTA pair kernel, k_pair3 (C = 8)
     const int pair3_c = (pl.real && pl.N == 32 && ctas != 2) ? nc : -1;

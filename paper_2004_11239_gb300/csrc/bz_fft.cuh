@@ -103,65 +103,8 @@ constexpr TwTable make_tw_table() {
     return t;
 }
 
-// Double-float numbers: an unevaluated sum hi + lo of two floats with |lo| <= ulp(hi)/2
-// (Dekker 1971; Knuth's TwoSum, FMA-based TwoProduct).  About 48 significant bits on the
-// FP32 pipes.  _rn intrinsics keep the compiler from contracting the error-free steps.
-struct ff { float hi, lo; };
-struct cff { ff x, y; };
-
-struct TwTableFF { cff v[kTwTotal]; };
-
-constexpr TwTableFF make_tw_table_ff() {
-    TwTableFF t{};
-    const int lens[12] = {8, 16, 24, 32, 48, 64, 12, 6, 4, 3, 2, 1};
-    const int offs[12] = {0, 8, 24, 48, 80, 128, 192, 204, 210, 214, 217, 219};
-    for (int a = 0; a < 12; ++a) {
-        int N = lens[a];
-        for (int j = 0; j < N; ++j) {
-            TwCS cs = unit_root(j * (192 / N), 192);
-            float ch = (float)cs.c, sh = (float)cs.s;
-            t.v[offs[a] + j].x.hi = ch;
-            t.v[offs[a] + j].x.lo = (float)(cs.c - (double)ch);
-            t.v[offs[a] + j].y.hi = sh;
-            t.v[offs[a] + j].y.lo = (float)(cs.s - (double)sh);
-        }
-    }
-    return t;
-}
-
 static __constant__ TwTable c_tw = make_tw_table();
 static __constant__ TwTableD c_twd = make_tw_table_d();
-static __constant__ TwTableFF c_twff = make_tw_table_ff();
-
-__device__ __forceinline__ ff ff_two_sum(float a, float b) {
-    float s = __fadd_rn(a, b);
-    float bb = __fsub_rn(s, a);
-    float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-    return {s, e};
-}
-__device__ __forceinline__ ff ff_fast_two_sum(float a, float b) {   // |a| >= |b|
-    float s = __fadd_rn(a, b);
-    return {s, __fsub_rn(b, __fsub_rn(s, a))};
-}
-__device__ __forceinline__ ff ff_add(ff a, ff b) {
-    ff s = ff_two_sum(a.hi, b.hi);
-    ff t = ff_two_sum(a.lo, b.lo);
-    s.lo = __fadd_rn(s.lo, t.hi);
-    s = ff_fast_two_sum(s.hi, s.lo);
-    s.lo = __fadd_rn(s.lo, t.lo);
-    return ff_fast_two_sum(s.hi, s.lo);
-}
-__device__ __forceinline__ ff ff_mul(ff a, ff b) {
-    float p = __fmul_rn(a.hi, b.hi);
-    float e = __fmaf_rn(a.hi, b.hi, -p);
-    e = __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, e));
-    return ff_fast_two_sum(p, e);
-}
-__device__ __forceinline__ ff ff_neg(ff a) { return {-a.hi, -a.lo}; }
-__device__ __forceinline__ ff ff_from(double d) {
-    float h = (float)d;
-    return {h, (float)(d - (double)h)};
-}
 
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
@@ -177,16 +120,10 @@ __device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2
 __device__ __forceinline__ double2 cscale(double2 a, double s) { return make_double2(s * a.x, s * a.y); }
 __device__ __forceinline__ float2 cneg(float2 a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ double2 cneg(double2 a) { return make_double2(-a.x, -a.y); }
-__device__ __forceinline__ cff cadd(cff a, cff b) { return {ff_add(a.x, b.x), ff_add(a.y, b.y)}; }
-__device__ __forceinline__ cff csub(cff a, cff b) { return {ff_add(a.x, ff_neg(b.x)), ff_add(a.y, ff_neg(b.y))}; }
-__device__ __forceinline__ cff cmul(cff a, cff b) {
-    return {ff_add(ff_mul(a.x, b.x), ff_neg(ff_mul(a.y, b.y))), ff_add(ff_mul(a.x, b.y), ff_mul(a.y, b.x))};
-}
-__device__ __forceinline__ cff cscale(cff a, ff s) { return {ff_mul(a.x, s), ff_mul(a.y, s)}; }
-__device__ __forceinline__ cff cneg(cff a) { return {ff_neg(a.x), ff_neg(a.y)}; }
-__device__ __forceinline__ ff neg_of(ff a) { return ff_neg(a); }
 __device__ __forceinline__ float neg_of(float a) { return -a; }
 __device__ __forceinline__ double neg_of(double a) { return -a; }
+__device__ __forceinline__ float fma_of(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_of(double a, double b, double c) { return fma(a, b, c); }
 // multiply by SIGN * i
 template <int SIGN, class T> __device__ __forceinline__ T mul_i(T a) {
     T r;
@@ -197,12 +134,10 @@ template <int SIGN, class T> __device__ __forceinline__ T mul_i(T a) {
 
 __device__ __forceinline__ float2 tw_entry(const float2 *, int i) { return c_tw.v[i]; }
 __device__ __forceinline__ double2 tw_entry(const double2 *, int i) { return c_twd.v[i]; }
-__device__ __forceinline__ cff tw_entry(const cff *, int i) { return c_twff.v[i]; }
 
 // real constants in the element precision
 __device__ __forceinline__ float real_const(const float2 *, double c) { return (float)c; }
 __device__ __forceinline__ double real_const(const double2 *, double c) { return c; }
-__device__ __forceinline__ ff real_const(const cff *, double c) { return ff_from(c); }
 
 template <int N, int SIGN, class T> __device__ __forceinline__ void mul_tw(T &v, int j) {
     // j is a compile-time constant after unrolling; trivial roots skip the multiply
@@ -281,6 +216,57 @@ template <int N, int SIGN, class T> __device__ __forceinline__ void fft_inplace(
     for (int k = 0; k < N; ++k) y[k] = x[slot_of<N>(k)];
     #pragma unroll
     for (int k = 0; k < N; ++k) x[k] = y[k];
+}
+
+// The same transform by decimation in time.  Fewer operations, but a longer chain from input to output
+// and more live registers: faster in the cluster kernels, which have registers to spare (k_fused at
+// N = 32 302 -> 290 us, N = 24 34.6 -> 33.6, N = 16 in batches 1960 -> 1918), slower in k_col32
+// (92 -> 95) and in the planes of bz_lines.cu (29 -> 44), which spill.
+// Input order of the recursion: slot i of the working array holds x[dit_source<N>(i)].
+template <int N> __host__ __device__ constexpr int dit_source(int i) {
+    if constexpr (N % 2 != 0) return i;
+    else return i < N / 2 ? 2 * dit_source<N / 2>(i) : 2 * dit_source<N / 2>(i - N / 2) + 1;
+}
+
+// b <- a - w b, a <- a + w b, w = exp(SIGN 2 pi i k / N): the sum by two fused multiply-adds a
+// component and the difference as 2 a - sum, six operations against eight for a product and two
+// additions.  (A 32-point line takes 388 FP32 operations this way; 432 by fft_inplace.)
+template <int N, int SIGN, class T> __device__ __forceinline__ void bfly_tw(T &a, T &b, int k) {
+    if (k == 0) { bfly2<SIGN>(a, b); return; }
+    if (4 * k == N) {
+        b = mul_i<SIGN>(b);
+        bfly2<SIGN>(a, b);
+        return;
+    }
+    const T w = tw_entry((const T *)nullptr, tw_off<N>() + k);
+    const auto wi = SIGN < 0 ? neg_of(w.y) : w.y;
+    T u;
+    u.x = fma_of(w.x, b.x, fma_of(-wi, b.y, a.x));
+    u.y = fma_of(w.x, b.y, fma_of(wi, b.x, a.y));
+    b.x = fma_of(a.x, 2, -u.x);
+    b.y = fma_of(a.y, 2, -u.y);
+    a = u;
+}
+
+// In-place decimation in time on x[0 .. N), inputs in dit_source order, outputs in natural order.
+template <int N, int SIGN, class T> __device__ __forceinline__ void dit(T *x) {
+    if constexpr (N == 3) {
+        bfly3<SIGN>(x[0], x[1], x[2]);
+    } else if constexpr (N > 1) {
+        dit<N / 2, SIGN>(x);
+        dit<N / 2, SIGN>(x + N / 2);
+        #pragma unroll
+        for (int k = 0; k < N / 2; ++k) bfly_tw<N, SIGN>(x[k], x[k + N / 2], k);
+    }
+}
+
+template <int N, int SIGN, class T> __device__ __forceinline__ void fft_dit(T (&x)[N]) {
+    T y[N];
+    #pragma unroll
+    for (int i = 0; i < N; ++i) y[i] = x[dit_source<N>(i)];
+    dit<N, SIGN>(y);
+    #pragma unroll
+    for (int i = 0; i < N; ++i) x[i] = y[i];
 }
 
 }  // namespace bz

@@ -102,11 +102,14 @@ template <int N, int C> static cudaError_t setup_nc(int *G, bool real) {
     return occupancy<N, C, false>(G);
 }
 
-// Cluster sizes compiled for each N (the plan times them and keeps the fastest).
-int fused_candidates(int N, int *cs) {
+// Cluster sizes compiled for each N (the plan times them and keeps the fastest).  N = 16 takes
+// one CTA unless two are asked for: a single collide takes the same time with either (8.6 us at
+// P = 192), which left the choice to chance, and batches run on the plan's size (32 instances of
+// P = 192: 108 us with one, 154 with two).
+int fused_candidates(int N, int *cs, int forced) {
     switch (N) {
         case 8: cs[0] = 1; return 1;
-        case 16: cs[0] = 1; cs[1] = 2; return 2;
+        case 16: cs[0] = forced == 2 ? 2 : 1; return 1;
         case 24: cs[0] = 2; cs[1] = 3; return 2;
         case 32: cs[0] = 4; cs[1] = 8; return 2;
     }

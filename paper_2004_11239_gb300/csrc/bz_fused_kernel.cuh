@@ -64,13 +64,13 @@ __device__ __forceinline__ void phase_a(const float2 *__restrict__ fin, const fl
         #pragma unroll
         for (int i = 0; i < N; ++i) x[i] = f[i * N + lane];
     }
-    fft_inplace<N, +1>(x);                                    // k2 -> j2
+    fft_dit<N, +1>(x);                                    // k2 -> j2
     #pragma unroll
     for (int i = 0; i < N; ++i) my[i * LD + lane] = x[i];
     __syncthreads();
     #pragma unroll
     for (int j = 0; j < N; ++j) x[j] = my[lane * LD + j];
-    fft_inplace<N, +1>(x);                                    // k3 -> j3 (row j2 = lane)
+    fft_dit<N, +1>(x);                                    // k3 -> j3 (row j2 = lane)
     #pragma unroll
     for (int j = 0; j < N; ++j) my[lane * LD + j] = x[j];
 }
@@ -90,13 +90,13 @@ __device__ __forceinline__ void phase_a_pair(const float2 *__restrict__ fin, con
         const float2 u = cmul(ta, tws[N + i]), v = cmul(tb, tws[4 * N + i]);
         x[i] = cmul(f[i * N + lane], make_float2(u.x - v.y, u.y + v.x));       // u + i v
     }
-    fft_inplace<N, +1>(x);                                    // k2 -> j2
+    fft_dit<N, +1>(x);                                    // k2 -> j2
     #pragma unroll
     for (int i = 0; i < N; ++i) my[i * LD + lane] = x[i];
     __syncthreads();
     #pragma unroll
     for (int j = 0; j < N; ++j) x[j] = my[lane * LD + j];
-    fft_inplace<N, +1>(x);                                    // k3 -> j3 (row j2 = lane)
+    fft_dit<N, +1>(x);                                    // k3 -> j3 (row j2 = lane)
     #pragma unroll
     for (int j = 0; j < N; ++j) my[lane * LD + j] = x[j];
 }
@@ -175,7 +175,7 @@ k_fused(ItemArgs a) {
             float2 x[N];
             #pragma unroll
             for (int k = 0; k < N; ++k) x[k] = ld_dsmem(pen[k / PPC] + (uint32_t)(k % PPC) * PLANE_BYTES);
-            fft_inplace<N, +1>(x);                            // k1 -> j1
+            fft_dit<N, +1>(x);                            // k1 -> j1
             #pragma unroll
             for (int j = 0; j < N; ++j) {
                 if constexpr (REAL) shr[((size_t)pid * N + j) * N + lane] = x[j].x;
@@ -229,7 +229,7 @@ k_fused(ItemArgs a) {
             float2 x[N];
             #pragma unroll
             for (int k = 0; k < N; ++k) x[k] = ld_dsmem(pen[k / PPC] + (uint32_t)(k % PPC) * PLANE_BYTES);
-            fft_inplace<N, +1>(x);                            // k1 -> j1
+            fft_dit<N, +1>(x);                            // k1 -> j1
             if constexpr (REAL) {
                 #pragma unroll
                 for (int j = 0; j < N; ++j) {                 // h is real
@@ -241,21 +241,21 @@ k_fused(ItemArgs a) {
                 #pragma unroll
                 for (int j = 0; j < N; ++j) x[j] = cmul(x[j], shs[((size_t)pid * N + j) * N + lane]);
             }
-            fft_inplace<N, -1>(x);                            // j1 -> k1
+            fft_dit<N, -1>(x);                            // j1 -> k1
             #pragma unroll
             for (int k = 0; k < N; ++k) st_dsmem(pen[k / PPC] + (uint32_t)(k % PPC) * PLANE_BYTES, x[k]);
             cluster_barrier<C>();
             // C: rows over j3, then column k3 = lane over j2, times alpha, accumulate
             #pragma unroll
             for (int j = 0; j < N; ++j) x[j] = my[lane * LD + j];
-            fft_inplace<N, -1>(x);                            // j3 -> k3 (row j2 = lane)
+            fft_dit<N, -1>(x);                            // j3 -> k3 (row j2 = lane)
             #pragma unroll
             for (int j = 0; j < N; ++j) my[lane * LD + j] = x[j];
             cp_async_wait_1();                                // alpha tile (the next twiddles may pend)
             __syncthreads();
             #pragma unroll
             for (int i = 0; i < N; ++i) x[i] = my[i * LD + lane];
-            fft_inplace<N, -1>(x);                            // j2 -> k2
+            fft_dit<N, -1>(x);                            // j2 -> k2
             #pragma unroll
             for (int i = 0; i < N; ++i) {
                 float2 al = sal[((size_t)pid * N + i) * N + lane];

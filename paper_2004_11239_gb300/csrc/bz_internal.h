@@ -177,7 +177,7 @@ struct ItemArgs {
     const float2 *cpair = nullptr;   // BZ_DATA_REAL: [pairs][3][N][N] Nyquist-plane table C
     float2 *part_s = nullptr;        // BZ_DATA_REAL: [slots][nblk][3][N][N] per-item sums X
 };
-int fused_candidates(int N, int *cs);
+int fused_candidates(int N, int *cs, int forced);
 cudaError_t fused_setup(int N, int C, int *G, bool real);
 bz_status launch_fused(const Plan &pl, const ItemArgs &a, cudaStream_t st);
 // bz_hff.cu: h[slot] = IFFT(f[slot]) in double-float arithmetic (about 47 bits), stored FP32, for the
