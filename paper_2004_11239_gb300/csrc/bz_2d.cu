@@ -85,24 +85,22 @@ template <int N> cudaError_t setup_n(Plan &pl) {
     return pl.fused_G > 0 ? cudaSuccess : cudaErrorInvalidConfiguration;
 }
 
-template <int N> bz_status run_n(Plan &pl, int p0, int p1, cudaStream_t st, int *launches) {
+template <int N> bz_status run_n(Plan &pl, int p0, int p1, cudaStream_t st, int *launches, const Sink &sink) {
     const int n2 = N * N;
     const int nt = p1 - p0;
     const int TB = nt > 0 ? (nt + pl.fused_G - 1) / pl.fused_G : 1;
     const int nblk = nt > 0 ? (nt + TB - 1) / TB : 0;
-    const void *src = pl.src ? pl.src : (const void *)pl.fin;
-    const int sdt = pl.src ? pl.src_dtype : BZ_C64;
     tm_begin(pl, st);
-    const bz_status hs = hff_launch_2d(N, src, sdt, pl.h, st);
+    const bz_status hs = hff_launch_2d(N, pl.src, pl.src_dtype, pl.h, pl.fcopy, st);
     if (hs != BZ_OK) return hs;
     tm_end(pl, st, TK_OTHER);
     tm_begin(pl, st);
     if (nblk > 0)
         k_collide_2d<N><<<nblk < pl.fused_G ? nblk : pl.fused_G, N, D2<N>::SMEM, st>>>(
-            pl.fin, pl.h, pl.tw, pl.alpha, pl.part, p0, p1, TB, nblk);
+            pl.f32, pl.h, pl.tw, pl.alpha, pl.part, p0, p1, TB, nblk);
     tm_end(pl, st, TK_FUSED);
     tm_begin(pl, st);
-    reduce_parts(pl.part, nblk, n2, pl.acc, st);
+    reduce_parts(pl.part, nblk, n2, sink, st);
     tm_end(pl, st, TK_REDUCE);
     BZ_CUDA_TRY(cudaGetLastError());
     if (launches) *launches += nblk > 0 ? 3 : 2;
@@ -121,12 +119,12 @@ cudaError_t setup_2d(Plan &pl) {
     return cudaErrorInvalidValue;
 }
 
-bz_status collide_2d(Plan &pl, int p0, int p1, cudaStream_t st, int *launches) {
+bz_status collide_2d(Plan &pl, int p0, int p1, cudaStream_t st, int *launches, const Sink &sink) {
     switch (pl.N) {
-        case 8: return run_n<8>(pl, p0, p1, st, launches);
-        case 16: return run_n<16>(pl, p0, p1, st, launches);
-        case 32: return run_n<32>(pl, p0, p1, st, launches);
-        case 64: return run_n<64>(pl, p0, p1, st, launches);
+        case 8: return run_n<8>(pl, p0, p1, st, launches, sink);
+        case 16: return run_n<16>(pl, p0, p1, st, launches, sink);
+        case 32: return run_n<32>(pl, p0, p1, st, launches, sink);
+        case 64: return run_n<64>(pl, p0, p1, st, launches, sink);
     }
     return BZ_ERR_UNSUPPORTED;
 }

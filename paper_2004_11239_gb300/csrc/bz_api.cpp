@@ -85,13 +85,16 @@ bz_status setup_col32(bz::Plan &pl) {
     if (dmalloc(&pl.part, part) != BZ_OK) return BZ_ERR_OOM;
     pl.use_fused = 1; pl.fused_C = 1; pl.fused_G = G;
     pl.ws_bytes += part;
+    pl.f32 = pl.fin;
+    pl.src = pl.fin;
+    pl.src_dtype = BZ_C64;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     bz_status s = cudaMemset(pl.fin, 0, (size_t)pl.N * pl.N * pl.N * sizeof(float2)) == cudaSuccess ? BZ_OK : BZ_ERR_CUDA;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) s = BZ_ERR_CUDA;
-    if (s == BZ_OK) s = bz::collide_fused(pl, 0, pl.P, nullptr, nullptr);     // warm-up
+    if (s == BZ_OK) s = bz::collide_fused(pl, 0, pl.P, nullptr, nullptr, bz::acc_sink(pl));     // warm-up
     if (s == BZ_OK) {
         cudaEventRecord(e0);
-        s = bz::collide_fused(pl, 0, pl.P, nullptr, nullptr);
+        s = bz::collide_fused(pl, 0, pl.P, nullptr, nullptr, bz::acc_sink(pl));
         cudaEventRecord(e1);
         if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&pl.fused_ms, e0, e1) != cudaSuccess)
             s = BZ_ERR_CUDA;
@@ -118,6 +121,9 @@ bz_status select_fused(bz::Plan &pl, int forced, int ctas) {
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return BZ_ERR_CUDA;
     if (cudaMemset(pl.fin, 0, field) != cudaSuccess) return BZ_ERR_CUDA;
+    pl.f32 = pl.fin;
+    pl.src = pl.fin;
+    pl.src_dtype = BZ_C64;
     for (int c = 0; c < nc; ++c) {
         if (forced > 0 && cs[c] != forced) continue;
         if (ctas == 3 && c != pair3_c) continue;
@@ -136,9 +142,9 @@ bz_status select_fused(bz::Plan &pl, int forced, int ctas) {
         std::swap(parts, pl.part_s);
         pl.use_fused = 1; pl.fused_C = cs[c]; pl.fused_G = G; pl.pair3 = c == pair3_c;
         float ms = 1e30f;
-        if (bz::collide_fused(pl, 0, pl.P, nullptr, nullptr) == BZ_OK) {      // warm-up
+        if (bz::collide_fused(pl, 0, pl.P, nullptr, nullptr, bz::acc_sink(pl)) == BZ_OK) {      // warm-up
             cudaEventRecord(e0);
-            bz::collide_fused(pl, 0, pl.P, nullptr, nullptr);
+            bz::collide_fused(pl, 0, pl.P, nullptr, nullptr, bz::acc_sink(pl));
             cudaEventRecord(e1);
             if (cudaEventSynchronize(e1) == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
         }
@@ -427,8 +433,7 @@ bz_status bz_collide_terms(bz_plan *plan, int p0, int p1, const void *fhat, void
     if (dtype != BZ_C64 && dtype != BZ_C128) return BZ_ERR_ARG;
     cudaStream_t st = (cudaStream_t)stream;
     int nl = 0;
-    bz_status s = bz::collide_range(pl, p0, p1, fhat, dtype, st, &nl);
-    if (s == BZ_OK) s = bz::write_output(pl, Qhat, dtype, st, &nl);
+    const bz_status s = bz::collide_range(pl, p0, p1, fhat, Qhat, dtype, st, &nl);
     pl.last_launches = nl;
     return s;
 }

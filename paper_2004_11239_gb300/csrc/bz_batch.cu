@@ -450,11 +450,10 @@ bz_status chunked_collide(bz_batch &B, int count, const int *slots, const void *
     int nl = 0;
     for (int b = 0; b < count && s == BZ_OK; ++b) {
         pl.gsc_cur = B.gsc + (size_t)slots[b] * pl.N_rho;
-        s = collide_range(pl, 0, pl.P, (const char *)fhat + slots[b] * bytes, dtype, st, &nl);
-        if (s == BZ_OK) s = write_output(pl, (char *)Qhat + slots[b] * bytes, dtype, st, &nl);
+        s = collide_range(pl, 0, pl.P, (const char *)fhat + slots[b] * bytes, (char *)Qhat + slots[b] * bytes, dtype, st,
+                          &nl);
     }
     pl.gsc_cur = nullptr;
-    pl.src = nullptr;
     B.last_launches = nl;
     return s;
 }
@@ -475,7 +474,6 @@ bz_status slot_graph(bz_batch &B, int slot, void *fhat_slot, int dtype, double d
     int nl = 0;
     const bz_status cs = rk4_steps(pl, fhat_slot, dtype, dt, 1, B.cap_stream, &nl);
     pl.gsc_cur = nullptr;
-    pl.src = nullptr;
     const cudaError_t ce = cudaStreamEndCapture(B.cap_stream, &g);
     if (cs != BZ_OK || ce != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
@@ -506,8 +504,7 @@ bz_status chunked_step_rk(bz_batch &B, int count, const int *slots, void *fhat, 
             s = rk4_steps(pl, (char *)fhat + slots[b] * bytes, dtype, dt, nsteps, st, &nl);
         }
         pl.gsc_cur = nullptr;
-        pl.src = nullptr;
-        B.last_launches = nl;
+            B.last_launches = nl;
         return s;
     }
     for (int b = 0; b < count && s == BZ_OK; ++b) {

@@ -349,9 +349,9 @@ __device__ __forceinline__ void col_modes(int e, int &i, int &j) {
     }
 }
 
-// acc = the sum over the G items on the full grid: block of 32 elements x 8 slices, slice s adds
+// sink = the sum over the G items on the full grid: block of 32 elements x 8 slices, slice s adds
 // items s, s + 8, ..., then the slices in order (compensated).
-__global__ void __launch_bounds__(256) k_reduce_col(const float2 *__restrict__ part, int G, double2 *__restrict__ acc) {
+__global__ void __launch_bounds__(256) k_reduce_col(const float2 *__restrict__ part, int G, Sink sink) {
     __shared__ float4 red[8][32];
     const int kk = threadIdx.x % 32, sl = threadIdx.x / 32;
     const int e = blockIdx.x * 32 + kk;
@@ -374,8 +374,8 @@ __global__ void __launch_bounds__(256) k_reduce_col(const float2 *__restrict__ p
     const double2 v = make_double2((double)t.sr - (double)t.cr, (double)t.si - (double)t.ci);
     int i, j;
     col_modes(e, i, j);
-    if (i >= 0) acc[i] = v;
-    if (j >= 0) acc[j] = make_double2(v.x, -v.y);
+    if (i >= 0) sink_put(sink, i, v);
+    if (j >= 0) sink_put(sink, j, make_double2(v.x, -v.y));
 }
 
 }  // namespace
@@ -412,8 +412,8 @@ bz_status col32_inputs(Plan &pl, cudaStream_t st) {
     return BZ_OK;
 }
 
-bz_status reduce_col(Plan &pl, int nblk, cudaStream_t st) {
-    k_reduce_col<<<18 * C2 / 32, 256, 0, st>>>(pl.part, nblk, pl.acc);
+bz_status reduce_col(Plan &pl, int nblk, cudaStream_t st, const Sink &sink) {
+    k_reduce_col<<<18 * C2 / 32, 256, 0, st>>>(pl.part, nblk, sink);
     BZ_CUDA_TRY(cudaGetLastError());
     return BZ_OK;
 }

@@ -264,19 +264,10 @@ __global__ void k_acc_add(double2 *__restrict__ a, const double2 *__restrict__ b
     }
 }
 
-// The plan's result to the caller's array in its dtype, raising the non-finite flag.
-__global__ void k_acc_out(const double2 *__restrict__ in, void *__restrict__ out, int dtype, int n, int *flag) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const double2 v = in[i];
-    if (dtype == BZ_C128) {
-        ((double2 *)out)[i] = v;
-        note_finite(v, flag);
-    } else {
-        const float2 w = make_float2((float)v.x, (float)v.y);
-        ((float2 *)out)[i] = w;
-        note_finite(w, flag);
-    }
+// The plan's accumulator to the sink.
+__global__ void k_acc_sink(const double2 *__restrict__ acc, int n, Sink sink) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) sink_put(sink, i, acc[i]);
 }
 
 // Padded plans (BZ_CONV_PADDED): the caller's Nin-grid lives inside the N = 2 Nin grid at the
@@ -405,13 +396,13 @@ static void pencil(float2 *S, const float2 *h, float2 *out, int T, cudaStream_t 
 // chunks run over term pairs [p0 / 2, p1 / 2) with the pair table A, the Nyquist sums X are
 // reduced beside V, and Q is symmetrised after the last chunk.
 template <int N>
-static bz_status run_chunks_real(Plan &pl, int p0, int p1, cudaStream_t st, int *launches) {
+static bz_status run_chunks_real(Plan &pl, int p0, int p1, cudaStream_t st, int *launches, const Sink &sink) {
     const int n3 = N * N * N, ns = 3 * N * N;
     if ((p0 | p1) & 1) return BZ_ERR_ARG;
     const int u0 = p0 / 2, u1 = p1 / 2;
     const int chunk = pl.chunk;
     tm_begin(pl, st);
-    bz_status s = sym_input(pl, pl.src ? pl.src : (const void *)pl.fin, pl.src ? pl.src_dtype : BZ_C64, st);
+    bz_status s = sym_input(pl, pl.src, pl.src_dtype, st);
     if (s != BZ_OK) return s;
     plane_inv<N, false>(pl.fsym, pl.tw, pl.S, 0, 1, 0, st);
     pencil<N, 0>(pl.S, nullptr, pl.h, 1, st);
@@ -465,7 +456,7 @@ static bz_status run_chunks_real(Plan &pl, int p0, int p1, cudaStream_t st, int 
         nl += 2;
     }
     tm_begin(pl, st);
-    s = sym_output(pl, st);
+    s = sym_output(pl, st, sink);
     if (s != BZ_OK) return s;
     tm_end(pl, st, TK_OTHER);
     ++nl;
@@ -475,12 +466,12 @@ static bz_status run_chunks_real(Plan &pl, int p0, int p1, cudaStream_t st, int 
 }
 
 template <int N>
-static bz_status run_chunks(Plan &pl, int p0, int p1, cudaStream_t st, int *launches) {
+static bz_status run_chunks(Plan &pl, int p0, int p1, cudaStream_t st, int *launches, const Sink &sink) {
     const int n3 = N * N * N;
-    if (pl.real) return run_chunks_real<N>(pl, p0, p1, st, launches);
+    if (pl.real) return run_chunks_real<N>(pl, p0, p1, st, launches, sink);
     // h = IFFT(fhat): planes without twiddles into S[0], then an inverse-only pencil pass
     tm_begin(pl, st);
-    plane_inv<N, false>(pl.fin, pl.tw, pl.S, 0, 1, 0, st);
+    plane_inv<N, false>(pl.f32, pl.tw, pl.S, 0, 1, 0, st);
     pencil<N, 0>(pl.S, nullptr, pl.h, 1, st);
     BZ_CUDA_TRY(cudaMemsetAsync(pl.acc, 0, (size_t)n3 * sizeof(double2), st));
     tm_end(pl, st, TK_OTHER);
@@ -501,7 +492,7 @@ static bz_status run_chunks(Plan &pl, int p0, int p1, cudaStream_t st, int *laun
         float2 *S = ln ? pl.xS[ln - 1] : pl.S;
         double2 *acc = ln ? pl.xacc[ln - 1] : pl.acc;
         tm_begin(pl, cs);
-        plane_inv<N, false>(pl.fin, pl.tw, S, c0, T, 1, cs);
+        plane_inv<N, false>(pl.f32, pl.tw, S, c0, T, 1, cs);
         tm_end(pl, cs, TK_PLANE_INV);
         tm_begin(pl, cs);
         pencil<N, 1>(S, pl.h, nullptr, T, cs);
@@ -522,6 +513,10 @@ static bz_status run_chunks(Plan &pl, int p0, int p1, cudaStream_t st, int *laun
         BZ_CUDA_TRY(cudaEventRecord(pl.xev_join[e], pl.xst[e]));
         BZ_CUDA_TRY(cudaStreamWaitEvent(st, pl.xev_join[e], 0));
         k_acc_add<<<(n3 + 255) / 256, 256, 0, st>>>(pl.acc, pl.xacc[e], n3);
+        ++nl;
+    }
+    if (sink.mode != Sink::ACC) {
+        k_acc_sink<<<(n3 + 255) / 256, 256, 0, st>>>(pl.acc, n3, sink);
         ++nl;
     }
     BZ_CUDA_TRY(cudaGetLastError());
@@ -545,9 +540,13 @@ bz_status h_fp32(Plan &pl, const float2 *fin, cudaStream_t st) {
     return BZ_OK;
 }
 
-bz_status load_input(Plan &pl, const void *fhat, int dtype, cudaStream_t st, int *launches) {
+// The input of a collide: pl.src (what h is formed from) and pl.f32 (what the terms transform).  Real
+// data is symmetrised from the caller's array; complex64 data is read where it is; complex128 data is
+// rounded to pl.fin by the h pass where there is one in front of the terms, else by a pass of its own.
+static bz_status load_input(Plan &pl, const void *fhat, int dtype, cudaStream_t st, int *launches) {
     const int n3 = (int)modes(pl);
-    if (dtype != BZ_C64 && dtype != BZ_C128) return BZ_ERR_ARG;
+    pl.f32 = pl.fin;
+    pl.fcopy = nullptr;
     if (pl.Nin) {
         // padded: embed into the 2N grid, in FP32 and (where the h pass reads it) FP64
         k_embed<<<(n3 + 255) / 256, 256, 0, st>>>(fhat, dtype, pl.Nin, pl.N, pl.fin, pl.fin64);
@@ -557,54 +556,54 @@ bz_status load_input(Plan &pl, const void *fhat, int dtype, cudaStream_t st, int
         if (launches) *launches += 1;
         return BZ_OK;
     }
-    pl.src = fhat;                 // the fused path forms h from the caller's array in FP64
+    pl.src = fhat;
     pl.src_dtype = dtype;
+    if (pl.real) return BZ_OK;
     if (dtype == BZ_C64) {
-        BZ_CUDA_TRY(cudaMemcpyAsync(pl.fin, fhat, (size_t)n3 * sizeof(float2), cudaMemcpyDeviceToDevice, st));
-    } else if (dtype == BZ_C128) {
+        pl.f32 = (const float2 *)fhat;
+    } else if (pl.dim == 2 || (pl.use_fused && (pl.h_fp64 || pl.precision == BZ_PREC_BF16X3))) {
+        pl.fcopy = pl.fin;
+    } else {
         k_c128_to_c64<<<(n3 + 255) / 256, 256, 0, st>>>((const double2 *)fhat, pl.fin, n3);
         BZ_CUDA_TRY(cudaGetLastError());
         if (launches) *launches += 1;
-    } else {
-        return BZ_ERR_ARG;
     }
     return BZ_OK;
 }
 
-// Q over terms [p0, p1) of the FP32 input already in pl.fin; result in pl.acc (FP64).
-bz_status collide_core(Plan &pl, int p0, int p1, cudaStream_t st, int *launches) {
-    if (pl.dim == 2) return collide_2d(pl, p0, p1, st, launches);
-    if (pl.use_fused) return collide_fused(pl, p0, p1, st, launches);
+// Q over terms [p0, p1) of the input in pl.f32 and pl.src.
+bz_status collide_core(Plan &pl, int p0, int p1, cudaStream_t st, int *launches, const Sink &sink) {
+    if (pl.dim == 2) return collide_2d(pl, p0, p1, st, launches, sink);
+    if (pl.use_fused) return collide_fused(pl, p0, p1, st, launches, sink);
     switch (pl.N) {
-        case 8: return run_chunks<8>(pl, p0, p1, st, launches);
-        case 16: return run_chunks<16>(pl, p0, p1, st, launches);
-        case 24: return run_chunks<24>(pl, p0, p1, st, launches);
-        case 32: return run_chunks<32>(pl, p0, p1, st, launches);
+        case 8: return run_chunks<8>(pl, p0, p1, st, launches, sink);
+        case 16: return run_chunks<16>(pl, p0, p1, st, launches, sink);
+        case 24: return run_chunks<24>(pl, p0, p1, st, launches, sink);
+        case 32: return run_chunks<32>(pl, p0, p1, st, launches, sink);
         case 48:
-        case 64: return collide_lines(pl, p0, p1, st, launches);
+        case 64: return collide_lines(pl, p0, p1, st, launches, sink);
     }
     return BZ_ERR_ARG;
 }
 
-bz_status collide_range(Plan &pl, int p0, int p1, const void *fhat, int in_dtype, cudaStream_t st,
+bz_status collide_range(Plan &pl, int p0, int p1, const void *fhat, void *Qhat, int dtype, cudaStream_t st,
                         int *launches) {
-    bz_status s = load_input(pl, fhat, in_dtype, st, launches);
-    if (s != BZ_OK) return s;
-    return collide_core(pl, p0, p1, st, launches);
-}
-
-bz_status write_output(Plan &pl, void *Qhat, int dtype, cudaStream_t st, int *launches) {
-    const int n3 = (int)modes(pl);
-    if (pl.Nin) {
-        if (dtype != BZ_C64 && dtype != BZ_C128) return BZ_ERR_ARG;
-        const int m3 = pl.Nin * pl.Nin * pl.Nin;
-        k_extract<<<(m3 + 255) / 256, 256, 0, st>>>(pl.acc, pl.Nin, pl.N, Qhat, dtype, nonfinite_flag(pl));
-        BZ_CUDA_TRY(cudaGetLastError());
-        if (launches) *launches += 1;
-        return BZ_OK;
-    }
     if (dtype != BZ_C64 && dtype != BZ_C128) return BZ_ERR_ARG;
-    k_acc_out<<<(n3 + 255) / 256, 256, 0, st>>>(pl.acc, Qhat, dtype, n3, nonfinite_flag(pl));
+    bz_status s = load_input(pl, fhat, dtype, st, launches);
+    Sink sink = acc_sink(pl);
+    if (!pl.Nin) {
+        sink.mode = Sink::OUT;
+        sink.out = Qhat;
+        sink.dtype = dtype;
+        sink.flag = nonfinite_flag(pl);
+    }
+    if (s == BZ_OK) s = collide_core(pl, p0, p1, st, launches, sink);
+    pl.src = nullptr;                                     // no pointer of the caller's outlives the call
+    pl.f32 = pl.fin;
+    pl.fcopy = nullptr;
+    if (s != BZ_OK || !pl.Nin) return s;
+    const int m3 = pl.Nin * pl.Nin * pl.Nin;
+    k_extract<<<(m3 + 255) / 256, 256, 0, st>>>(pl.acc, pl.Nin, pl.N, Qhat, dtype, nonfinite_flag(pl));
     BZ_CUDA_TRY(cudaGetLastError());
     if (launches) *launches += 1;
     return BZ_OK;

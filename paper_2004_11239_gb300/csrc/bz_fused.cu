@@ -5,7 +5,7 @@
 
 namespace bz {
 
-// acc[k] = sum over g of part[g][k] with a fixed shape: thread (kk, s) of a 32 x 8 block sums
+// sink(k) = sum over g of part[g][k] with a fixed shape: thread (kk, s) of a 32 x 8 block sums
 // g = s, s + 8, ... for mode k = 32 blockIdx.x + kk with Kahan compensation in FP32, then the
 // eight slices are added in order s = 0..7 (compensated).  FP32 pipes only.
 struct Kahan2 {
@@ -20,8 +20,7 @@ struct Kahan2 {
     }
 };
 
-__global__ void __launch_bounds__(256) k_reduce_parts(const float2 *__restrict__ part, int G, int n3,
-                                                     double2 *__restrict__ acc) {
+__global__ void __launch_bounds__(256) k_reduce_parts(const float2 *__restrict__ part, int G, int n3, Sink sink) {
     __shared__ float4 red[8][32];
     const int kk = threadIdx.x % 32, sl = threadIdx.x / 32;
     const int k = blockIdx.x * 32 + kk;
@@ -42,7 +41,7 @@ __global__ void __launch_bounds__(256) k_reduce_parts(const float2 *__restrict__
             t.add(q.x, q.y);
             t.add(-q.z, -q.w);
         }
-        acc[k] = make_double2((double)t.sr - (double)t.cr, (double)t.si - (double)t.ci);
+        sink_put(sink, k, make_double2((double)t.sr - (double)t.cr, (double)t.si - (double)t.ci));
     }
 }
 
@@ -177,22 +176,20 @@ bz_status launch_fused(const Plan &pl, const ItemArgs &a, cudaStream_t st) {
     return BZ_ERR_UNSUPPORTED;
 }
 
-// acc[k] = sum over the nblk item partials of part (fixed order, compensated).
-void reduce_parts(const float2 *part, int nblk, int n, double2 *acc, cudaStream_t st) {
-    k_reduce_parts<<<(n + 31) / 32, 256, 0, st>>>(part, nblk, n, acc);
+// sink(k) = sum over the nblk item partials of part (fixed order, compensated).
+void reduce_parts(const float2 *part, int nblk, int n, const Sink &sink, cudaStream_t st) {
+    k_reduce_parts<<<(n + 31) / 32, 256, 0, st>>>(part, nblk, n, sink);
 }
 
-// One instance (pl.fin), terms [p0, p1): one block of terms per resident cluster, then the
-// fixed-order FP64 sum of the blocks into pl.acc.  BZ_DATA_REAL: the input is first reduced to
+// One instance (pl.f32), terms [p0, p1): one block of terms per resident cluster, then the
+// fixed-order sum of the blocks into the sink.  BZ_DATA_REAL: the input is first reduced to
 // its Hermitian, Nyquist-free part, the blocks are of term pairs [p0 / 2, p1 / 2), and the sum
 // is symmetrised at the end.
-bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches) {
+bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches, const Sink &sink) {
     const int n3 = pl.N * pl.N * pl.N;
     ItemArgs a;
-    a.fin = pl.fin; a.tw = pl.tw; a.alpha = pl.alpha; a.part = pl.part; a.hg = pl.h;
+    a.fin = pl.f32; a.tw = pl.tw; a.alpha = pl.alpha; a.part = pl.part; a.hg = pl.h;
     a.count = 1; a.p0 = p0; a.p1 = p1; a.M = pl.M; a.N_rho = pl.N_rho;
-    const void *src = pl.src ? pl.src : (const void *)pl.fin;
-    int src_dtype = pl.src ? pl.src_dtype : BZ_C64;
     int nl = 0;
     bz_status s = BZ_OK;
     if (pl.real) {
@@ -200,7 +197,7 @@ bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches
         if (!(pl.h_fp64 || pl.precision == BZ_PREC_BF16X3)) {
             // h formed in FP32 in the kernel from the symmetrised copy (the h pass writes it otherwise)
             tm_begin(pl, st);
-            s = sym_input(pl, src, src_dtype, st);
+            s = sym_input(pl, pl.src, pl.src_dtype, st);
             if (s != BZ_OK) return s;
             tm_end(pl, st, TK_OTHER);
             ++nl;
@@ -217,9 +214,9 @@ bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches
     a.nblk = nt > 0 ? (nt + a.TB - 1) / a.TB : 0;
     if (pl.h_fp64 || pl.precision == BZ_PREC_BF16X3) {
         tm_begin(pl, st);
-        s = hff_launch(pl.N, src, src_dtype, nullptr, nullptr, 1, pl.scr64,
+        s = hff_launch(pl.N, pl.src, pl.src_dtype, nullptr, nullptr, 1, pl.scr64,
                        pl.col32 ? (float2 *)pl.hcol : pl.h, st, pl.col32 ? pl.fcol : (pl.real ? pl.fsym : nullptr),
-                       pl.col32 != 0);
+                       pl.col32 != 0, pl.fcopy);
         if (s != BZ_OK) return s;
         tm_end(pl, st, TK_OTHER);
         nl += hff_launches(pl.N);
@@ -241,10 +238,10 @@ bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches
     tm_end(pl, st, TK_FUSED);
     tm_begin(pl, st);
     if (pl.real) {
-        s = pl.col32 ? reduce_col(pl, a.nblk, st) : reduce_sym(pl, a.nblk, st);   // sums of the blocks, symmetrised
+        s = pl.col32 ? reduce_col(pl, a.nblk, st, sink) : reduce_sym(pl, a.nblk, st, sink);   // sums of the blocks, symmetrised
         if (s != BZ_OK) return s;
     } else {
-        k_reduce_parts<<<(n3 + 31) / 32, 256, 0, st>>>(pl.part, a.nblk, n3, pl.acc);
+        reduce_parts(pl.part, a.nblk, n3, sink, st);
     }
     tm_end(pl, st, TK_REDUCE);
     BZ_CUDA_TRY(cudaGetLastError());

@@ -98,12 +98,15 @@ __device__ __forceinline__ ff split(double d) {
     const float s = __fadd_rn(h, l);                      // |lo| <= ulp(hi) / 2
     return {s, __fsub_rn(l, __fsub_rn(s, h))};
 }
-__device__ __forceinline__ ffc load_ff(const void *f, int dtype, size_t i) {
+// fcopy: the entry rounded to FP32 is stored there too
+__device__ __forceinline__ ffc load_ff(const void *f, int dtype, size_t i, float2 *fcopy = nullptr) {
     if (dtype == BZ_C128) {
         const double2 v = ((const double2 *)f)[i];
+        if (fcopy) fcopy[i] = make_float2((float)v.x, (float)v.y);
         return {split(v.x), split(v.y)};
     }
     const float2 v = ((const float2 *)f)[i];
+    if (fcopy) fcopy[i] = v;
     return {{v.x, 0.f}, {v.y, 0.f}};
 }
 
@@ -181,6 +184,7 @@ struct HArgs {
     float4 *scr;               // [slots][N^3] between the two launches (N = 24, 32)
     float2 *h;                 // [slots][N^3]
     float2 *fout;              // real data: the Hermitian, Nyquist-free part in FP32, or null
+    float2 *fcopy;             // complex data: f in FP32, or null
     int col;                   // k_col32's layouts: fout [k3 < 16][k1][k2], h packed floats [j3][j1][j2]
 };
 
@@ -188,7 +192,7 @@ struct HArgs {
 // stored.
 template <int N> __device__ __forceinline__ ffc input(const HArgs &a, size_t vol, int k1, int k2, int k3) {
     const size_t i = vol + ((size_t)k1 * N + k2) * N + k3;
-    if (!a.fout) return load_ff(a.f, a.dtype, i);
+    if (!a.fout) return load_ff(a.f, a.dtype, i, a.fcopy);
     constexpr int H = N / 2;
     ffc v = {{0.f, 0.f}, {0.f, 0.f}};
     if (k1 != H && k2 != H && k3 != H) {
@@ -294,7 +298,7 @@ template <int N> __global__ void __launch_bounds__(N * N) k_hff_cube(HArgs a) {
 }
 
 // 2D: one cluster of 8 CTAs, rows k1 = R c ..
-template <int N> __global__ void __launch_bounds__(N < 32 ? 32 : N) k_hff_2d(const void *f, int dtype, float2 *h) {
+template <int N> __global__ void __launch_bounds__(N < 32 ? 32 : N) k_hff_2d(const void *f, int dtype, float2 *h, float2 *fcopy) {
     constexpr int R = N / 8, LD = N + 1;
     __shared__ float4 s[R * LD];
     const int c = (int)cooperative_groups::this_cluster().block_rank();
@@ -302,7 +306,7 @@ template <int N> __global__ void __launch_bounds__(N < 32 ? 32 : N) k_hff_2d(con
     const int i = threadIdx.x / 8 < R ? threadIdx.x / 8 : R - 1;         // spare lanes repeat the last line
     ffc v[R];
     #pragma unroll
-    for (int m = 0; m < R; ++m) v[m] = load_ff(f, dtype, (size_t)(R * c + i) * N + F.l + 8 * m);
+    for (int m = 0; m < R; ++m) v[m] = load_ff(f, dtype, (size_t)(R * c + i) * N + F.l + 8 * m, fcopy);
     F(v);                                                    // k2 -> j2
     #pragma unroll
     for (int r = 0; r < R; ++r) s[i * LD + r + R * F.q] = pack(v[r]);
@@ -341,10 +345,10 @@ cudaError_t launch8(void (*k)(P...), dim3 grid, int threads, cudaStream_t st, A.
 }  // namespace
 
 bz_status hff_launch(int N, const void *f, int dtype, const int *slots, const int *count_dev, int count,
-                     double2 *scr, float2 *h, cudaStream_t st, float2 *fsym, bool col) {
+                     double2 *scr, float2 *h, cudaStream_t st, float2 *fsym, bool col, float2 *fcopy) {
     if (count <= 0) return BZ_OK;
     if ((col && N != 32) || (fsym && N == 24)) return BZ_ERR_UNSUPPORTED;
-    HArgs a = {f, dtype, slots, count_dev, (float4 *)scr, h, fsym, col};
+    HArgs a = {f, dtype, slots, count_dev, (float4 *)scr, h, fsym, fcopy, col};
     cudaError_t e = cudaSuccess;
     switch (N) {
         case 8: e = launch8(k_hff_cube<8>, dim3(8, count), 64, st, a); break;
@@ -364,13 +368,13 @@ bz_status hff_launch(int N, const void *f, int dtype, const int *slots, const in
     return BZ_OK;
 }
 
-bz_status hff_launch_2d(int N, const void *f, int dtype, float2 *h, cudaStream_t st) {
+bz_status hff_launch_2d(int N, const void *f, int dtype, float2 *h, float2 *fcopy, cudaStream_t st) {
     cudaError_t e = cudaSuccess;
     switch (N) {
-        case 8: e = launch8(k_hff_2d<8>, dim3(8), 32, st, f, dtype, h); break;
-        case 16: e = launch8(k_hff_2d<16>, dim3(8), 32, st, f, dtype, h); break;
-        case 32: e = launch8(k_hff_2d<32>, dim3(8), 32, st, f, dtype, h); break;
-        case 64: e = launch8(k_hff_2d<64>, dim3(8), 64, st, f, dtype, h); break;
+        case 8: e = launch8(k_hff_2d<8>, dim3(8), 32, st, f, dtype, h, fcopy); break;
+        case 16: e = launch8(k_hff_2d<16>, dim3(8), 32, st, f, dtype, h, fcopy); break;
+        case 32: e = launch8(k_hff_2d<32>, dim3(8), 32, st, f, dtype, h, fcopy); break;
+        case 64: e = launch8(k_hff_2d<64>, dim3(8), 64, st, f, dtype, h, fcopy); break;
         default: return BZ_ERR_UNSUPPORTED;
     }
     BZ_CUDA_TRY(e);

@@ -63,6 +63,8 @@ struct Plan {
     float2 *S = nullptr;            // [chunk][N^3]
     float2 *h = nullptr;            // [N^3]
     float2 *fin = nullptr;          // [N^3] FP32 input
+    const float2 *f32 = nullptr;    // the FP32 input of the call being issued: fin, or a complex64 caller's array
+    float2 *fcopy = nullptr;        // where the h pass stores it (complex128 callers), or null
     double2 *acc = nullptr;         // [N^3] FP64 accumulator (while a chunked collide runs, the same
                                     // bytes hold k_reduce's compensated FP32 state: s, c per mode pair)
     double2 *rk = nullptr;          // [3][N^3] RK4 state (f0, fsum) + spare
@@ -127,6 +129,62 @@ __device__ __forceinline__ void note_finite(float2 v, int *flag) {
 #endif
 inline int *nonfinite_flag(const Plan &pl) { return pl.dev_err ? pl.dev_err + 1 : nullptr; }
 
+// Where a collide's result goes: each kernel that finishes a mode's sum over the terms hands it on.
+struct Sink {
+    enum { ACC, OUT, RK };
+    int mode = ACC;
+    double2 *acc = nullptr;          // ACC: the plan's FP64 accumulator
+    void *out = nullptr;             // OUT: the caller's array; RK: the same after the last stage, or null
+    int dtype = BZ_C128;
+    int *flag = nullptr;             // raised by a NaN or Inf written to out
+    // RK: stage 1 .. 4 of a step (Sec. 5.2); k is the derivative at the stage's input
+    double2 *f0 = nullptr, *fsum = nullptr, *fin64 = nullptr;
+    float2 *fin = nullptr;
+    int stage = 0;
+    double dt = 0;
+};
+#ifdef __CUDACC__
+__device__ __forceinline__ void sink_store(void *out, int dtype, int *flag, size_t i, double2 v) {
+    if (dtype == BZ_C128) {
+        ((double2 *)out)[i] = v;
+        note_finite(v, flag);
+    } else {
+        const float2 w = make_float2((float)v.x, (float)v.y);
+        ((float2 *)out)[i] = w;
+        note_finite(w, flag);
+    }
+}
+__device__ __forceinline__ void sink_put(const Sink &s, size_t i, double2 v) {
+    if (s.mode == Sink::ACC) {
+        s.acc[i] = v;
+    } else if (s.mode == Sink::OUT) {
+        sink_store(s.out, s.dtype, s.flag, i, v);
+    } else {
+        // the state f0 and the running combination f0 + dt/6 (k1 + 2 k2 + 2 k3 + k4) in FP64; the next stage's
+        // input in FP32 (and FP64 for the h pass)
+        const double2 a = s.f0[i];
+        const double dt = s.dt;
+        double2 y;
+        if (s.stage == 1) {
+            s.fsum[i] = make_double2(a.x + dt / 6.0 * v.x, a.y + dt / 6.0 * v.y);
+            y = make_double2(a.x + 0.5 * dt * v.x, a.y + 0.5 * dt * v.y);
+        } else if (s.stage == 2 || s.stage == 3) {
+            const double2 u = s.fsum[i];
+            s.fsum[i] = make_double2(u.x + dt / 3.0 * v.x, u.y + dt / 3.0 * v.y);
+            const double c = s.stage == 2 ? 0.5 * dt : dt;
+            y = make_double2(a.x + c * v.x, a.y + c * v.y);
+        } else {
+            const double2 u = s.fsum[i];
+            y = make_double2(u.x + dt / 6.0 * v.x, u.y + dt / 6.0 * v.y);
+            s.f0[i] = y;
+            if (s.out) sink_store(s.out, s.dtype, s.flag, i, y);
+        }
+        s.fin[i] = make_float2((float)y.x, (float)y.y);
+        if (s.fin64) s.fin64[i] = y;
+    }
+}
+#endif
+
 // Fourier modes of one field: N^3 (3D) or N^2 (2D).
 inline size_t modes(const Plan &pl) { return (size_t)pl.N * pl.N * (pl.dim == 2 ? 1 : pl.N); }
 
@@ -152,11 +210,16 @@ bz_status ftable_build(Plan &pl);
 bz_status ftable_entries(Plan &pl, int count, const int *k_idx, const int *term, double *out);
 
 // bz_collide.cu
-bz_status collide_range(Plan &pl, int p0, int p1, const void *fhat, int in_dtype,
-                        cudaStream_t st, int *launches);
-bz_status write_output(Plan &pl, void *Qhat, int dtype, cudaStream_t st, int *launches);
-bz_status load_input(Plan &pl, const void *fhat, int dtype, cudaStream_t st, int *launches);
-bz_status collide_core(Plan &pl, int p0, int p1, cudaStream_t st, int *launches);
+// Qhat = Q over terms [p0, p1) of fhat (device arrays of one dtype)
+bz_status collide_range(Plan &pl, int p0, int p1, const void *fhat, void *Qhat, int dtype, cudaStream_t st,
+                        int *launches);
+// the input set by collide_range or rk4_steps (pl.f32, pl.src), the result to the sink
+bz_status collide_core(Plan &pl, int p0, int p1, cudaStream_t st, int *launches, const Sink &sink);
+inline Sink acc_sink(Plan &pl) {
+    Sink s;
+    s.acc = pl.acc;
+    return s;
+}
 // pl.h = IFFT(fin) in FP32 (one plane pass and one pencil pass through pl.S; N = 8, 16, 32)
 bz_status h_fp32(Plan &pl, const float2 *fin, cudaStream_t st);
 
@@ -188,30 +251,32 @@ inline int hff_launches(int N) { return N <= 16 ? 1 : 2; }
 // packed floats [j3][j1][j2]; the same stride of N^3 float2 per slot).  scr: 16 N^3 bytes per slot
 // (N = 24, 32).
 bz_status hff_launch(int N, const void *f, int dtype, const int *slots, const int *count_dev, int count,
-                     double2 *scr, float2 *h, cudaStream_t st, float2 *fsym = nullptr, bool col = false);
-bz_status hff_launch_2d(int N, const void *f, int dtype, float2 *h, cudaStream_t st);
-bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches);
+                     double2 *scr, float2 *h, cudaStream_t st, float2 *fsym = nullptr, bool col = false,
+                     float2 *fcopy = nullptr);
+// fcopy (complex data, c128): where f goes in FP32, or null
+bz_status hff_launch_2d(int N, const void *f, int dtype, float2 *h, float2 *fcopy, cudaStream_t st);
+bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches, const Sink &sink);
 // bz_real.cu (BZ_DATA_REAL): the pair table from alpha (after ftable_build); pl.fsym from a
 // c64 / c128 array
 bz_status build_pair_table(Plan &pl);
 bz_status sym_input(Plan &pl, const void *f, int dtype, cudaStream_t st);
-// pl.acc <- Q from the nblk item sums of pl.part (V) and pl.part_s (X): one kernel
-bz_status reduce_sym(Plan &pl, int nblk, cudaStream_t st);
-// chunked pipeline: pl.acc (V, FP64) <- Q in place, with pl.acc_s (X)
-bz_status sym_output(Plan &pl, cudaStream_t st);
+// sink <- Q from the nblk item sums of pl.part (V) and pl.part_s (X): one kernel
+bz_status reduce_sym(Plan &pl, int nblk, cudaStream_t st, const Sink &sink);
+// chunked pipeline: sink <- Q from pl.acc (V, FP64; may be the sink) with pl.acc_s (X)
+bz_status sym_output(Plan &pl, cudaStream_t st, const Sink &sink);
 
 // bz_pair3.cu (BZ_DATA_REAL, N = 32): resident clusters and launch of k_pair3
 cudaError_t pair3_setup(int *G);
 bz_status launch_pair3(const Plan &pl, const ItemArgs &a, cudaStream_t st);
 
 // bz_col32.cu (BZ_DATA_REAL, N = 32): one CTA per SM; items count terms.  The table from pl.alpha;
-// inputs from pl.fsym and pl.h (FP32 h); pl.acc <- the sum of nblk items
+// inputs from pl.fsym and pl.h (FP32 h); sink <- the sum of nblk items
 constexpr size_t kCol32Part = (size_t)18 * 32 * 32;     // float2 per item's sums
 cudaError_t col32_setup(int *G);
 bz_status launch_col32(const Plan &pl, const ItemArgs &a, cudaStream_t st);
 bz_status col32_table(Plan &pl);
 bz_status col32_inputs(Plan &pl, cudaStream_t st);
-bz_status reduce_col(Plan &pl, int nblk, cudaStream_t st);
+bz_status reduce_col(Plan &pl, int nblk, cudaStream_t st, const Sink &sink);
 
 // bz_mixed.cu (BZ_PREC_BF16X3, N = 32)
 cudaError_t mixed_setup(int N, int *G);
@@ -220,7 +285,7 @@ bz_status launch_mixed(const Plan &pl, const ItemArgs &a, cudaStream_t st);
 // one bounded wait that nothing completes, giving up after `limit` clocks (bz_plan_wait_selftest)
 bz_status wait_selftest(const Plan &pl, long long limit, cudaStream_t st);
 cudaError_t collide_set_attributes(int N);
-void reduce_parts(const float2 *part, int nblk, int n, double2 *acc, cudaStream_t st);
+void reduce_parts(const float2 *part, int nblk, int n, const Sink &sink, cudaStream_t st);
 int chunk_terms_for(int N);          // after collide_set_attributes(N)
 int supported_N(int N);
 
@@ -229,11 +294,11 @@ int lines_chunk(int N);
 int lines_splits(int N);
 inline bool lines_N(int N) { return N == 48 || N == 64; }
 cudaError_t lines_set_attributes(int N);
-bz_status collide_lines(Plan &pl, int p0, int p1, cudaStream_t st, int *launches);
+bz_status collide_lines(Plan &pl, int p0, int p1, cudaStream_t st, int *launches, const Sink &sink);
 
 // bz_2d.cu (dim = 2)
 cudaError_t setup_2d(Plan &pl);                       // persistent grid size (pl.fused_G)
-bz_status collide_2d(Plan &pl, int p0, int p1, cudaStream_t st, int *launches);
+bz_status collide_2d(Plan &pl, int p0, int p1, cudaStream_t st, int *launches, const Sink &sink);
 
 // bz_inhom.cu: free streaming of nx cells (bz_transport_x)
 bz_status transport_x(int N, double L, int nx, double Lx, void *f, int dtype, double t, cudaStream_t st);

@@ -300,9 +300,9 @@ __global__ void __launch_bounds__(256) k_x_sum(const float2 *__restrict__ xs, in
     acc[e] = make_double2((double)a.x - (double)a.z, (double)a.y - (double)a.w);
 }
 
-// acc[i] = the sum of the n_states running sums in order, compensated in FP32 and turned into FP64 once
+// sink(i) = the sum of the n_states running sums in order, compensated in FP32 and turned into FP64 once
 // (FP64 additions of every state took 26 us at N = 64).
-__global__ void k_state_sum(const float4 *__restrict__ state, int n_states, int n, double2 *__restrict__ acc) {
+__global__ void k_state_sum(const float4 *__restrict__ state, int n_states, int n, Sink sink) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -313,7 +313,7 @@ __global__ void k_state_sum(const float4 *__restrict__ state, int n_states, int 
         kahan(a.x, a.z, -v.z);
         kahan(a.y, a.w, -v.w);
     }
-    acc[i] = make_double2((double)a.x - (double)a.z, (double)a.y - (double)a.w);
+    sink_put(sink, i, make_double2((double)a.x - (double)a.z, (double)a.y - (double)a.w));
 }
 
 template <int N> cudaError_t attrs() {
@@ -332,7 +332,7 @@ template <int N> cudaError_t attrs() {
     return e;
 }
 
-template <int N, bool REAL> bz_status run(Plan &pl, int p0, int p1, cudaStream_t st, int *launches) {
+template <int N, bool REAL> bz_status run(Plan &pl, int p0, int p1, cudaStream_t st, int *launches, const Sink &sink) {
     using P = LP<N>;
     const int u0 = REAL ? p0 / 2 : p0, u1 = REAL ? p1 / 2 : p1;
     const int n3 = (int)P::N3, ns = REAL ? 3 * P::N2 : 0;
@@ -340,9 +340,9 @@ template <int N, bool REAL> bz_status run(Plan &pl, int p0, int p1, cudaStream_t
     int nl = 0;
     auto inv_smem = [](int per) { return (size_t)(2 * N * 32 + per * (REAL ? 6 : 3) * N) * sizeof(float2); };
     tm_begin(pl, st);
-    const float2 *f = pl.fin;
+    const float2 *f = pl.f32;
     if (REAL) {
-        const bz_status s = sym_input(pl, pl.src ? pl.src : (const void *)pl.fin, pl.src ? pl.src_dtype : BZ_C64, st);
+        const bz_status s = sym_input(pl, pl.src, pl.src_dtype, st);
         if (s != BZ_OK) return s;
         f = pl.fsym;
         ++nl;
@@ -352,9 +352,6 @@ template <int N, bool REAL> bz_status run(Plan &pl, int p0, int p1, cudaStream_t
     tm_end(pl, st, TK_OTHER);
     nl += 2;
     const int nchunks = (u1 - u0 + pl.chunk - 1) / pl.chunk;
-    if (nchunks == 0) {
-        BZ_CUDA_TRY(cudaMemsetAsync(pl.acc, 0, (size_t)n3 * sizeof(double2), st));
-    }
     // lanes: as many streams as chunks, up to 1 + pl.xn
     const int lanes = 1 + (pl.xn < nchunks - 1 ? pl.xn : (nchunks > 1 ? nchunks - 1 : 0));
     if (lanes > 1) {
@@ -385,14 +382,13 @@ template <int N, bool REAL> bz_status run(Plan &pl, int p0, int p1, cudaStream_t
         BZ_CUDA_TRY(cudaStreamWaitEvent(st, pl.xev_join[e], 0));
     }
     tm_begin(pl, st);
-    if (nchunks > 0) {
-        k_state_sum<<<(n3 + 255) / 256, 256, 0, st>>>(pl.lstate, lanes * P::SPLITS, n3, pl.acc);
-        ++nl;
-    }
+    k_state_sum<<<(n3 + 255) / 256, 256, 0, st>>>(pl.lstate, nchunks > 0 ? lanes * P::SPLITS : 0, n3,
+                                                 REAL ? acc_sink(pl) : sink);
+    ++nl;
     if (REAL) {
         k_x_sum<<<ns / 32, 256, 0, st>>>(pl.xs, u0, u1, ns, pl.acc_s);
         ++nl;
-        const bz_status s = sym_output(pl, st);
+        const bz_status s = sym_output(pl, st, sink);
         if (s != BZ_OK) return s;
         ++nl;
     }
@@ -408,9 +404,9 @@ cudaError_t lines_set_attributes(int N) { return N == 64 ? attrs<64>() : attrs<4
 int lines_chunk(int N) { return N == 64 ? LP<64>::CHUNK : LP<48>::CHUNK; }
 int lines_splits(int N) { return N == 64 ? LP<64>::SPLITS : LP<48>::SPLITS; }
 
-bz_status collide_lines(Plan &pl, int p0, int p1, cudaStream_t st, int *launches) {
-    if (pl.N == 64) return pl.real ? run<64, true>(pl, p0, p1, st, launches) : run<64, false>(pl, p0, p1, st, launches);
-    return pl.real ? run<48, true>(pl, p0, p1, st, launches) : run<48, false>(pl, p0, p1, st, launches);
+bz_status collide_lines(Plan &pl, int p0, int p1, cudaStream_t st, int *launches, const Sink &sink) {
+    if (pl.N == 64) return pl.real ? run<64, true>(pl, p0, p1, st, launches, sink) : run<64, false>(pl, p0, p1, st, launches, sink);
+    return pl.real ? run<48, true>(pl, p0, p1, st, launches, sink) : run<48, false>(pl, p0, p1, st, launches, sink);
 }
 
 }  // namespace bz

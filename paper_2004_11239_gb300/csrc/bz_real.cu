@@ -56,13 +56,13 @@ struct Kahan {
     }
 };
 
-// acc(k) = V(k) + conj V(-k) off S and V(k) + conj X(-k) on S, with V and X the sums over the
+// sink(k) = V(k) + conj V(-k) off S and V(k) + conj X(-k) on S, with V and X the sums over the
 // G items of part and part_s.  Block: 32 modes k x 8 slices; slice s sums items s, s + 8, ...
 // of the two entries mode k needs (V(k) and V(-k), or V(k) and X(-k)), then the eight slices are
 // added in order (compensated, as k_reduce_parts).  Off S the lane of the smaller index of each
 // pair {k, -k} writes both entries; k = 0 is its own mirror.
 __global__ void __launch_bounds__(256) k_reduce_sym(const float2 *__restrict__ part, const float2 *__restrict__ part_s,
-                                                   int G, int N, double2 *__restrict__ acc) {
+                                                   int G, int N, Sink sink) {
     __shared__ float4 red[2][8][32];
     const int n3 = N * N * N;
     const int kk = threadIdx.x % 32, sl = threadIdx.x / 32;
@@ -109,17 +109,17 @@ __global__ void __launch_bounds__(256) k_reduce_sym(const float2 *__restrict__ p
     const double2 va = make_double2((double)ta.sr - (double)ta.cr, (double)ta.si - (double)ta.ci);
     const double2 vb = make_double2((double)tb.sr - (double)tb.cr, (double)tb.si - (double)tb.ci);
     if (role == 2 || (size_t)k != j) {
-        acc[k] = make_double2(va.x + vb.x, va.y - vb.y);
-        if (role == 1) acc[j] = make_double2(vb.x + va.x, vb.y - va.y);
+        sink_put(sink, k, make_double2(va.x + vb.x, va.y - vb.y));
+        if (role == 1) sink_put(sink, j, make_double2(vb.x + va.x, vb.y - va.y));
     } else {
-        acc[k] = make_double2(2.0 * va.x, 0.0);                       // k = 0
+        sink_put(sink, k, make_double2(2.0 * va.x, 0.0));             // k = 0
     }
 }
 
-// In place: acc(k) <- V(k) + conj V(-k) off S, V(k) + conj X(-k) on S (xs: the FP64 sums X in
+// sink(k) <- V(k) + conj V(-k) off S, V(k) + conj X(-k) on S (acc: V, may be the sink; xs: the FP64 sums X in
 // the family layout).  Off S the thread of the smaller index of each pair {k, -k} writes both
 // entries; k = 0 is its own mirror.
-__global__ void k_sym_out(double2 *__restrict__ acc, const double2 *__restrict__ xs, int N) {
+__global__ void k_sym_out(const double2 *acc, const double2 *__restrict__ xs, int N, Sink sink) {
     const int n3 = N * N * N;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n3) return;
@@ -128,18 +128,18 @@ __global__ void k_sym_out(double2 *__restrict__ acc, const double2 *__restrict__
     const double2 a = acc[k];
     if (nyquist(i1, i2, i3, N)) {
         const double2 x = xs[family_index(m1, m2, m3, N)];
-        acc[k] = make_double2(a.x + x.x, a.y - x.y);
+        sink_put(sink, k, make_double2(a.x + x.x, a.y - x.y));
         return;
     }
     const size_t m = ((size_t)m1 * N + m2) * N + m3;
     if ((size_t)k > m) return;
     if ((size_t)k == m) {
-        acc[k] = make_double2(2.0 * a.x, 0.0);
+        sink_put(sink, k, make_double2(2.0 * a.x, 0.0));
         return;
     }
     const double2 b = acc[m];
-    acc[k] = make_double2(a.x + b.x, a.y - b.y);
-    acc[m] = make_double2(b.x + a.x, b.y - a.y);
+    sink_put(sink, k, make_double2(a.x + b.x, a.y - b.y));
+    sink_put(sink, m, make_double2(b.x + a.x, b.y - a.y));
 }
 
 // A_q(k) = (alpha_2q(k) - i alpha_2q+1(k)) / 2 for every k.
@@ -193,9 +193,9 @@ bz_status sym_input(Plan &pl, const void *f, int dtype, cudaStream_t st) {
     return BZ_OK;
 }
 
-bz_status reduce_sym(Plan &pl, int nblk, cudaStream_t st) {
+bz_status reduce_sym(Plan &pl, int nblk, cudaStream_t st, const Sink &sink) {
     const int n3 = (int)modes(pl);
-    k_reduce_sym<<<(n3 + 31) / 32, 256, 0, st>>>(pl.part, pl.part_s, nblk, pl.N, pl.acc);
+    k_reduce_sym<<<(n3 + 31) / 32, 256, 0, st>>>(pl.part, pl.part_s, nblk, pl.N, sink);
     BZ_CUDA_TRY(cudaGetLastError());
     return BZ_OK;
 }
@@ -204,9 +204,9 @@ bz_status reduce_sym(Plan &pl, int nblk, cudaStream_t st) {
 
 namespace bz {
 
-bz_status sym_output(Plan &pl, cudaStream_t st) {
+bz_status sym_output(Plan &pl, cudaStream_t st, const Sink &sink) {
     const int n3 = (int)modes(pl);
-    k_sym_out<<<(n3 + 255) / 256, 256, 0, st>>>(pl.acc, pl.acc_s, pl.N);
+    k_sym_out<<<(n3 + 255) / 256, 256, 0, st>>>(pl.acc, pl.acc_s, pl.N, sink);
     BZ_CUDA_TRY(cudaGetLastError());
     return BZ_OK;
 }

@@ -1,8 +1,8 @@
 // Classical RK4 for d fhat/dt = Q(fhat, fhat) (Sec. 5.2) and FP64 moments (Sec. 1, Sec. 4).
 //
 // RK4: the step state f0 and the running combination fsum = f0 + dt/6 (k1 + 2k2 + 2k3 + k4)
-// are FP64; each stage's collide input is rounded to FP32 (pl.fin) and each stage
-// derivative k_s arrives in the FP64 accumulator of the collide pipeline.
+// are FP64; each stage's collide input is rounded to FP32 (pl.fin), and the kernel that finishes
+// a mode of a stage's collide updates the mode's state (Sink::RK).
 #include <cmath>
 
 #include "bz_internal.h"
@@ -25,41 +25,9 @@ __global__ void k_rk_init(const void *fhat, int dtype, double2 *f0, float2 *fin,
     if (fin64) fin64[i] = v;
 }
 
-// stage s in {1, 2, 3, 4}; k = acc (FP64 derivative of stage s)
-__global__ void k_rk_stage(const double2 *__restrict__ k, double2 *__restrict__ f0,
-                           double2 *__restrict__ fsum, float2 *__restrict__ fin, double2 *__restrict__ fin64,
-                           int n, int stage, double dt) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double2 kv = k[i], a = f0[i], y;
-    if (stage == 1) {
-        fsum[i] = make_double2(a.x + dt / 6.0 * kv.x, a.y + dt / 6.0 * kv.y);
-        y = make_double2(a.x + 0.5 * dt * kv.x, a.y + 0.5 * dt * kv.y);
-    } else if (stage == 2 || stage == 3) {
-        double2 s = fsum[i];
-        fsum[i] = make_double2(s.x + dt / 3.0 * kv.x, s.y + dt / 3.0 * kv.y);
-        double c = stage == 2 ? 0.5 * dt : dt;
-        y = make_double2(a.x + c * kv.x, a.y + c * kv.y);
-    } else {
-        double2 s = fsum[i];
-        y = make_double2(s.x + dt / 6.0 * kv.x, s.y + dt / 6.0 * kv.y);
-        f0[i] = y;
-    }
-    fin[i] = make_float2((float)y.x, (float)y.y);
-    if (fin64) fin64[i] = y;
-}
-
 __global__ void k_rk_out(const double2 *f0, void *fhat, int dtype, int n, int *flag) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    if (dtype == BZ_C128) {
-        ((double2 *)fhat)[i] = f0[i];
-        note_finite(f0[i], flag);
-    } else {
-        const float2 w = make_float2((float)f0[i].x, (float)f0[i].y);
-        ((float2 *)fhat)[i] = w;
-        note_finite(w, flag);
-    }
+    if (i < n) sink_store(fhat, dtype, flag, i, f0[i]);
 }
 
 // Moments of f_N over [-L, L]^3.  Only the modes on the three axes contribute:
@@ -105,19 +73,30 @@ bz_status rk4_steps(Plan &pl, void *fhat, int dtype, double dt, int nsteps, cuda
     const int bs = 256, gs = (n + bs - 1) / bs;
     double2 *f0 = pl.rk, *fsum = pl.rk + n;
     k_rk_init<<<gs, bs, 0, st>>>(fhat, dtype, f0, pl.fin, pl.fin64, n);
-    pl.src = pl.fin64;             // stage inputs for the h pass (fused plans)
-    pl.src_dtype = BZ_C128;
     int nl = 1;
-    for (int step = 0; step < nsteps; ++step) {
-        for (int stage = 1; stage <= 4; ++stage) {
-            bz_status s = collide_core(pl, 0, pl.P, st, &nl);
-            if (s != BZ_OK) return s;
-            k_rk_stage<<<gs, bs, 0, st>>>(pl.acc, f0, fsum, pl.fin, pl.fin64, n, stage, dt);
-            ++nl;
+    // stage inputs: FP32 for the terms; FP64 for h where the plan has it (fused and 2D), else the FP32 ones
+    pl.f32 = pl.fin;
+    pl.fcopy = nullptr;
+    pl.src = pl.fin64 ? (const void *)pl.fin64 : pl.fin;
+    pl.src_dtype = pl.fin64 ? BZ_C128 : BZ_C64;
+    Sink sink;
+    sink.mode = Sink::RK;
+    sink.f0 = f0; sink.fsum = fsum; sink.fin = pl.fin; sink.fin64 = pl.fin64; sink.dt = dt;
+    sink.dtype = dtype; sink.flag = nonfinite_flag(pl);
+    bz_status s = BZ_OK;
+    for (int step = 0; step < nsteps && s == BZ_OK; ++step) {
+        for (int stage = 1; stage <= 4 && s == BZ_OK; ++stage) {
+            sink.stage = stage;
+            sink.out = stage == 4 && step == nsteps - 1 ? fhat : nullptr;
+            s = collide_core(pl, 0, pl.P, st, &nl, sink);
         }
     }
-    k_rk_out<<<gs, bs, 0, st>>>(f0, fhat, dtype, n, nonfinite_flag(pl));
-    ++nl;
+    pl.src = nullptr;
+    if (s != BZ_OK) return s;
+    if (nsteps == 0) {
+        k_rk_out<<<gs, bs, 0, st>>>(f0, fhat, dtype, n, nonfinite_flag(pl));
+        ++nl;
+    }
     BZ_CUDA_TRY(cudaGetLastError());
     if (launches) *launches += nl;
     return BZ_OK;
