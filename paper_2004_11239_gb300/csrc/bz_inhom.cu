@@ -5,78 +5,122 @@
 // fhat_c(k1, k2, k3) is transformed over the cells (x-DFT), over k1 to the node values
 // f(v_1j) = sum_k1 (-1)^k1 fhat(k1) exp(2 pi i k1 j / N) (the factor (-1)^k1 = exp(-i pi k1)
 // from the grid origin -L), multiplied by exp(-2 pi i kappa v_1j t / Lx), and transformed back.
-// One CTA per (k2, k3); FP64 register FFTs; the array sits in shared memory between the passes.
+// One CTA per (k2, k3); the array sits in shared memory between the passes, a line takes eight
+// lanes (bz_line8.cuh).  complex128 cells are computed in FP64, complex64 ones in double-float (the
+// stored result has the error of its rounding; an FP64 instruction of a warp takes 68 clocks of a
+// scheduler).  The phases are products of two tables of powers of exp(2 pi i t L / (Lx N)), 64 FP64
+// sincospi a CTA.
 #include <cmath>
 
-#include "bz_fft.cuh"
 #include "bz_internal.h"
+#include "bz_line8.cuh"
 
 namespace bz {
 
 namespace {
 
-__device__ __forceinline__ double2 load_cd(const void *f, int dtype, size_t i) {
-    if (dtype == BZ_C128) return ((const double2 *)f)[i];
-    const float2 v = ((const float2 *)f)[i];
-    return make_double2(v.x, v.y);
+// exp(i m theta) = a[m / 32] b[m mod 32] for |m| <= 512
+struct Phases {
+    double2 a[17], b[32];
+};
+__device__ __forceinline__ void load_c(const void *f, size_t i, cd &v) {
+    const double2 u = ((const double2 *)f)[i];
+    v = {u.x, u.y};
 }
-__device__ __forceinline__ void store_cd(void *f, int dtype, size_t i, double2 v) {
-    if (dtype == BZ_C128) ((double2 *)f)[i] = v;
-    else ((float2 *)f)[i] = make_float2((float)v.x, (float)v.y);
+__device__ __forceinline__ void load_c(const void *f, size_t i, ffc &v) {
+    const float2 u = ((const float2 *)f)[i];
+    v = {{u.x, 0.f}, {u.y, 0.f}};
 }
+__device__ __forceinline__ void store_c(void *f, size_t i, cd v) { ((double2 *)f)[i] = make_double2(v.x, v.y); }
+__device__ __forceinline__ void store_c(void *f, size_t i, ffc v) { ((float2 *)f)[i] = round2(v); }
+__device__ __forceinline__ void from_d(double2 u, cd &v) { v = {u.x, u.y}; }
+__device__ __forceinline__ void from_d(double2 u, ffc &v) { v = {split(u.x), split(u.y)}; }
+__device__ __forceinline__ cd times(cd v, double s) { return scale(v, s); }
+__device__ __forceinline__ ffc times(ffc v, double s) { return scale(v, split(s)); }
 
-template <int N, int NX>
-__global__ void __launch_bounds__(N > NX ? N : NX) k_transport(void *f, int dtype, double L, double Lx, double t) {
-    __shared__ double2 s[NX][N + 1];
+// Threads: 8 lanes a line, max(N, NX) lines.  C = cd (complex128 cells) or ffc (complex64).
+// Bound by FP64 issue (cd) or by latency (ffc).  N = 16, 32 cells of complex64: 9.0 us; one line a
+// thread in FP64 with a sincospi per value took 63.
+template <int N, int NX, class C>
+__global__ void __launch_bounds__(8 * (N > NX ? N : NX)) k_transport(void *f, double tau) {
+    constexpr int R = N / 8, RX = NX / 8;
+    __shared__ C s[NX][N + 1];
+    __shared__ Phases ph;
     const size_t n3 = (size_t)N * N * N;
-    const size_t line = blockIdx.x;                          // k2 N + k3
-    const int tid = threadIdx.x;
-    if (tid < N) {                                           // column k1 = tid over the cells
-        double2 x[NX];
+    const size_t at = blockIdx.x;                            // k2 N + k3
+    const int tid = threadIdx.x, line = tid / 8;
+    if (tid < 49) {
+        const int m = tid < 32 ? tid : 32 * (tid - 32);
+        double sn, cs;
+        sincospi(2.0 * tau * m, &sn, &cs);
+        if (tid < 32) ph.b[tid] = make_double2(cs, sn);
+        else ph.a[tid - 32] = make_double2(cs, sn);
+    }
+    const LineFF<NX, C> X(tid & 7);
+    const bool col = line < N;                               // whole warps: N and NX are multiples of 4
+    C x[RX];
+    if (col) {                                               // column k1 = line over the cells
         #pragma unroll
-        for (int c = 0; c < NX; ++c) x[c] = load_cd(f, dtype, c * n3 + (size_t)tid * N * N + line);
-        fft_inplace<NX, -1>(x);                              // cells -> x-modes kappa
+        for (int m = 0; m < RX; ++m) {
+            load_c(f, (X.l + 8 * m) * n3 + (size_t)line * N * N + at, x[m]);
+            x[m] = conj(x[m]);                               // forward by the inverse: conj, transform, conj
+        }
+        X(x);                                                // cells -> x-modes kappa
         #pragma unroll
-        for (int c = 0; c < NX; ++c) s[c][tid] = x[c];
+        for (int r = 0; r < RX; ++r) s[r + RX * X.q][line] = conj(x[r]);
     }
     __syncthreads();
-    if (tid < NX) {                                          // x-mode row c over k1
-        double2 y[N];
+    if (line < NX) {                                         // x-mode row over k1
+        const LineFF<N, C> F(tid & 7);
+        C y[R];
         #pragma unroll
-        for (int i = 0; i < N; ++i) {
-            const double2 v = s[tid][i];
-            y[i] = (i & 1) ? make_double2(-v.x, -v.y) : v;
+        for (int m = 0; m < R; ++m) {
+            y[m] = s[line][F.l + 8 * m];
+            if (F.l & 1) y[m] = neg(y[m]);                   // (-1)^k1
         }
-        fft_inplace<N, +1>(y);                               // k1 -> node values f(v_1j)
-        const double kappa = tid < NX / 2 ? tid : tid - NX;
-        const double a = -2.0 * kappa * t / Lx;              // phase exp(i pi a v_1j)
+        F(y);                                                // k1 -> node values f(v_1j)
+        // phase exp(-2 pi i kappa v_1j t / Lx), v_1j = -L + 2 L j / N: exp(i kappa (N - 2 j) theta)
+        const int kappa = line < NX / 2 ? line : line - NX;
         #pragma unroll
-        for (int j = 0; j < N; ++j) {
-            double sn, cs;
-            sincospi(a * (-L + 2.0 * L * j / N), &sn, &cs);
-            y[j] = make_double2(y[j].x * cs - y[j].y * sn, y[j].x * sn + y[j].y * cs);
+        for (int r = 0; r < R; ++r) {
+            const int j = r + R * F.q, m = kappa * (N - 2 * j), am = m < 0 ? -m : m;
+            C a, b;
+            from_d(ph.a[am >> 5], a);
+            from_d(ph.b[am & 31], b);
+            a = mul(a, b);
+            y[r] = conj(mul(y[r], m < 0 ? conj(a) : a));
         }
-        fft_inplace<N, -1>(y);                               // node values -> k1
+        // node values -> k1: y[r] sits at j = r + R q of lane bitrev; back to j = l + 8 m through shared memory
+        __syncwarp();
+        #pragma unroll
+        for (int r = 0; r < R; ++r) s[line][r + R * F.q] = y[r];
+        __syncwarp();
+        #pragma unroll
+        for (int m = 0; m < R; ++m) y[m] = s[line][F.l + 8 * m];
+        F(y);
+        __syncwarp();
         const double inv = 1.0 / ((double)N * NX);           // both inverse normalisations
         #pragma unroll
-        for (int i = 0; i < N; ++i) {
-            const double sg = (i & 1) ? -inv : inv;
-            s[tid][i] = make_double2(y[i].x * sg, y[i].y * sg);
+        for (int r = 0; r < R; ++r) {
+            const int k = r + R * F.q;
+            s[line][k] = times(conj(y[r]), (k & 1) ? -inv : inv);
         }
     }
     __syncthreads();
-    if (tid < N) {
-        double2 x[NX];
+    if (col) {
         #pragma unroll
-        for (int c = 0; c < NX; ++c) x[c] = s[c][tid];
-        fft_inplace<NX, +1>(x);                              // x-modes -> cells
+        for (int m = 0; m < RX; ++m) x[m] = s[X.l + 8 * m][line];
+        X(x);                                                // x-modes -> cells
         #pragma unroll
-        for (int c = 0; c < NX; ++c) store_cd(f, dtype, c * n3 + (size_t)tid * N * N + line, x[c]);
+        for (int r = 0; r < RX; ++r) store_c(f, (r + RX * X.q) * n3 + (size_t)line * N * N + at, x[r]);
     }
 }
 
 template <int N, int NX> bz_status run(void *f, int dtype, double L, double Lx, double t, cudaStream_t st) {
-    k_transport<N, NX><<<N * N, N > NX ? N : NX, 0, st>>>(f, dtype, L, Lx, t);
+    const double tau = t * L / (Lx * N);
+    constexpr int threads = 8 * (N > NX ? N : NX);
+    if (dtype == BZ_C128) k_transport<N, NX, cd><<<N * N, threads, 0, st>>>(f, tau);
+    else k_transport<N, NX, ffc><<<N * N, threads, 0, st>>>(f, tau);
     BZ_CUDA_TRY(cudaGetLastError());
     return BZ_OK;
 }
