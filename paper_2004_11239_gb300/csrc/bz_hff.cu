@@ -186,7 +186,7 @@ template <int N> __global__ void __launch_bounds__(N < 32 ? 32 : N) k_hff_2d(con
     }
     F(v);                                                    // k1 -> j1 of column j2 = R c + i
     #pragma unroll
-    for (int r = 0; r < R; ++r) h[(size_t)(r + R * F.q) * N + R * c + i] = round2(v[r]);
+    for (int r = 0; r < R; ++r) h[(size_t)(R * c + i) * N + r + R * F.q] = round2(v[r]);   // [j2][j1]
     cooperative_groups::this_cluster().sync();
 }
 
