@@ -21,9 +21,11 @@
 //     Legendre series of about z + 25 terms of three FP64 operations, against a few hundred rule
 //     nodes of some hundred operations each.
 #include <cmath>
+#include <cstring>
 #include <vector>
 
 #include "bz_internal.h"
+#include "bz_line8.cuh"
 
 namespace bz {
 
@@ -71,6 +73,11 @@ struct TableArgs {
     int i0, g0, nkk, stride; // node of blockIdx.z = 0, term group of blockIdx.y = 0
     const double *coef;
     const int *cut;
+    const double *g;         // [stride] g_l of the recurrence (double-float form: hi, lo as float2)
+    // the double-float form
+    const float2 *rk;        // [nkk] 1 / |k|
+    const float2 *tq;        // [P][4] qhat, c_p / N^3
+    const float4 *ph;        // [P][3][N] exp(i a qhat_d k)
 };
 
 // Coefficients of the Legendre series: row (radial node i, m = |k|^2) holds
@@ -78,9 +85,13 @@ struct TableArgs {
 // sign of (-i)^l and the scale of the recurrence's polynomials; cut (even) drops the tail below
 // 2^-60 of the row's largest.  j_l by downward recurrence from lmax (where |j_l| < 1e-22 for the
 // largest z, or from the l where that holds for this z), normalised by sum (2l + 1) j_l^2 = 1 with
-// the sign of j_0 = sin z / z or j_1.  One thread per row; the work is a few percent of the table's.
+// the sign of j_0 = sin z / z or j_1.  One thread per row.
+// Double-float form (dblf): entries as (hi, lo) float2, and ahead of them kRowHead with part I in the same
+// variables, x = z c, y^2 = z^2 (1 - c^2): w0 + w1 c^2 + i w2 c.
+constexpr int kRowHead = 4;
 struct CoefArgs {
-    int i0, ni, nkk, stride, lmax;
+    int i0, ni, nkk, stride, lmax, dblf;
+    double A0, A1, A2;
     double L;
     const double *r;         // [N_rho] radial nodes
     const double *mu;        // [lmax + 1]
@@ -93,7 +104,18 @@ __global__ void __launch_bounds__(64) k_legendre_coef(CoefArgs a) {
     if (m >= a.nkk) return;
     const size_t row = (size_t)blockIdx.y * a.nkk + m;
     const double z = M_PI * a.r[a.i0 + blockIdx.y] * sqrt((double)m) / (2.0 * a.L);
-    double *c = a.coef + row * a.stride;
+    double *c = a.coef + row * a.stride + (a.dblf ? kRowHead : 0);
+    auto pair = [](double v) {
+        const float h = (float)v;
+        return make_float2(h, (float)(v - (double)h));
+    };
+    if (a.dblf) {
+        float2 *w = (float2 *)(c - kRowHead);
+        w[0] = pair(-0.5 * M_PI * z * z * a.A2);
+        w[1] = pair(-2.0 * M_PI * z * z * (0.5 * a.A1 - 0.25 * a.A2));
+        w[2] = pair(2.0 * M_PI * z * a.A0);
+        w[3] = make_float2(0.f, 0.f);
+    }
     if (!(z > 0.0)) {                                     // k = 0: F = 0
         a.cut[row] = 0;
         return;
@@ -131,19 +153,21 @@ __global__ void __launch_bounds__(64) k_legendre_coef(CoefArgs a) {
     while (n > 1 && fabs(c[n]) < 0x1p-60 * big) --n;
     if ((n & 1) == 0) c[n + 1] = 0.0;                     // pairs (even, odd); stride >= lmax + 2
     a.cut[row] = (n | 1) + 1;
+    if (a.dblf)
+        for (int l = 0; l <= (n | 1); ++l) ((float2 *)c)[l] = pair(c[l]);
 }
 
 // Thread: one mode k (of each pair k, -k) and up to kLegTerms terms of one radial node, sharing the
 // coefficient row.  The polynomials are 2^l times the monic Legendre ones, q_{l+1} = 2c q_l -
 // g_l q_{l-1}, g_l = 4 l^2 / (4 l^2 - 1): two FP64 operations a step and a third for the sum; no
 // over- or underflow for any l.  FP64 bound (this part runs about two FP64 lanes per clock and SM).
-// Measured at N = 32, P = 384 (R = 6, s = 1/2): 4.6 ms, and 0.19 ms for the rows; the direct sum over
-// the rule took 578 ms (plan creation 582 -> 8.0 ms).
+// Measured at N = 32, P = 384 (R = 6, s = 1/2): 4.6 ms; the direct sum over the rule took 578 ms.  It serves
+// series longer than kFfSeries, where the double-float form below has fewer bits to spare.
 constexpr int kLegTerms = 4;
 
 __global__ void __launch_bounds__(128) ftable_kernel(TableArgs a) {
     extern __shared__ double sg[];                        // g_l, l = 0 .. lmax + 1
-    for (int t = threadIdx.x; t < a.stride; t += blockDim.x) sg[t] = 4.0 * t * t / (4.0 * t * t - 1.0);
+    for (int t = threadIdx.x; t < a.stride; t += blockDim.x) sg[t] = a.g[t];
     __syncthreads();
     const int N = a.N, n3 = N * N * N;
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -212,6 +236,94 @@ __global__ void __launch_bounds__(128) ftable_kernel(TableArgs a) {
         float2 *al = a.alpha + (size_t)(p0 + u) * n3;
         al[idx] = in_k ? make_float2((float)fr, (float)fi) : make_float2(0.f, 0.f);
         if (midx > idx) al[midx] = in_m ? make_float2((float)fr, (float)(-fi)) : make_float2(0.f, 0.f);
+    }
+}
+
+// The same series in double-float arithmetic (pairs of FP32, about 47 bits; bz_line8.cuh): an FP64 instruction of a
+// warp takes 68 clocks of a scheduler, a double-float product and sum 37 FP32 instructions.  No FP64 in
+// the kernel: 1 / |k|, the axes' exp(i a qhat_d k_d) and part I's coefficients come from tables.  The
+// table's error against 64 bits stays that of its FP32 rounding (2.6e-8).  Bound by FP32 issue.
+// Measured at N = 32, P = 384: 0.80 ms and 0.20 for the rows, 4.6 in FP64 (plan creation 7.1 -> 2.9 ms; 46 s ->
+// 91 ms at N = 64, P = 4096 since the direct sum).
+__device__ __forceinline__ ff fmul(ff a, ff b) {
+    const float p = __fmul_rn(a.h, b.h);
+    const float e = __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.h, -p)));
+    const float h = __fadd_rn(p, e);
+    return {h, __fsub_rn(e, __fsub_rn(h, p))};
+}
+__device__ __forceinline__ ff ld(float2 v) { return {v.x, v.y}; }
+
+__global__ void k_axis_phases(int N, int M, double L, const double *__restrict__ term, float4 *__restrict__ ph) {
+    const int p = blockIdx.x, d = threadIdx.x / N, i = threadIdx.x % N, k = i < N / 2 ? i : i - N;
+    double sn, cs;
+    sincos(M_PI * term[5 * p] / (2.0 * L) * term[5 * p + 1 + d] * k, &sn, &cs);
+    const float c = (float)cs, s = (float)sn;
+    ph[(size_t)p * 3 * N + threadIdx.x] = make_float4(c, (float)(cs - c), s, (float)(sn - s));
+}
+
+__global__ void __launch_bounds__(128) ftable_ff_kernel(TableArgs a) {
+    extern __shared__ float2 sgf[];                       // g_l
+    const int N = a.N, n3 = N * N * N;
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    for (int t = threadIdx.x; t < a.stride; t += blockDim.x) sgf[t] = ((const float2 *)a.g)[t];
+    __syncthreads();
+    if (idx >= n3) return;
+    const int il = blockIdx.z, j0 = (a.g0 + blockIdx.y) * kLegTerms;
+    const int p0 = (a.i0 + il) * a.M + j0, np = min(kLegTerms, a.M - j0);
+    const int i1 = idx / (N * N), i2 = (idx / N) % N, i3 = idx % N;
+    const int k1 = i1 < N / 2 ? i1 : i1 - N, k2 = i2 < N / 2 ? i2 : i2 - N, k3 = i3 < N / 2 ? i3 : i3 - N;
+    // pairs (k, -k) and the padded range as in ftable_kernel
+    const bool nyq = k1 == -N / 2 || k2 == -N / 2 || k3 == -N / 2;
+    int midx = -1;
+    if (!nyq) {
+        midx = (((-k1 + N) % N) * N + ((-k2 + N) % N)) * N + ((-k3 + N) % N);
+        if (midx < idx) return;
+    }
+    const int h = a.nin / 2;
+    const bool in_k = a.nin == 0 || (k1 >= -h && k1 < h && k2 >= -h && k2 < h && k3 >= -h && k3 < h);
+    const bool in_m = midx >= 0 && (a.nin == 0 || (-k1 >= -h && -k1 < h && -k2 >= -h && -k2 < h && -k3 >= -h && -k3 < h));
+    const int kk = k1 * k1 + k2 * k2 + k3 * k3;
+    const size_t row = (size_t)il * a.nkk + kk;
+    const float2 *rw = (const float2 *)(a.coef + row * a.stride);
+    const float4 *c = (const float4 *)(rw + kRowHead);
+    const int cut = in_k || in_m ? a.cut[row] : 0;
+    const ff rk = ld(a.rk[kk]), zero = {0.f, 0.f};
+    ff ch[kLegTerms], c2[kLegTerms], q0[kLegTerms], q1[kLegTerms], sr[kLegTerms], si[kLegTerms];
+    #pragma unroll
+    for (int u = 0; u < kLegTerms; ++u) {
+        const float2 *tq = a.tq + 4 * (size_t)(p0 + (u < np ? u : 0));
+        const ff f1 = {(float)k1, 0.f}, f2 = {(float)k2, 0.f}, f3 = {(float)k3, 0.f};
+        ch[u] = fmul(fadd(fdot<1>(ld(tq[0]), f1, ld(tq[1]), f2), fmul(ld(tq[2]), f3)), rk);   // cos chi
+        c2[u] = {2.f * ch[u].h, 2.f * ch[u].l};
+        q0[u] = {1.f, 0.f};
+        q1[u] = c2[u];
+        sr[u] = si[u] = zero;
+    }
+    for (int l = 0; l < cut; l += 2) {
+        const float4 cl = c[l / 2];
+        const ff ca = {cl.x, cl.y}, cb = {cl.z, cl.w}, ga = ld(sgf[l + 1]), gb = ld(sgf[l + 2]);
+        #pragma unroll
+        for (int u = 0; u < kLegTerms; ++u) {
+            sr[u] = fadd(sr[u], fmul(ca, q0[u]));
+            si[u] = fadd(si[u], fmul(cb, q1[u]));
+            q0[u] = fdot<-1>(c2[u], q1[u], ga, q0[u]);
+            q1[u] = fdot<-1>(c2[u], q0[u], gb, q1[u]);
+        }
+    }
+    const ff w0 = ld(rw[0]), w1 = ld(rw[1]), w2 = ld(rw[2]);
+    #pragma unroll
+    for (int u = 0; u < kLegTerms; ++u) {
+        if (u >= np) break;
+        const float4 *ph = a.ph + (size_t)(p0 + u) * 3 * N;
+        const ffc e = mul(mul(unpack(ph[i1]), unpack(ph[N + i2])), unpack(ph[2 * N + i3]));
+        ffc F = mul(e, {sr[u], si[u]});
+        F.x = fadd(F.x, fadd(w0, fmul(w1, fmul(ch[u], ch[u]))));
+        F.y = fadd(F.y, fmul(w2, ch[u]));
+        const ff sc = ld(a.tq[4 * (size_t)(p0 + u) + 3]);
+        const float fr = fmul(F.x, sc).h, fi = fmul(F.y, sc).h;
+        float2 *al = a.alpha + (size_t)(p0 + u) * n3;
+        al[idx] = in_k ? make_float2(fr, fi) : make_float2(0.f, 0.f);
+        if (midx > idx) al[midx] = in_m ? make_float2(fr, -fi) : make_float2(0.f, 0.f);
     }
 }
 
@@ -314,6 +426,7 @@ namespace {
 // The 3D table: mu_l on the host, then per group of radial nodes the coefficient rows and the
 // table entries.  A group's rows take at most kCoefBytes (at least one node).
 constexpr size_t kCoefBytes = (size_t)64 << 20;
+constexpr int kFfSeries = 160;
 
 bz_status table3(Plan &pl, TableArgs a) {
     const int N = pl.N, nkk = 3 * (N / 2) * (N / 2) + 1;
@@ -327,7 +440,9 @@ bz_status table3(Plan &pl, TableArgs a) {
     const double zmax = M_PI * rmax * std::sqrt((double)(nkk - 1)) / (2.0 * pl.L);
     int lmax = 1;
     for (double lb = 0.0; !(lmax > zmax && lb < -50.7); ++lmax) lb += std::log(zmax) - std::log(2.0 * lmax + 3.0);
-    const int stride = (lmax + 4) & ~1;
+    // the double-float form up to l = kFfSeries: every plan whose R is within the box (N = 64: about 140)
+    const bool dblf = lmax <= kFfSeries;
+    const int stride = ((lmax + 4) & ~1) + (dblf ? kRowHead : 0);
     // mu'_l = 2 pi sum_n W_n (P_l(cos t_n) - 1) times (2l + 1), the sign of (-i)^l (the sum over odd l
     // is the imaginary part) and P_l / q_l; D_l = P_l - 1 by its own recurrence (no cancellation at
     // small angles), on the rule with the most nodes
@@ -360,20 +475,45 @@ bz_status table3(Plan &pl, TableArgs a) {
     const size_t gsm = (size_t)stride * sizeof(double);
     if (gsm > 48 * 1024)
         BZ_CUDA_TRY(cudaFuncSetAttribute(ftable_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm));
-    double *buf = nullptr;                                 // coefficient rows, r, mu, row lengths
-    const size_t head = r.size() + mu.size();
-    if (cudaMalloc(&buf, ni * row + head * sizeof(double) + (size_t)ni * nkk * sizeof(int)) != cudaSuccess) {
+    // one upload: r, mu, g_l and, for the double-float form, 1 / |k| and the terms as (hi, lo)
+    auto pair = [](double v) {
+        const float f[2] = {(float)v, (float)(v - (double)(float)v)};
+        double d;
+        std::memcpy(&d, f, sizeof(d));
+        return d;
+    };
+    std::vector<double> up(r);
+    up.insert(up.end(), mu.begin(), mu.end());
+    const size_t at_g = up.size();
+    for (int t = 0; t < stride; ++t) {
+        const double g = 4.0 * t * t / (4.0 * t * t - 1.0);
+        up.push_back(dblf ? pair(g) : g);
+    }
+    const size_t at_rk = up.size(), at_tq = at_rk + (dblf ? nkk : 0);
+    if (dblf) {
+        for (int m = 0; m < nkk; ++m) up.push_back(pair(m ? 1.0 / std::sqrt((double)m) : 0.0));
+        for (int p = 0; p < pl.P; ++p) {
+            for (int d = 0; d < 3; ++d) up.push_back(pair(pl.terms.q[3 * (size_t)p + d]));
+            up.push_back(pair(pl.terms.c[p] * a.inv_n3));
+        }
+    }
+    const size_t head = (up.size() + 1) & ~(size_t)1;      // (the phases are 16-byte values)
+    const size_t phases = dblf ? (size_t)pl.P * 3 * N * sizeof(float4) : 0;
+    double *buf = nullptr;                                 // coefficient rows, the upload, phases, row lengths
+    if (cudaMalloc(&buf, ni * row + head * sizeof(double) + phases + (size_t)ni * nkk * sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
         return BZ_ERR_OOM;
     }
     double *coef = buf, *r_dev = coef + ni * row / sizeof(double), *mu_dev = r_dev + r.size();
-    int *cut = (int *)(mu_dev + mu.size());
-    cudaError_t e = cudaMemcpy(r_dev, r.data(), r.size() * sizeof(double), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(mu_dev, mu.data(), mu.size() * sizeof(double), cudaMemcpyHostToDevice);
+    float4 *ph = (float4 *)(r_dev + head);
+    int *cut = (int *)((char *)ph + phases);
+    cudaError_t e = cudaMemcpy(r_dev, up.data(), up.size() * sizeof(double), cudaMemcpyHostToDevice);
     CoefArgs ca;
     ca.nkk = nkk; ca.stride = stride; ca.lmax = lmax; ca.L = pl.L; ca.r = r_dev; ca.mu = mu_dev; ca.coef = coef;
-    ca.cut = cut;
-    a.nkk = nkk; a.stride = stride; a.coef = coef; a.cut = cut;
+    ca.cut = cut; ca.dblf = dblf; ca.A0 = a.A0; ca.A1 = a.A1; ca.A2 = a.A2;
+    a.nkk = nkk; a.stride = stride; a.coef = coef; a.cut = cut; a.g = r_dev + at_g;
+    a.rk = (const float2 *)(r_dev + at_rk); a.tq = (const float2 *)(r_dev + at_tq); a.ph = ph;
+    if (dblf) k_axis_phases<<<pl.P, 3 * N>>>(N, pl.M, pl.L, a.term, ph);
     for (int i0 = 0; e == cudaSuccess && i0 < pl.N_rho; i0 += ni) {
         const int n = pl.N_rho - i0 < ni ? pl.N_rho - i0 : ni;
         ca.i0 = a.i0 = i0;
@@ -381,7 +521,9 @@ bz_status table3(Plan &pl, TableArgs a) {
         k_legendre_coef<<<dim3((nkk + 63) / 64, n), 64>>>(ca);
         for (a.g0 = 0; a.g0 < groups; a.g0 += 65535) {
             const int ng = groups - a.g0 < 65535 ? groups - a.g0 : 65535;
-            ftable_kernel<<<dim3((N * N * N + 127) / 128, ng, n), 128, gsm>>>(a);
+            const dim3 grid((N * N * N + 127) / 128, ng, n);
+            if (dblf) ftable_ff_kernel<<<grid, 128, gsm>>>(a);
+            else ftable_kernel<<<grid, 128, gsm>>>(a);
         }
         e = cudaGetLastError();
     }

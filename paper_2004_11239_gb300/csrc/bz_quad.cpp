@@ -256,6 +256,7 @@ void build_theta_rules(Plan &pl) {
     std::vector<double> wr;
     gauss_legendre(pl.N_rho, 0.0, pl.R, rr, wr);
     pl.rules.assign(pl.N_rho, ThetaRule());
+    double last = -1.0;                                    // panel width of the node before
     for (int i = 0; i < pl.N_rho; ++i) {
         double z = M_PI * rr[i] * kmax / (2.0 * pl.L);
         double width = std::fmin(0.25, 10.0 / std::fmax(z, 1e-300));
@@ -279,6 +280,11 @@ void build_theta_rules(Plan &pl) {
             lo = stop;
         }
         ThetaRule &R = pl.rules[i];
+        if (i > 0 && width == last) {                      // the same panels as the node before
+            R = pl.rules[i - 1];
+            continue;
+        }
+        last = width;
         for (size_t e = 0; e + 1 < edges.size(); ++e) {
             double a = edges[e], b = edges[e + 1];
             for (int q = 0; q < 16; ++q) {
