@@ -144,8 +144,8 @@ typedef struct {
     int chunk_terms;  /* terms per pipeline chunk; <= 0 selects automatically          */
     int pipeline;     /* BZ_PIPE_*; BZ_ERR_UNSUPPORTED if FUSED cannot run for this N     */
     int cluster;      /* FUSED: CTAs per cluster (N=16: 1|2, 24: 2|3, 32: 4|8); <= 0 times the
-                         compiled sizes at creation and keeps the fastest (BZ_DATA_REAL at N = 32:
-                         see ctas_per_sm)                                                   */
+                         compiled sizes at creation and keeps the fastest.  N = 16 takes 1, and N = 32
+                         the one-term-per-SM kernels (k_col32, k_cube32), unless a size is given */
     int h_precision;  /* BZ_H_*                                                            */
     int conv;         /* BZ_CONV_*                                                         */
     int dim;          /* 3 (or 0): the 3D operator; 2: the 2D operator of Sec. 4.1 (i) and Sec. 5.2 on
@@ -185,9 +185,9 @@ bz_status bz_plan_info(const bz_plan *plan, int *P, size_t *alpha_bytes, size_t 
  * *tuned_ms = the timed collide that selected the cluster size.  Any pointer may be NULL. */
 bz_status bz_plan_pipeline(const bz_plan *plan, int *pipeline, int *cluster, int *clusters, float *tuned_ms);
 
-/* Name of the kernel that carries the plan's per-term work: "k_fused", "k_col32" (a
- * BZ_DATA_REAL plan at N = 32), "k_pair3" (the same on request, ctas_per_sm = 3), "k_mixed",
- * "k_collide_2d" or "chunked"; NULL for a NULL plan.  The string is static. */
+/* Name of the kernel that carries the plan's per-term work: "k_fused", "k_col32" and
+ * "k_cube32" (N = 32, BZ_DATA_REAL and complex: one term per SM), "k_pair3" (real data on
+ * request, ctas_per_sm = 3), "k_mixed", "k_collide_2d" or "chunked"; NULL for a NULL plan.  The string is static. */
 const char *bz_plan_kernel(const bz_plan *plan);
 
 /* Copies the term list to host arrays of length P (any may be NULL):

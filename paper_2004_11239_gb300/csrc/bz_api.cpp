@@ -77,11 +77,11 @@ std::vector<float2> make_twiddles(const bz::Plan &pl) {
     return tw;
 }
 
-// k_col32's plan: one CTA per SM, nothing to select.  tuned_ms is one timed collide of a zero field.
-bz_status setup_col32(bz::Plan &pl) {
+// The plans of k_col32 and k_cube32: one CTA per SM, nothing to select.  tuned_ms is one timed collide of a zero field.
+bz_status setup_one_sm(bz::Plan &pl) {
     int G = 0;
-    if (bz::col32_setup(&G) != cudaSuccess || G <= 0) return BZ_ERR_CUDA;
-    const size_t part = (size_t)G * bz::kCol32Part * sizeof(float2);
+    if ((pl.col32 ? bz::col32_setup(&G) : bz::cube32_setup(&G)) != cudaSuccess || G <= 0) return BZ_ERR_CUDA;
+    const size_t part = (size_t)G * (pl.col32 ? bz::kCol32Part : bz::modes(pl)) * sizeof(float2);
     if (dmalloc(&pl.part, part) != BZ_OK) return BZ_ERR_OOM;
     pl.use_fused = 1; pl.fused_C = 1; pl.fused_G = G;
     pl.ws_bytes += part;
@@ -265,7 +265,17 @@ bz_status create(bz_plan **out, const bz_plan_desc *d) {
             (s = dmalloc(&pl.fsym, field)) == BZ_OK)
             s = bz::col32_table(pl);
         pl.ws_bytes += 2 * field + n3 * sizeof(float);
-    } else if (s == BZ_OK && pl.real) {
+    }
+    // complex data at N = 32: k_cube32 likewise (FP32 form, h beyond FP32)
+    pl.cube32 = !pl.real && dim == 3 && N == 32 && pl.precision == BZ_PREC_FP32 && pl.h_fp64 &&
+                d->pipeline != BZ_PIPE_CHUNKED && d->cluster <= 0 && d->ctas_per_sm <= 0;
+    if (s == BZ_OK && pl.cube32) {
+        if ((s = dmalloc(&pl.acol, (size_t)pl.P * field)) == BZ_OK && (s = dmalloc(&pl.fcol, field)) == BZ_OK &&
+            (s = dmalloc(&pl.hcol, field)) == BZ_OK)
+            s = bz::cube32_table(pl);
+        pl.ws_bytes += 2 * field;
+    }
+    if (s == BZ_OK && pl.real && !pl.col32) {
         // term pairs (2q, 2q + 1) share a radial node (M even) and one pair of transforms
         const size_t ns = (size_t)3 * N * N;
         if ((s = dmalloc(&pl.apair, (size_t)(pl.P / 2) * field)) == BZ_OK &&
@@ -300,13 +310,13 @@ bz_status create(bz_plan **out, const bz_plan_desc *d) {
     if (d->pipeline != BZ_PIPE_CHUNKED && N <= 32) {
         if (dmalloc(&pl.fin64, n3 * sizeof(double2)) == BZ_OK && dmalloc(&pl.scr64, n3 * sizeof(double2)) == BZ_OK) {
             pl.ws_bytes += 2 * n3 * sizeof(double2);
-            if (pl.col32) s = setup_col32(pl);
+            if (pl.col32 || pl.cube32) s = setup_one_sm(pl);
             else if (select_fused(pl, d->cluster, d->ctas_per_sm) != BZ_OK) cudaGetLastError();
-        } else if (pl.col32) {
+        } else if (pl.col32 || pl.cube32) {
             s = BZ_ERR_OOM;
         }
     }
-    if (s != BZ_OK) {                         // k_col32's plan has no other pipeline's tables
+    if (s != BZ_OK) {                         // these plans have no other pipeline's tables
         cudaGetLastError();
         free_plan(pl);
         delete h;
@@ -383,7 +393,7 @@ bz_status bz_plan_info(const bz_plan *plan, int *P, size_t *alpha_bytes, size_t 
     size_t n3 = bz::modes(p);
     if (P) *P = p.P;
     if (alpha_bytes)
-        *alpha_bytes = ((size_t)p.P * n3 + (p.col32 ? (size_t)p.P * bz::kCol32Part : p.real ? (size_t)(p.P / 2) * (n3 + 3 * (size_t)p.N * p.N) : 0)) *
+        *alpha_bytes = ((size_t)p.P * n3 + (p.col32 ? (size_t)p.P * bz::kCol32Part : p.cube32 ? (size_t)p.P * n3 : p.real ? (size_t)(p.P / 2) * (n3 + 3 * (size_t)p.N * p.N) : 0)) *
                        sizeof(float2);
     if (workspace_bytes) *workspace_bytes = p.ws_bytes;
     return BZ_OK;
@@ -395,7 +405,7 @@ const char *bz_plan_kernel(const bz_plan *plan) {
     if (p.dim == 2) return "k_collide_2d";
     if (!p.use_fused) return "chunked";
     if (p.precision == BZ_PREC_BF16X3) return "k_mixed";
-    return p.col32 ? "k_col32" : p.pair3 ? "k_pair3" : "k_fused";
+    return p.col32 ? "k_col32" : p.cube32 ? "k_cube32" : p.pair3 ? "k_pair3" : "k_fused";
 }
 
 bz_status bz_plan_pipeline(const bz_plan *plan, int *pipeline, int *cluster, int *clusters, float *tuned_ms) {

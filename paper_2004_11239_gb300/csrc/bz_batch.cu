@@ -222,7 +222,7 @@ __device__ __forceinline__ void rk_stage_mode(size_t idx, double2 kv, double2 *f
         y = make_double2(s.x + dt / 6.0 * kv.x, s.y + dt / 6.0 * kv.y);
         f0[idx] = y;
     }
-    fin[idx] = make_float2((float)y.x, (float)y.y);
+    if (fin) fin[idx] = make_float2((float)y.x, (float)y.y);
     fin64[idx] = y;
 }
 
@@ -292,10 +292,28 @@ __device__ __forceinline__ void col_modes_of(const float2 *part, int nblk, int s
     }
 }
 
+// k_cube32's items (part [nblk][32][32][32] as [k3][k1][k2]) likewise.
+template <class Sink>
+__device__ __forceinline__ void cube_modes_of(const float2 *part, int nblk, int slot, int k1, Sink sink) {
+    constexpr int N = 32, N2 = N * N;
+    __shared__ double2 s1[N][N + 1];                      // [k3][k2]
+    const float2 *base = part + (size_t)slot * nblk * N * N2;
+    for (int e = threadIdx.x; e < N2; e += blockDim.x)
+        s1[e / N][e % N] = sum_blocks(base + (size_t)(e / N) * N2 + k1 * N + e % N, 0, nblk, N * N2, 0);
+    __syncthreads();
+    for (int e = threadIdx.x; e < N2; e += blockDim.x)
+        sink((size_t)slot * N * N2 + (size_t)k1 * N2 + e, s1[e % N][e / N]);
+}
+
+template <bool CUBE>
 __global__ void __launch_bounds__(512) k_batch_out_col(const float2 *part, int nblk, const int *slots,
                                                        const int *count_dev, void *Qhat, int dtype, int *flag) {
     if ((int)blockIdx.y >= *count_dev) return;
-    col_modes_of(part, nblk, slots[blockIdx.y], blockIdx.x, [&](size_t idx, double2 q) {
+    auto modes_of = [&](auto sink) {
+        if constexpr (CUBE) cube_modes_of(part, nblk, slots[blockIdx.y], blockIdx.x, sink);
+        else col_modes_of(part, nblk, slots[blockIdx.y], blockIdx.x, sink);
+    };
+    modes_of([&](size_t idx, double2 q) {
         if (dtype == BZ_C128) {
             ((double2 *)Qhat)[idx] = q;
             note_finite(q, flag);
@@ -307,16 +325,17 @@ __global__ void __launch_bounds__(512) k_batch_out_col(const float2 *part, int n
     });
 }
 
+template <bool CUBE>
 __global__ void __launch_bounds__(512) k_batch_rk_stage_col(const float2 *part, int nblk, const int *slots,
                                                             const int *count_dev, double2 *f0, double2 *fsum,
                                                             float2 *fin, double2 *fin64, int stage, double dt) {
     if ((int)blockIdx.y >= *count_dev) return;
-    col_modes_of(part, nblk, slots[blockIdx.y], blockIdx.x, [&](size_t idx, double2 q) {
-        rk_stage_mode(idx, q, f0, fsum, fin, fin64, stage, dt);
-    });
+    auto update = [&](size_t idx, double2 q) { rk_stage_mode(idx, q, f0, fsum, fin, fin64, stage, dt); };
+    if constexpr (CUBE) cube_modes_of(part, nblk, slots[blockIdx.y], blockIdx.x, update);
+    else col_modes_of(part, nblk, slots[blockIdx.y], blockIdx.x, update);
 }
 
-// Terms per item for k_col32: the items of a full batch run on G CTAs in waves; an item costs its
+// Terms per item for k_col32 and k_cube32: the items of a full batch run on G CTAs in waves; an item costs its
 // terms and about one more (h and the sums in, the sums out and added up).  Fewest term times.
 int col_terms(int P, int capacity, int G) {
     int best = P;
@@ -341,6 +360,7 @@ ItemArgs item_args(const bz_batch &B) {
         a.real = 1; a.fin = B.fsym; a.alpha = pl.apair; a.cpair = pl.cpair; a.part_s = B.part_s;
         if (pl.col32) a.alpha = pl.acol;             // (units are terms)
     }
+    if (pl.cube32) a.alpha = pl.acol;                // (B.fin: in the kernel's layout, from the h pass)
     return a;
 }
 
@@ -571,7 +591,7 @@ bz_status bz_batch_create(bz_batch **out, const bz_plan *plan, int capacity, int
     }
     if (upload_gsc(*B) != BZ_OK) return fail(BZ_ERR_CUDA);
     int tb = pl->real && !pl->col32 && terms_per_item > 0 ? (terms_per_item + 1) / 2 : terms_per_item;   // in units
-    if (tb <= 0 && pl->col32) tb = col_terms(pl->P, capacity, pl->fused_G);
+    if (tb <= 0 && (pl->col32 || pl->cube32)) tb = col_terms(pl->P, capacity, pl->fused_G);
     if (tb <= 0) {
         // autotune on a trial of up to 4 instances per resident cluster
         int trial = capacity < 4 * pl->fused_G ? capacity : 4 * pl->fused_G;
@@ -636,18 +656,19 @@ bz_status bz_batch_collide(bz_batch *batch, int count, const int *slots, const v
     bz_status s = stage_slots(B, count, slots, st);
     if (s != BZ_OK) return s;
     const int n3 = B.pl->N * B.pl->N * B.pl->N;
-    if (!B.pl->real)
+    const bool one_sm = B.pl->col32 || B.pl->cube32;
+    if (!B.pl->real && !B.pl->cube32)
         k_batch_load<<<grid_for(B), 256, 0, st>>>(fhat, dtype, B.slots_dev, B.count_dev, n3, B.fin);
     if (B.pl->h_fp64) {                                   // (the real-data form's inputs come from the first pass)
         s = hff_launch(B.pl->N, fhat, dtype, B.slots_dev, B.count_dev, B.capacity, B.scr64, B.h, st, B.fsym,
-                       B.pl->col32 != 0);
+                       one_sm, B.pl->cube32 ? B.fin : nullptr);
         if (s != BZ_OK) return s;
     }
     s = launch_fused(*B.pl, item_args(B), st);
     if (s != BZ_OK) return s;
-    if (B.pl->col32)
-        k_batch_out_col<<<dim3(32, B.capacity), 512, 0, st>>>(B.part, B.nblk, B.slots_dev, B.count_dev, Qhat, dtype,
-                                                             nonfinite_flag(*B.pl));
+    if (one_sm)
+        (B.pl->cube32 ? k_batch_out_col<true> : k_batch_out_col<false>)<<<dim3(32, B.capacity), 512, 0, st>>>(
+            B.part, B.nblk, B.slots_dev, B.count_dev, Qhat, dtype, nonfinite_flag(*B.pl));
     else if (B.pl->real)
         k_batch_out_real<<<grid_for(B), 256, 0, st>>>(B.part, B.part_s, B.nblk, B.slots_dev, B.count_dev, B.pl->N,
                                                      Qhat, dtype, nonfinite_flag(*B.pl));
@@ -655,7 +676,7 @@ bz_status bz_batch_collide(bz_batch *batch, int count, const int *slots, const v
         k_batch_out<<<grid_for(B), 256, 0, st>>>(B.part, B.nblk, B.slots_dev, B.count_dev, n3, Qhat, dtype,
                                                 nonfinite_flag(*B.pl));
     BZ_CUDA_TRY(cudaGetLastError());
-    B.last_launches = (B.pl->real ? 2 : 3) + (B.pl->h_fp64 ? hff_launches(B.pl->N) : 0);
+    B.last_launches = (B.pl->real || B.pl->cube32 ? 2 : 3) + (B.pl->h_fp64 ? hff_launches(B.pl->N) : 0);
     return BZ_OK;
 }
 
@@ -678,12 +699,13 @@ bz_status bz_batch_step_rk(bz_batch *batch, int count, const int *slots, void *f
         for (int stage = 1; stage <= 4 && cs == BZ_OK; ++stage) {
             if (B.pl->h_fp64)
                 cs = hff_launch(B.pl->N, B.fin64, BZ_C128, B.slots_dev, B.count_dev, B.capacity, B.scr64, B.h,
-                                B.cap_stream, B.fsym, B.pl->col32 != 0);
+                                B.cap_stream, B.fsym, B.pl->col32 || B.pl->cube32,
+                                B.pl->cube32 ? B.fin : nullptr);
             if (cs == BZ_OK) cs = launch_fused(*B.pl, item_args(B), B.cap_stream);
-            if (B.pl->col32)
-                k_batch_rk_stage_col<<<dim3(32, B.capacity), 512, 0, B.cap_stream>>>(B.part, B.nblk, B.slots_dev,
-                                                                                    B.count_dev, B.f0, B.fsum, B.fin,
-                                                                                    B.fin64, stage, dt);
+            if (B.pl->col32 || B.pl->cube32)             // (their inputs come from the h pass)
+                (B.pl->cube32 ? k_batch_rk_stage_col<true> : k_batch_rk_stage_col<false>)
+                    <<<dim3(32, B.capacity), 512, 0, B.cap_stream>>>(B.part, B.nblk, B.slots_dev, B.count_dev, B.f0,
+                                                                    B.fsum, nullptr, B.fin64, stage, dt);
             else if (B.pl->real)
                 k_batch_rk_stage_real<<<grid_for(B), 256, 0, B.cap_stream>>>(B.part, B.part_s, B.nblk, B.slots_dev,
                                                                             B.count_dev, B.pl->N, B.f0, B.fsum,

@@ -52,7 +52,7 @@ void fill(const bz::Plan &pl, Header &h) {
     h.f[F_HPREC] = pl.h_fp64 ? BZ_H_FP64 : BZ_H_FP32;
     // 2D plans have one pipeline and split-BF16 plans one cluster size: left to the plan
     h.f[F_PIPE] = pl.dim == 2 ? BZ_PIPE_AUTO : (pl.use_fused ? BZ_PIPE_FUSED : BZ_PIPE_CHUNKED);
-    h.f[F_CLUSTER] = pl.use_fused && pl.dim == 3 && pl.precision == BZ_PREC_FP32 && !pl.col32 ? pl.fused_C : 0;   // 0: k_col32
+    h.f[F_CLUSTER] = pl.use_fused && pl.dim == 3 && pl.precision == BZ_PREC_FP32 && !pl.col32 && !pl.cube32 ? pl.fused_C : 0;   // 0: one term per SM
     h.f[F_CTAS] = pl.pair3 ? 3 : 0;
     h.f[F_CHUNK] = pl.chunk;
     h.d[D_L] = pl.L;

@@ -165,6 +165,7 @@ bz_status launch_fused(const Plan &pl, const ItemArgs &a, cudaStream_t st) {
     const int N = pl.N, C = pl.fused_C;
     if (pl.precision == BZ_PREC_BF16X3) return a.real ? BZ_ERR_UNSUPPORTED : launch_mixed(pl, a, st);
     if (pl.col32) return launch_col32(pl, a, st);
+    if (pl.cube32) return launch_cube32(pl, a, st);
     if (pl.pair3 && a.real) return launch_pair3(pl, a, st);
     if (N == 8 && C == 1) return launch_sc<8, 1>(pl, a, st);
     if (N == 16 && C == 1) return launch_sc<16, 1>(pl, a, st);
@@ -192,6 +193,9 @@ bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches
     a.count = 1; a.p0 = p0; a.p1 = p1; a.M = pl.M; a.N_rho = pl.N_rho;
     int nl = 0;
     bz_status s = BZ_OK;
+    if (pl.cube32) {
+        a.fin = pl.fcol; a.alpha = pl.acol; a.hg = (const float2 *)pl.hcol;
+    }
     if (pl.real) {
         if ((p0 | p1) & 1) return BZ_ERR_ARG;
         if (!(pl.h_fp64 || pl.precision == BZ_PREC_BF16X3)) {
@@ -215,8 +219,9 @@ bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches
     if (pl.h_fp64 || pl.precision == BZ_PREC_BF16X3) {
         tm_begin(pl, st);
         s = hff_launch(pl.N, pl.src, pl.src_dtype, nullptr, nullptr, 1, pl.scr64,
-                       pl.col32 ? (float2 *)pl.hcol : pl.h, st, pl.col32 ? pl.fcol : (pl.real ? pl.fsym : nullptr),
-                       pl.col32 != 0, pl.fcopy);
+                       pl.col32 || pl.cube32 ? (float2 *)pl.hcol : pl.h, st,
+                       pl.col32 ? pl.fcol : (pl.real ? pl.fsym : nullptr), pl.col32 || pl.cube32,
+                       pl.cube32 ? pl.fcol : pl.fcopy);
         if (s != BZ_OK) return s;
         tm_end(pl, st, TK_OTHER);
         nl += hff_launches(pl.N);
@@ -239,6 +244,9 @@ bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches
     tm_begin(pl, st);
     if (pl.real) {
         s = pl.col32 ? reduce_col(pl, a.nblk, st, sink) : reduce_sym(pl, a.nblk, st, sink);   // sums of the blocks, symmetrised
+        if (s != BZ_OK) return s;
+    } else if (pl.cube32) {
+        s = reduce_cube(pl, a.nblk, st, sink);
         if (s != BZ_OK) return s;
     } else {
         reduce_parts(pl.part, a.nblk, n3, sink, st);

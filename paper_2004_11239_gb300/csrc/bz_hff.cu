@@ -49,14 +49,21 @@ struct HArgs {
     float2 *h;                 // [slots][N^3]
     float2 *fout;              // real data: the Hermitian, Nyquist-free part in FP32, or null
     float2 *fcopy;             // complex data: f in FP32, or null
-    int col;                   // k_col32's layouts: fout [k3 < 16][k1][k2], h packed floats [j3][j1][j2]
+    int col;                   // fout [k3 < 16][k1][k2] and h packed floats [j3][j1][j2] (k_col32), or fcopy [k3][k1][k2]
+                               // and h [j3][j1][j2] (k_cube32)
 };
 
 // fhat(k) of the instance, or (fout) its Hermitian part, zero where an index is N / 2, which is also
 // stored.
 template <int N> __device__ __forceinline__ ffc input(const HArgs &a, size_t vol, int k1, int k2, int k3) {
     const size_t i = vol + ((size_t)k1 * N + k2) * N + k3;
-    if (!a.fout) return load_ff(a.f, a.dtype, i, a.fcopy);
+    if (!a.fout) {
+        if (!a.col) return load_ff(a.f, a.dtype, i, a.fcopy);
+        a.fcopy[vol + ((size_t)k3 * N + k1) * N + k2] =
+            a.dtype == BZ_C128 ? make_float2((float)((const double2 *)a.f)[i].x, (float)((const double2 *)a.f)[i].y)
+                               : ((const float2 *)a.f)[i];
+        return load_ff(a.f, a.dtype, i);
+    }
     constexpr int H = N / 2;
     ffc v = {{0.f, 0.f}, {0.f, 0.f}};
     if (k1 != H && k2 != H && k3 != H) {
@@ -128,7 +135,8 @@ template <int N> __global__ void __launch_bounds__(8 * N) k_hff_line(HArgs a) {
         const float2 o = round2(v[r]);
         const float2 t = make_float2(__shfl_sync(0xffffffffu, o.x, back), __shfl_sync(0xffffffffu, o.y, back));
         const int j1 = r + R * q;
-        if (a.col) ((float *)(a.h + vol))[((size_t)u * N + j1) * N + v0] = t.x;
+        if (a.col && a.fout) ((float *)(a.h + vol))[((size_t)u * N + j1) * N + v0] = t.x;
+        else if (a.col) a.h[vol + ((size_t)u * N + j1) * N + v0] = t;
         else a.h[vol + ((size_t)j1 * N + u) * N + v0] = t;
     }
 }
@@ -211,7 +219,7 @@ cudaError_t launch8(void (*k)(P...), dim3 grid, int threads, cudaStream_t st, A.
 bz_status hff_launch(int N, const void *f, int dtype, const int *slots, const int *count_dev, int count,
                      double2 *scr, float2 *h, cudaStream_t st, float2 *fsym, bool col, float2 *fcopy) {
     if (count <= 0) return BZ_OK;
-    if ((col && N != 32) || (fsym && N == 24)) return BZ_ERR_UNSUPPORTED;
+    if ((col && (N != 32 || !(fsym || fcopy))) || (fsym && N == 24)) return BZ_ERR_UNSUPPORTED;
     HArgs a = {f, dtype, slots, count_dev, (float4 *)scr, h, fsym, fcopy, col};
     cudaError_t e = cudaSuccess;
     switch (N) {

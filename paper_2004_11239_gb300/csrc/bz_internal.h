@@ -84,9 +84,10 @@ struct Plan {
     // BZ_DATA_REAL: terms 2q and 2q + 1 share one pair of transforms
     int real = 0;
     int col32 = 0;                  // N = 32: one term per SM (k_col32): the default of the fused pipeline
-    float2 *acol = nullptr;         // its table [P][18][32][32] (bz_col32.cu)
-    float2 *fcol = nullptr;         // its input [k3 < 16][k1][k2] (N^3 allocated)
-    float *hcol = nullptr;          // its h [j3][j1][j2], packed floats
+    int cube32 = 0;                 // the same for complex data (k_cube32)
+    float2 *acol = nullptr;         // their table [P][18][32][32] (bz_col32.cu), [P][32][32][32] (bz_cube32.cu)
+    float2 *fcol = nullptr;         // input [k3 (< 16)][k1][k2] (N^3 allocated)
+    float *hcol = nullptr;          // h [j3][j1][j2], packed floats (k_cube32: float2)
     int pair3 = 0;                  // N = 32, on request: the three-CTA-per-SM pair kernel (k_pair3) instead of k_fused
     float2 *apair = nullptr;        // [P / 2][N^3] A = (alpha_2q - i alpha_2q+1) / 2
     float2 *cpair = nullptr;        // [P / 2][3][N][N] C = conj B(-k), B = (alpha_2q + i alpha_2q+1) / 2, on the
@@ -247,8 +248,9 @@ bz_status launch_fused(const Plan &pl, const ItemArgs &a, cudaStream_t st);
 // active slots (N <= 32).  Kernel launches of one hff_launch:
 inline int hff_launches(int N) { return N <= 16 ? 1 : 2; }
 // fsym (BZ_DATA_REAL, N a power of two): transform the Hermitian, Nyquist-free part of f and
-// store that part in FP32 to fsym; col (N = 32): in k_col32's layouts ([k3 < 16][k1][k2], and h as
-// packed floats [j3][j1][j2]; the same stride of N^3 float2 per slot).  scr: 16 N^3 bytes per slot
+// store that part in FP32 to fsym; col (N = 32): in the layouts of k_col32 (fsym [k3 < 16][k1][k2], h packed
+// floats [j3][j1][j2]; the same stride of N^3 float2 per slot) or, without fsym, of k_cube32 (fcopy
+// [k3][k1][k2], h [j3][j1][j2]).  fcopy (complex data): f in FP32.  scr: 16 N^3 bytes per slot
 // (N = 24, 32).
 bz_status hff_launch(int N, const void *f, int dtype, const int *slots, const int *count_dev, int count,
                      double2 *scr, float2 *h, cudaStream_t st, float2 *fsym = nullptr, bool col = false,
@@ -277,6 +279,12 @@ bz_status launch_col32(const Plan &pl, const ItemArgs &a, cudaStream_t st);
 bz_status col32_table(Plan &pl);
 bz_status col32_inputs(Plan &pl, cudaStream_t st);
 bz_status reduce_col(Plan &pl, int nblk, cudaStream_t st, const Sink &sink);
+
+// bz_cube32.cu (complex data, N = 32): as above; items' sums are N^3
+cudaError_t cube32_setup(int *G);
+bz_status launch_cube32(const Plan &pl, const ItemArgs &a, cudaStream_t st);
+bz_status cube32_table(Plan &pl);
+bz_status reduce_cube(Plan &pl, int nblk, cudaStream_t st, const Sink &sink);
 
 // bz_mixed.cu (BZ_PREC_BF16X3, N = 32)
 cudaError_t mixed_setup(int N, int *G);

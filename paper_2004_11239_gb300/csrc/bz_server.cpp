@@ -128,6 +128,12 @@ size_t plan_bytes(const bz_request &r) {
     const size_t P = (size_t)r.N_rho * r.M;
     size_t b = P * n3 * 8 + P * 3 * r.N * 8 + (size_t)(64u << 20) + 6 * n3 * 16;
     if (r.data == BZ_DATA_REAL) b += (P / 2) * (n3 * 8 + (size_t)3 * r.N * r.N * 8) + 2 * n3 * 16;
+    if (r.N == 32 && r.precision == BZ_PREC_FP32)                           // one term per SM: tables in another order
+        b += r.data == BZ_DATA_REAL ? P * 4096 : P * n3 * 8;
+    if (r.N > 32) {                                                         // running sums, Nyquist products
+        b += 6 * n3 * 16;
+        if (r.data == BZ_DATA_REAL) b += (P / 2) * 3 * r.N * r.N * 8;
+    }
     return b;
 }
 
