@@ -110,8 +110,18 @@ _PROFILES = {
     "mixed": ("mixed_rk4_n32.md", ("bz_mixed.cu", "bz_fft.cuh", "bz_cluster.cuh")),
     "fused_real": ("fused_real_rk4_n32.md", ("bz_fused_kernel.cuh", "bz_fft.cuh", "bz_cluster.cuh")),
     "pair3": ("pair3_rk4_n32.md", ("bz_pair3.cu", "bz_fft.cuh", "bz_cluster.cuh")),
+    "col32": ("one_sm_rk4_n32.md", ("bz_col32.cu", "bz_fft.cuh", "bz_tmem.cuh")),
+    "cube32": ("one_sm_complex_rk4_n32.md", ("bz_cube32.cu", "bz_fft.cuh", "bz_tmem.cuh")),
     "n64:pipeline": ("chunked_single_n64.md", ("bz_lines.cu", "bz_fft.cuh")),
 }
+
+
+_KERNEL_PROFILES = {"k_col32": "col32", "k_cube32": "cube32", "k_pair3": "pair3", "k_mixed": "mixed"}
+
+
+def _profile_key(kernel, real):
+    """The committed profile of the kernel that a plan runs."""
+    return _KERNEL_PROFILES.get(kernel, "fused_real" if real else "fused")
 
 
 def _sources_hash(files):
@@ -777,11 +787,11 @@ def run_ours(args, w):
         roof = _pipeline_roofline(w, ms / args.steps, peaks, src,
                                   "n64:pipeline" if (args.workload == "single_n64" and real) else None)
     else:
-        roof = _roofline(args, w, kern, peaks, src, "pair3" if kname == "k_pair3" else ("fused_real" if real else "fused"))
+        roof = _roofline(args, w, kern, peaks, src, _profile_key(kname, real))
     roof["kernel_name"] = kname
     if real:
-        roof["executed"] = ("term pairs share every pair of 3D transforms: about half the counted FFT "
-                            "flops and half the alpha bytes (plus a 3 N^2 Nyquist table per pair) are executed")
+        roof["executed"] = ("real data: half spectra (k_col32) or term pairs sharing their transforms: about half the "
+                            "counted FFT flops and half the alpha bytes (plus the Nyquist tables) are executed")
 
     # the other data form on the same workload (complex beside real, and the reverse where it applies)
     other = None
@@ -798,7 +808,8 @@ def run_ours(args, w):
         other = {"data_form": "complex" if real else "real", "value": vo, "unit": "evals/s",
                  "ms_per_step": mso / args.steps, "gpu_launches": lo * args.steps,
                  "rel_linf_headline_vs_this": dev,
-                 "roofline": _roofline(args, w, kerno, peaks, src, "fused" if real else "fused_real")}
+                 "roofline": _roofline(args, w, kerno, peaks, src,
+                                       _profile_key(bz.bz_plan_pipeline(po)["kernel"], not real))}
         po.close()
 
     # the same workload with h formed in FP32 too: FP64 only in the weight tables, the RK state
@@ -1302,7 +1313,7 @@ def main():
     ap.add_argument("--cluster", type=int, default=0,
                     help="CTAs per cluster of the fused kernel (0: timed at plan creation, fastest kept)")
     ap.add_argument("--ctas-per-sm", type=int, default=0, choices=[0, 2, 3],
-                    help="real-data form at N = 32: 2 runs k_fused, 3 k_pair3, 0 times both at plan creation")
+                    help="real-data form at N = 32: 2 runs k_fused, 3 k_pair3, 0 k_col32")
     ap.add_argument("--h-precision", type=int, default=0, choices=[0, 1, 2],
                     help="h = IFFT(fhat) precision on the fused path: 0 auto (FP64), 1 FP64, 2 FP32")
     args = ap.parse_args()
