@@ -59,10 +59,11 @@ template <int N, int C, bool R> static cudaError_t occupancy(int *G) {
     const void *kern;
     if constexpr (R) kern = (const void *)k_fused<N, C, false, true>;
     else kern = (const void *)k_fused<N, C, true, false>;
-    cudaError_t e;
+    cudaError_t e = cudaSuccess;
     if (C == 1) {
         int per_sm = 0, dev = 0, sms = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, K::THREADS, K::SMEM);
+        if constexpr (K::TM) per_sm = K::MIN_BLOCKS;         // (the query reports one CTA for kernels that allocate tensor memory)
+        else e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, K::THREADS, K::SMEM);
         if (e != cudaSuccess) return e;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -102,9 +103,8 @@ template <int N, int C> static cudaError_t setup_nc(int *G, bool real) {
 }
 
 // Cluster sizes compiled for each N (the plan times them and keeps the fastest).  N = 16 takes
-// one CTA unless two are asked for: a single collide takes the same time with either (8.6 us at
-// P = 192), which left the choice to chance, and batches run on the plan's size (32 instances of
-// P = 192: 108 us with one, 154 with two).
+// one CTA unless two are asked for: 7.8 us at P = 192 against 8.6 for a single collide, and for 32
+// instances of P = 192, 98 us against 154.
 int fused_candidates(int N, int *cs, int forced) {
     switch (N) {
         case 8: cs[0] = 1; return 1;
