@@ -11,6 +11,7 @@
 // its block partials, independent of the other instances in the call.  One RK4 step
 // (4 x [fused items, stage update]) is captured once per dt into a CUDA graph and replayed;
 // the active count and slot list are read from device memory at run time.
+#include <algorithm>
 #include <cmath>
 #include <map>
 #include <tuple>
@@ -591,7 +592,21 @@ bz_status bz_batch_create(bz_batch **out, const bz_plan *plan, int capacity, int
     }
     if (upload_gsc(*B) != BZ_OK) return fail(BZ_ERR_CUDA);
     int tb = pl->real && !pl->col32 && terms_per_item > 0 ? (terms_per_item + 1) / 2 : terms_per_item;   // in units
-    if (tb <= 0 && (pl->col32 || pl->cube32)) tb = col_terms(pl->P, capacity, pl->fused_G);
+    if (pl->col32 || pl->cube32) {
+        // an item of these runs on one SM where the cluster kernels took eight CTAs: a quarter of the terms
+        // asked for keeps a batch with few active slots as quick (P = 1024 real data, 100 RK4 steps of one of 32
+        // slots with 32 terms an item: 165 ms undivided, 63 so, 104 on clusters; 16 slots 584, 572, 939).  Less
+        // where a full batch would have more than 32 waves of items, whose partial sums take memory.
+        if (tb <= 0) {
+            tb = col_terms(pl->P, capacity, pl->fused_G);
+        } else {
+            int d = 4;
+            tb = (int)std::min<long long>(tb, 4LL * pl->P);
+            auto items = [&] { const int t = (tb + d - 1) / d; return (long long)capacity * ((pl->P + t - 1) / t); };
+            while (d > 1 && items() > 32LL * pl->fused_G) d /= 2;
+            tb = (tb + d - 1) / d;
+        }
+    }
     if (tb <= 0) {
         // autotune on a trial of up to 4 instances per resident cluster
         int trial = capacity < 4 * pl->fused_G ? capacity : 4 * pl->fused_G;

@@ -140,7 +140,7 @@ size_t plan_bytes(const bz_request &r) {
 size_t batch_bytes(const bz_request &r, int capacity) {
     const size_t n3 = (size_t)r.N * r.N * r.N;
     const size_t P = (size_t)r.N_rho * r.M;
-    const size_t nblk_max = (P + 15) / 16;
+    const size_t nblk_max = r.N == 32 && r.precision == BZ_PREC_FP32 ? (P + 7) / 8 : (P + 15) / 16;
     if (!fused(r)) return (size_t)capacity * n3 * 16;                       // the slots' state
     return (size_t)capacity * n3 * (8 + 8 * nblk_max + 32 + 16 + 16 + (r.data == BZ_DATA_REAL ? 8 : 0));
 }
