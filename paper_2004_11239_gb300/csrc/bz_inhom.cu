@@ -8,8 +8,9 @@
 // One CTA per (k2, k3); the array sits in shared memory between the passes, a line takes eight
 // lanes (bz_line8.cuh).  complex128 cells are computed in FP64, complex64 ones in double-float (the
 // stored result has the error of its rounding; an FP64 instruction of a warp takes 68 clocks of a
-// scheduler).  The phases are products of two tables of powers of exp(2 pi i t L / (Lx N)), 64 FP64
-// sincospi a CTA.
+// scheduler), whose exponents are those of FP32: a CTA brings its largest component near 1 by a power
+// of two first, or the sums over the lines could leave the range that the cells are in.  The phases are
+// products of two tables of powers of exp(2 pi i t L / (Lx N)), 49 FP64 sincospi a CTA.
 #include <cmath>
 
 #include "bz_internal.h"
@@ -33,19 +34,27 @@ __device__ __forceinline__ void load_c(const void *f, size_t i, ffc &v) {
 }
 __device__ __forceinline__ void store_c(void *f, size_t i, cd v) { ((double2 *)f)[i] = make_double2(v.x, v.y); }
 __device__ __forceinline__ void store_c(void *f, size_t i, ffc v) { ((float2 *)f)[i] = round2(v); }
+// The bits of the larger |component|, and x times a power of two (cd needs no scaling)
+__device__ __forceinline__ unsigned top_bits(ffc v) {
+    return max(__float_as_uint(v.x.h) & 0x7fffffffu, __float_as_uint(v.y.h) & 0x7fffffffu);
+}
+__device__ __forceinline__ cd times2(cd v, float) { return v; }
+__device__ __forceinline__ ffc times2(ffc v, float s) { return {{v.x.h * s, v.x.l * s}, {v.y.h * s, v.y.l * s}}; }
 __device__ __forceinline__ void from_d(double2 u, cd &v) { v = {u.x, u.y}; }
 __device__ __forceinline__ void from_d(double2 u, ffc &v) { v = {split(u.x), split(u.y)}; }
 __device__ __forceinline__ cd times(cd v, double s) { return scale(v, s); }
 __device__ __forceinline__ ffc times(ffc v, double s) { return scale(v, split(s)); }
 
 // Threads: 8 lanes a line, max(N, NX) lines.  C = cd (complex128 cells) or ffc (complex64).
-// Bound by FP64 issue (cd) or by latency (ffc).  N = 16, 32 cells of complex64: 9.0 us; one line a
-// thread in FP64 with a sincospi per value took 63.
+// Bound by FP64 issue (cd) or by latency (ffc).  N = 16, 32 cells of complex64: 11 us (10 without the scaling);
+// one line a thread in FP64 with a sincospi per value took 65.
 template <int N, int NX, class C>
 __global__ void __launch_bounds__(8 * (N > NX ? N : NX)) k_transport(void *f, double tau) {
-    constexpr int R = N / 8, RX = NX / 8;
+    constexpr int R = N / 8, RX = NX / 8, WARPS = (N > NX ? N : NX) / 4;
+    constexpr bool SCALE = std::is_same<C, ffc>::value;
     __shared__ C s[NX][N + 1];
     __shared__ Phases ph;
+    __shared__ unsigned s_top[WARPS];
     const size_t n3 = (size_t)N * N * N;
     const size_t at = blockIdx.x;                            // k2 N + k3
     const int tid = threadIdx.x, line = tid / 8;
@@ -65,6 +74,24 @@ __global__ void __launch_bounds__(8 * (N > NX ? N : NX)) k_transport(void *f, do
             load_c(f, (X.l + 8 * m) * n3 + (size_t)line * N * N + at, x[m]);
             x[m] = conj(x[m]);                               // forward by the inverse: conj, transform, conj
         }
+    }
+    float up = 1.f;                                          // 2^e and 2^-e of the array's largest component
+    if constexpr (SCALE) {
+        unsigned top = 0;
+        #pragma unroll
+        for (int m = 0; m < RX; ++m) top = max(top, col ? top_bits(x[m]) : 0u);
+        top = __reduce_max_sync(0xffffffffu, top);
+        if ((tid & 31) == 0) s_top[tid >> 5] = top;
+        __syncthreads();
+        #pragma unroll
+        for (int w = 0; w < WARPS; ++w) top = max(top, s_top[w]);
+        const unsigned e = min(max(top >> 23, 1u), 253u);    // both powers stay normal
+        up = __uint_as_float(e << 23);
+        const float down = __uint_as_float((254u - e) << 23);
+        #pragma unroll
+        for (int m = 0; m < RX; ++m) x[m] = times2(x[m], down);
+    }
+    if (col) {
         X(x);                                                // cells -> x-modes kappa
         #pragma unroll
         for (int r = 0; r < RX; ++r) s[r + RX * X.q][line] = conj(x[r]);
@@ -112,7 +139,7 @@ __global__ void __launch_bounds__(8 * (N > NX ? N : NX)) k_transport(void *f, do
         for (int m = 0; m < RX; ++m) x[m] = s[X.l + 8 * m][line];
         X(x);                                                // x-modes -> cells
         #pragma unroll
-        for (int r = 0; r < RX; ++r) store_c(f, (r + RX * X.q) * n3 + (size_t)line * N * N + at, x[r]);
+        for (int r = 0; r < RX; ++r) store_c(f, (r + RX * X.q) * n3 + (size_t)line * N * N + at, times2(x[r], up));
     }
 }
 
