@@ -6,7 +6,7 @@
 // f(v_1j) = sum_k1 (-1)^k1 fhat(k1) exp(2 pi i k1 j / N) (the factor (-1)^k1 = exp(-i pi k1)
 // from the grid origin -L), multiplied by exp(-2 pi i kappa v_1j t / Lx), and transformed back.
 // One CTA per (k2, k3); the array sits in shared memory between the passes, a line takes eight
-// lanes (bz_line8.cuh).  complex128 cells are computed in FP64, complex64 ones in double-float (the
+// lanes (bz_line8.cuh) or, in FP64 from N = 24 and 16 cells on, one thread.  complex128 cells are computed in FP64, complex64 ones in double-float (the
 // stored result has the error of its rounding; an FP64 instruction of a warp takes 68 clocks of a
 // scheduler), whose exponents are those of FP32: a CTA brings its largest component near 1 by a power
 // of two first, or the sums over the lines could leave the range that the cells are in.  The phases are
@@ -45,6 +45,16 @@ __device__ __forceinline__ void from_d(double2 u, ffc &v) { v = {split(u.x), spl
 __device__ __forceinline__ cd times(cd v, double s) { return scale(v, s); }
 __device__ __forceinline__ ffc times(ffc v, double s) { return scale(v, split(s)); }
 
+__device__ __forceinline__ void load_phases(Phases &ph, double tau) {
+    for (int e = threadIdx.x; e < 49; e += blockDim.x) {
+        const int m = e < 32 ? e : 32 * (e - 32);
+        double sn, cs;
+        sincospi(2.0 * tau * m, &sn, &cs);
+        if (e < 32) ph.b[e] = make_double2(cs, sn);
+        else ph.a[e - 32] = make_double2(cs, sn);
+    }
+}
+
 // Threads: 8 lanes a line, max(N, NX) lines.  C = cd (complex128 cells) or ffc (complex64).
 // Bound by FP64 issue (cd) or by latency (ffc).  N = 16, 32 cells of complex64: 11 us (10 without the scaling);
 // one line a thread in FP64 with a sincospi per value took 65.
@@ -58,13 +68,7 @@ __global__ void __launch_bounds__(8 * (N > NX ? N : NX)) k_transport(void *f, do
     const size_t n3 = (size_t)N * N * N;
     const size_t at = blockIdx.x;                            // k2 N + k3
     const int tid = threadIdx.x, line = tid / 8;
-    if (tid < 49) {
-        const int m = tid < 32 ? tid : 32 * (tid - 32);
-        double sn, cs;
-        sincospi(2.0 * tau * m, &sn, &cs);
-        if (tid < 32) ph.b[tid] = make_double2(cs, sn);
-        else ph.a[tid - 32] = make_double2(cs, sn);
-    }
+    load_phases(ph, tau);
     const LineFF<NX, C> X(tid & 7);
     const bool col = line < N;                               // whole warps: N and NX are multiples of 4
     C x[RX];
@@ -143,11 +147,64 @@ __global__ void __launch_bounds__(8 * (N > NX ? N : NX)) k_transport(void *f, do
     }
 }
 
+// The same with a whole line to a thread, complex128 cells: fewer FP64 operations (a 32-point line takes about 13 a
+// point, 17 over eight lanes), which bound the longer lines; the short ones are latency.  us with a line over
+// eight lanes / to a thread: N = 32: 58 / 90 (8 cells), 116 / 105 (16), 179 / 127 (24), 235 / 143 (32);
+// N = 24: 27 / 43, 52 / 51, 78 / 64, 103 / 74; N = 16, 32 cells: 35 / 49.
+template <int N, int NX>
+__global__ void __launch_bounds__(N > NX ? N : NX) k_transport_line(double2 *f, double tau) {
+    __shared__ double2 s[NX][N + 1];
+    __shared__ Phases ph;
+    const size_t n3 = (size_t)N * N * N, at = blockIdx.x;    // at: k2 N + k3
+    const int tid = threadIdx.x;
+    load_phases(ph, tau);
+    if (tid < N) {                                           // column k1 = tid over the cells
+        double2 x[NX];
+        #pragma unroll
+        for (int c = 0; c < NX; ++c) x[c] = f[c * n3 + (size_t)tid * N * N + at];
+        fft_inplace<NX, -1>(x);                              // cells -> x-modes kappa
+        #pragma unroll
+        for (int c = 0; c < NX; ++c) s[c][tid] = x[c];
+    }
+    __syncthreads();
+    if (tid < NX) {                                          // x-mode row over k1
+        double2 y[N];
+        #pragma unroll
+        for (int i = 0; i < N; ++i) y[i] = i & 1 ? cneg(s[tid][i]) : s[tid][i];
+        fft_inplace<N, +1>(y);                               // k1 -> node values
+        const int kappa = tid < NX / 2 ? tid : tid - NX;
+        #pragma unroll
+        for (int j = 0; j < N; ++j) {
+            const int m = kappa * (N - 2 * j), am = m < 0 ? -m : m;
+            double2 w = cmul(ph.a[am >> 5], ph.b[am & 31]);
+            if (m < 0) w.y = -w.y;
+            y[j] = cmul(y[j], w);
+        }
+        fft_inplace<N, -1>(y);                               // node values -> k1
+        const double inv = 1.0 / ((double)N * NX);           // both inverse normalisations
+        #pragma unroll
+        for (int i = 0; i < N; ++i) s[tid][i] = cscale(y[i], i & 1 ? -inv : inv);
+    }
+    __syncthreads();
+    if (tid < N) {
+        double2 x[NX];
+        #pragma unroll
+        for (int c = 0; c < NX; ++c) x[c] = s[c][tid];
+        fft_inplace<NX, +1>(x);                              // x-modes -> cells
+        #pragma unroll
+        for (int c = 0; c < NX; ++c) f[c * n3 + (size_t)tid * N * N + at] = x[c];
+    }
+}
+
 template <int N, int NX> bz_status run(void *f, int dtype, double L, double Lx, double t, cudaStream_t st) {
     const double tau = t * L / (Lx * N);
     constexpr int threads = 8 * (N > NX ? N : NX);
-    if (dtype == BZ_C128) k_transport<N, NX, cd><<<N * N, threads, 0, st>>>(f, tau);
-    else k_transport<N, NX, ffc><<<N * N, threads, 0, st>>>(f, tau);
+    if constexpr (N >= 24 && NX >= 16) {
+        if (dtype == BZ_C128) k_transport_line<N, NX><<<N * N, N > NX ? N : NX, 0, st>>>((double2 *)f, tau);
+    } else {
+        if (dtype == BZ_C128) k_transport<N, NX, cd><<<N * N, threads, 0, st>>>(f, tau);
+    }
+    if (dtype == BZ_C64) k_transport<N, NX, ffc><<<N * N, threads, 0, st>>>(f, tau);
     BZ_CUDA_TRY(cudaGetLastError());
     return BZ_OK;
 }
