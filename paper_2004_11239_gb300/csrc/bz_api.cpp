@@ -84,6 +84,11 @@ bz_status setup_one_sm(bz::Plan &pl) {
     const size_t part = (size_t)G * (pl.col32 ? bz::kCol32Part : bz::modes(pl)) * sizeof(float2);
     if (dmalloc(&pl.part, part) != BZ_OK) return BZ_ERR_OOM;
     pl.use_fused = 1; pl.fused_C = 1; pl.fused_G = G;
+    // (the clusters' sums go where the items' do, which are more)
+    if (pl.cube32 && (bz::fused_setup(32, 8, &pl.few_G, false) != cudaSuccess || pl.few_G > G)) {
+        cudaGetLastError();
+        pl.few_G = 0;
+    }
     pl.ws_bytes += part;
     pl.f32 = pl.fin;
     pl.src = pl.fin;

@@ -558,7 +558,7 @@ static bz_status load_input(Plan &pl, const void *fhat, int dtype, cudaStream_t 
     }
     pl.src = fhat;
     pl.src_dtype = dtype;
-    if (pl.real || pl.cube32) return BZ_OK;               // (the h pass lays k_cube32's input out)
+    if (pl.real) return BZ_OK;
     if (dtype == BZ_C64) {
         pl.f32 = (const float2 *)fhat;
     } else if (pl.dim == 2 || (pl.use_fused && (pl.h_fp64 || pl.precision == BZ_PREC_BF16X3))) {

@@ -129,9 +129,8 @@ cudaError_t fused_setup(int N, int C, int *G, bool real) {
     return cudaErrorInvalidValue;
 }
 
-template <int N, int C, bool SC, bool R> static bz_status launch_nc(const Plan &pl, const ItemArgs &a, cudaStream_t st) {
+template <int N, int C, bool SC, bool R> static bz_status launch_nc(int G, const ItemArgs &a, cudaStream_t st) {
     using K = FK<N, C, R>;
-    const int G = pl.fused_G;
     if (C == 1) {
         k_fused<N, C, SC, R><<<G, K::THREADS, K::SMEM, st>>>(a);
     } else {
@@ -153,12 +152,12 @@ template <int N, int C, bool SC, bool R> static bz_status launch_nc(const Plan &
     return BZ_OK;
 }
 
-template <int N, int C> static bz_status launch_sc(const Plan &pl, const ItemArgs &a, cudaStream_t st) {
+template <int N, int C> static bz_status launch_sc(int G, const ItemArgs &a, cudaStream_t st) {
     if (a.real) {
-        if constexpr (pair_form<N>()) return a.gsc ? launch_nc<N, C, true, true>(pl, a, st) : launch_nc<N, C, false, true>(pl, a, st);
+        if constexpr (pair_form<N>()) return a.gsc ? launch_nc<N, C, true, true>(G, a, st) : launch_nc<N, C, false, true>(G, a, st);
         else return BZ_ERR_UNSUPPORTED;
     }
-    return a.gsc ? launch_nc<N, C, true, false>(pl, a, st) : launch_nc<N, C, false, false>(pl, a, st);
+    return a.gsc ? launch_nc<N, C, true, false>(G, a, st) : launch_nc<N, C, false, false>(G, a, st);
 }
 
 bz_status launch_fused(const Plan &pl, const ItemArgs &a, cudaStream_t st) {
@@ -167,13 +166,13 @@ bz_status launch_fused(const Plan &pl, const ItemArgs &a, cudaStream_t st) {
     if (pl.col32) return launch_col32(pl, a, st);
     if (pl.cube32) return launch_cube32(pl, a, st);
     if (pl.pair3 && a.real) return launch_pair3(pl, a, st);
-    if (N == 8 && C == 1) return launch_sc<8, 1>(pl, a, st);
-    if (N == 16 && C == 1) return launch_sc<16, 1>(pl, a, st);
-    if (N == 16 && C == 2) return launch_sc<16, 2>(pl, a, st);
-    if (N == 24 && C == 2) return launch_sc<24, 2>(pl, a, st);
-    if (N == 24 && C == 3) return launch_sc<24, 3>(pl, a, st);
-    if (N == 32 && C == 4) return launch_sc<32, 4>(pl, a, st);
-    if (N == 32 && C == 8) return launch_sc<32, 8>(pl, a, st);
+    if (N == 8 && C == 1) return launch_sc<8, 1>(pl.fused_G, a, st);
+    if (N == 16 && C == 1) return launch_sc<16, 1>(pl.fused_G, a, st);
+    if (N == 16 && C == 2) return launch_sc<16, 2>(pl.fused_G, a, st);
+    if (N == 24 && C == 2) return launch_sc<24, 2>(pl.fused_G, a, st);
+    if (N == 24 && C == 3) return launch_sc<24, 3>(pl.fused_G, a, st);
+    if (N == 32 && C == 4) return launch_sc<32, 4>(pl.fused_G, a, st);
+    if (N == 32 && C == 8) return launch_sc<32, 8>(pl.fused_G, a, st);
     return BZ_ERR_UNSUPPORTED;
 }
 
@@ -181,6 +180,11 @@ bz_status launch_fused(const Plan &pl, const ItemArgs &a, cudaStream_t st) {
 void reduce_parts(const float2 *part, int nblk, int n, const Sink &sink, cudaStream_t st) {
     k_reduce_parts<<<(n + 31) / 32, 256, 0, st>>>(part, nblk, n, sink);
 }
+
+// Whether a k_cube32 plan runs n terms of one instance on k_fused's 8-CTA clusters: in one or two rounds of them
+// (8.6 us each) they take less than k_cube32 for a term on each SM (23 us).  Measured, a whole collide, k_cube32 /
+// clusters: n = 8 48 / 31 us, 36 49 / 35, 72 49 / 45, 73 49 / 53.
+static bool few_terms(const Plan &pl, int n) { return pl.cube32 && n > 0 && n <= 2 * pl.few_G; }
 
 // One instance (pl.f32), terms [p0, p1): one block of terms per resident cluster, then the
 // fixed-order sum of the blocks into the sink.  BZ_DATA_REAL: the input is first reduced to
@@ -193,7 +197,8 @@ bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches
     a.count = 1; a.p0 = p0; a.p1 = p1; a.M = pl.M; a.N_rho = pl.N_rho;
     int nl = 0;
     bz_status s = BZ_OK;
-    if (pl.cube32) {
+    const bool few = few_terms(pl, p1 - p0), cube = pl.cube32 && !few;
+    if (cube) {
         a.fin = pl.fcol; a.alpha = pl.acol; a.hg = (const float2 *)pl.hcol;
     }
     if (pl.real) {
@@ -213,15 +218,15 @@ bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches
             a.p0 = p0; a.p1 = p1;                         // one term at a time
         }
     }
-    const int nt = a.p1 - a.p0;
-    a.TB = nt > 0 ? (nt + pl.fused_G - 1) / pl.fused_G : 1;
+    const int nt = a.p1 - a.p0, G = few ? pl.few_G : pl.fused_G;
+    a.TB = nt > 0 ? (nt + G - 1) / G : 1;
     a.nblk = nt > 0 ? (nt + a.TB - 1) / a.TB : 0;
     if (pl.h_fp64 || pl.precision == BZ_PREC_BF16X3) {
         tm_begin(pl, st);
         s = hff_launch(pl.N, pl.src, pl.src_dtype, nullptr, nullptr, 1, pl.scr64,
-                       pl.col32 || pl.cube32 ? (float2 *)pl.hcol : pl.h, st,
-                       pl.col32 ? pl.fcol : (pl.real ? pl.fsym : nullptr), pl.col32 || pl.cube32,
-                       pl.cube32 ? pl.fcol : pl.fcopy);
+                       pl.col32 || cube ? (float2 *)pl.hcol : pl.h, st,
+                       pl.col32 ? pl.fcol : (pl.real ? pl.fsym : nullptr), pl.col32 || cube,
+                       cube ? pl.fcol : pl.fcopy);
         if (s != BZ_OK) return s;
         tm_end(pl, st, TK_OTHER);
         nl += hff_launches(pl.N);
@@ -238,14 +243,14 @@ bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches
         a.hg = nullptr;                                   // h formed in FP32 in the item prologue
     }
     tm_begin(pl, st);
-    s = launch_fused(pl, a, st);
+    s = few ? launch_sc<32, 8>(G, a, st) : launch_fused(pl, a, st);
     if (s != BZ_OK) return s;
     tm_end(pl, st, TK_FUSED);
     tm_begin(pl, st);
     if (pl.real) {
         s = pl.col32 ? reduce_col(pl, a.nblk, st, sink) : reduce_sym(pl, a.nblk, st, sink);   // sums of the blocks, symmetrised
         if (s != BZ_OK) return s;
-    } else if (pl.cube32) {
+    } else if (cube) {
         s = reduce_cube(pl, a.nblk, st, sink);
         if (s != BZ_OK) return s;
     } else {

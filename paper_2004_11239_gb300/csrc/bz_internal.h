@@ -85,6 +85,7 @@ struct Plan {
     int real = 0;
     int col32 = 0;                  // N = 32: one term per SM (k_col32): the default of the fused pipeline
     int cube32 = 0;                 // the same for complex data (k_cube32)
+    int few_G = 0;                  // its 8-CTA clusters of k_fused, for collides of few terms (0: not used)
     float2 *acol = nullptr;         // their table [P][18][32][32] (bz_col32.cu), [P][32][32][32] (bz_cube32.cu)
     float2 *fcol = nullptr;         // input [k3 (< 16)][k1][k2] (N^3 allocated)
     float *hcol = nullptr;          // h [j3][j1][j2], packed floats (k_cube32: float2)
