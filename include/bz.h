@@ -330,9 +330,9 @@ bz_status bz_checkpoint_read(const bz_plan *plan, const char *path, void *fhat, 
 typedef struct bz_batch bz_batch;
 
 /* terms_per_item <= 0 autotunes the number of terms per work item (timed on the device at
- * creation).  Synchronous.  At N = 32 the kernels that run a
- * term on one SM take a quarter of the terms asked for (more in large batches; bz_batch_info tells
- * how many). */
+ * creation).  Synchronous.  At N = 32 the kernels that run a term on one SM take a quarter of the terms asked
+ * for (more in large batches), and without a figure a split that serves one active slot and a full batch
+ * by a fixed rule; bz_batch_info tells how many. */
 bz_status bz_batch_create(bz_batch **out, const bz_plan *plan, int capacity, int terms_per_item);
 void bz_batch_destroy(bz_batch *batch);
 bz_status bz_batch_info(const bz_batch *batch, int *capacity, int *terms_per_item, size_t *workspace_bytes);

@@ -336,20 +336,6 @@ __global__ void __launch_bounds__(512) k_batch_rk_stage_col(const float2 *part, 
     else col_modes_of(part, nblk, slots[blockIdx.y], blockIdx.x, update);
 }
 
-// Terms per item for k_col32 and k_cube32: the items of a full batch run on G CTAs in waves; an item costs its
-// terms and about one more (h and the sums in, the sums out and added up).  Fewest term times.
-int col_terms(int P, int capacity, int G) {
-    int best = P;
-    double cost = 1e300;
-    for (int nblk = 1; nblk <= P && nblk <= 256; ++nblk) {
-        const int tb = (P + nblk - 1) / nblk;
-        const double waves = std::ceil((double)capacity * ((P + tb - 1) / tb) / G);
-        const double c = waves * (tb + 1.0);
-        if (c < cost) { cost = c; best = tb; }
-    }
-    return best;
-}
-
 ItemArgs item_args(const bz_batch &B) {
     const Plan &pl = *B.pl;
     ItemArgs a;
@@ -449,6 +435,36 @@ int autotune_tb(bz_batch &B, int trial, cudaStream_t st) {
 using namespace bz;
 
 namespace bz {
+
+// Terms per item of a batch on k_col32 (real) or k_cube32, whose items run on one SM of G each.  No more than 32 waves
+// of items in a full batch, as their sums take memory (147 and 262 KB an item): at P = 1024 and 150 slots 32 terms.
+// asked > 0: a quarter of the terms asked for (the cluster kernels, on which a caller's figure may rest, ran
+// an item on eight CTAs), more where the bound wants it, up to what was asked.
+// Else two times are weighed.  A full batch takes its waves of items, each of its terms and `over` more (h and the
+// sums in, the sums out and added up); one active slot takes one item's terms, of which `few` cost what the
+// same slot took on clusters.  Items of twice `few` terms have to make a full batch 15% faster to be taken.
+// us for an RK4 step of one slot / of all, P = 384, real data, 32 slots: 8 terms an item 500 / 4591, 14 (taken)
+// 755 / 4204, 28 1347 / 4074, 96 4184 / 4506, on clusters 732 / 7963; 150 slots: 12 672 / 18975, 16 (taken)
+// 849 / 18451, 384 16419 / 17896, on clusters 1295 / 36308.  Complex data, 16 slots: 7 (taken) 810 / 4353, 14
+// 1419 / 4164, 43 4103 / 4195, on clusters 774 / 7855; 32 slots, P = 1024: 9 (taken) 1048 / 21632, 54 5155 / 20326,
+// on clusters 1463 / 38690.
+int one_sm_terms(bool real, int P, int capacity, int asked, int G) {
+    const int most = (int)(32LL * G / capacity), least = most > 0 ? (P + most - 1) / most : P;
+    if (asked > 0) return std::min({asked, P, std::max(asked / 4 + (asked % 4 != 0), least)});
+    const int few = real ? 14 : 10;
+    const double over = real ? 1.5 : 0.8;
+    auto full = [&](int tb) { return std::ceil((double)capacity * ((P + tb - 1) / tb) / G) * (tb + over); };
+    double lowest = 1e300, cost = 1e300;
+    for (int tb = least; tb <= P; ++tb) lowest = std::min(lowest, full(tb));
+    int best = P;
+    for (int tb = least; tb <= P; ++tb) {
+        const double c = full(tb) / lowest + 0.15 * std::max(0, tb - few) / few;
+        if (c <= cost) { cost = c; best = tb; }
+    }
+    const int nblk = (P + best - 1) / best;
+    return (P + nblk - 1) / nblk;                         // items of one size
+}
+
 namespace {
 
 bz_status check_slots(const bz_batch &B, int count, const int *slots) {
@@ -592,21 +608,7 @@ bz_status bz_batch_create(bz_batch **out, const bz_plan *plan, int capacity, int
     }
     if (upload_gsc(*B) != BZ_OK) return fail(BZ_ERR_CUDA);
     int tb = pl->real && !pl->col32 && terms_per_item > 0 ? (terms_per_item + 1) / 2 : terms_per_item;   // in units
-    if (pl->col32 || pl->cube32) {
-        // an item of these runs on one SM where the cluster kernels took eight CTAs: a quarter of the terms
-        // asked for keeps a batch with few active slots as quick (P = 1024 real data, 100 RK4 steps of one of 32
-        // slots with 32 terms an item: 165 ms undivided, 63 so, 104 on clusters; 16 slots 584, 572, 939).  Less
-        // where a full batch would have more than 32 waves of items, whose partial sums take memory.
-        if (tb <= 0) {
-            tb = col_terms(pl->P, capacity, pl->fused_G);
-        } else {
-            int d = 4;
-            tb = (int)std::min<long long>(tb, 4LL * pl->P);
-            auto items = [&] { const int t = (tb + d - 1) / d; return (long long)capacity * ((pl->P + t - 1) / t); };
-            while (d > 1 && items() > 32LL * pl->fused_G) d /= 2;
-            tb = (tb + d - 1) / d;
-        }
-    }
+    if (pl->col32 || pl->cube32) tb = one_sm_terms(pl->real, pl->P, capacity, terms_per_item, pl->fused_G);
     if (tb <= 0) {
         // autotune on a trial of up to 4 instances per resident cluster
         int trial = capacity < 4 * pl->fused_G ? capacity : 4 * pl->fused_G;
@@ -654,10 +656,12 @@ bz_status bz_batch_set_gamma(bz_batch *batch, int slot, double gamma) {
 bz_status bz_batch_info(const bz_batch *batch, int *capacity, int *terms_per_item, size_t *workspace_bytes) {
     if (!batch) return BZ_ERR_ARG;
     const size_t n3 = (size_t)batch->pl->N * batch->pl->N * batch->pl->N;
+    const size_t part = batch->pl->col32 ? kCol32Part : n3;
     if (capacity) *capacity = batch->capacity;
     if (terms_per_item) *terms_per_item = batch->TB * (batch->pl->real && !batch->pl->col32 ? 2 : 1);
     if (workspace_bytes)
-        *workspace_bytes = (size_t)batch->capacity * n3 * (sizeof(float2) * (1 + batch->nblk) + 2 * sizeof(double2));
+        *workspace_bytes = (size_t)batch->capacity * (n3 * (sizeof(float2) + 2 * sizeof(double2)) +
+                                                      part * sizeof(float2) * batch->nblk);
     return BZ_OK;
 }
 

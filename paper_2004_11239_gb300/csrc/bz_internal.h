@@ -281,6 +281,9 @@ bz_status col32_table(Plan &pl);
 bz_status col32_inputs(Plan &pl, cudaStream_t st);
 bz_status reduce_col(Plan &pl, int nblk, cudaStream_t st, const Sink &sink);
 
+// bz_batch.cu: terms per item of a batch of one-term-per-SM items; asked <= 0: chosen
+int one_sm_terms(bool real, int P, int capacity, int asked, int G);
+
 // bz_cube32.cu (complex data, N = 32): as above; items' sums are N^3
 cudaError_t cube32_setup(int *G);
 bz_status launch_cube32(const Plan &pl, const ItemArgs &a, cudaStream_t st);

@@ -98,6 +98,7 @@ struct Group {
 
 struct bz_server {
     int device = 0;
+    int sms = 0;
     size_t budget = 0, used = 0;
     int max_batch = 64;
     int terms_per_item = 0;
@@ -137,12 +138,25 @@ size_t plan_bytes(const bz_request &r) {
     return b;
 }
 
-size_t batch_bytes(const bz_request &r, int capacity) {
+// The partial sums as bz_batch_create splits them; where it times the split, its finest one (16 terms or pairs an item).
+size_t batch_bytes(const bz_server *S, const bz_request &r, int capacity) {
     const size_t n3 = (size_t)r.N * r.N * r.N;
-    const size_t P = (size_t)r.N_rho * r.M;
-    const size_t nblk_max = r.N == 32 && r.precision == BZ_PREC_FP32 ? (P + 7) / 8 : (P + 15) / 16;
+    const int P = r.N_rho * r.M;
     if (!fused(r)) return (size_t)capacity * n3 * 16;                       // the slots' state
-    return (size_t)capacity * n3 * (8 + 8 * nblk_max + 32 + 16 + 16 + (r.data == BZ_DATA_REAL ? 8 : 0));
+    const bool real = r.data == BZ_DATA_REAL;
+    int units = P, tb = S->terms_per_item > 0 ? S->terms_per_item : 16;
+    size_t item = n3 * 8;
+    if (r.N == 32 && r.precision == BZ_PREC_FP32) {                         // one term per SM
+        tb = bz::one_sm_terms(real, P, capacity, S->terms_per_item, S->sms);
+        if (real) item = bz::kCol32Part * 8;
+    } else if (real) {
+        units = P / 2;
+        if (S->terms_per_item > 0) tb = (tb + 1) / 2;
+        item += (size_t)3 * r.N * r.N * 8;
+    }
+    const size_t nblk = ((size_t)units + tb - 1) / tb;
+    // fin, f0 and fsum, fin64, scr64, h, the served state (, fsym)
+    return (size_t)capacity * (n3 * (8 + 32 + 16 + 16 + 8 + 16 + (real ? 8 : 0)) + nblk * item);
 }
 
 Key key_of(const bz_request &r) {
@@ -179,7 +193,7 @@ Group *get_group(bz_server *S, const bz_request &r, int *err) {
     auto it = S->groups.find(k);
     if (it != S->groups.end()) return it->second.get();
     const int cap = S->max_batch;
-    const size_t need = plan_bytes(r) + batch_bytes(r, cap);
+    const size_t need = plan_bytes(r) + batch_bytes(S, r, cap);
     if (need > S->budget) { *err = BZ_ERR_OOM; return nullptr; }
     if (!make_room(S, need)) { *err = BZ_ERR_BUSY; return nullptr; }
     std::unique_ptr<Group> g(new Group());
@@ -392,6 +406,7 @@ bz_status bz_server_create(bz_server **out, size_t hbm_budget_bytes, int max_bat
     bz_server *S = new (std::nothrow) bz_server();
     if (!S) return BZ_ERR_OOM;
     cudaGetDevice(&S->device);
+    cudaDeviceGetAttribute(&S->sms, cudaDevAttrMultiProcessorCount, S->device);
     S->budget = hbm_budget_bytes;
     S->max_batch = max_batch;
     S->terms_per_item = terms_per_item;
