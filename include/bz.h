@@ -188,7 +188,7 @@ bz_status bz_plan_pipeline(const bz_plan *plan, int *pipeline, int *cluster, int
 /* Name of the kernel that carries the plan's per-term work: "k_fused", "k_col32" and
  * "k_cube32" (N = 32, BZ_DATA_REAL and complex: one term per SM), "k_pair3" (real data on
  * request, ctas_per_sm = 3), "k_mixed", "k_collide_2d" or "chunked"; NULL for a NULL plan.  The string is static.
- * A "k_cube32" plan runs single collides and RK4 steps of too few terms for one per SM (up to 72 on this part) on
+ * A "k_cube32" plan runs single collides and RK4 steps of too few terms for one per SM (up to 35 on this part) on
  * k_fused's clusters, its batches and everything larger on k_cube32. */
 const char *bz_plan_kernel(const bz_plan *plan);
 

@@ -181,10 +181,11 @@ void reduce_parts(const float2 *part, int nblk, int n, const Sink &sink, cudaStr
     k_reduce_parts<<<(n + 31) / 32, 256, 0, st>>>(part, nblk, n, sink);
 }
 
-// Whether a k_cube32 plan runs n terms of one instance on k_fused's 8-CTA clusters: in one or two rounds of them
-// (8.6 us each) they take less than k_cube32 for a term on each SM (23 us).  Measured, a whole collide, k_cube32 /
-// clusters: n = 8 48 / 31 us, 36 49 / 35, 72 49 / 45, 73 49 / 53.
-static bool few_terms(const Plan &pl, int n) { return pl.cube32 && n > 0 && n <= 2 * pl.few_G; }
+// Whether a k_cube32 plan runs n terms of one instance on k_fused's 8-CTA clusters: while there is a cluster for each,
+// they take 8.6 us where k_cube32 takes 23.  Measured, a whole collide, k_cube32 / clusters: n = 8 48 / 31 us, 32
+// 49 / 33.  (Two rounds of clusters would still win a little, 49 / 45 at n = 72, but a plan's batches are on
+// k_cube32, and a batch and a collide of the same terms then differ by the rounding of two kernels.)
+static bool few_terms(const Plan &pl, int n) { return pl.cube32 && n > 0 && n < pl.few_G; }
 
 // One instance (pl.f32), terms [p0, p1): one block of terms per resident cluster, then the
 // fixed-order sum of the blocks into the sink.  BZ_DATA_REAL: the input is first reduced to
