@@ -9,6 +9,10 @@
 // (octant-reduced), so they are FFMA constant-bank operands.
 //
 // fft_inplace<N, SIGN>(x): x[k] <- sum_j x[j] exp(SIGN 2 pi i j k / N), unnormalised.
+//
+// Radix 2 by decimation in time with fused multiply-adds takes fewer operations (388 for 32 points, 432 here) and was
+// 2 to 4% faster in the cluster kernels, but it rounds more often: collides at N = 8, 16, 24 were 2 to 17%
+// further from the exact ones (2-norm, up to 46% in the largest mode), so it is not used.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -122,8 +126,6 @@ __device__ __forceinline__ float2 cneg(float2 a) { return make_float2(-a.x, -a.y
 __device__ __forceinline__ double2 cneg(double2 a) { return make_double2(-a.x, -a.y); }
 __device__ __forceinline__ float neg_of(float a) { return -a; }
 __device__ __forceinline__ double neg_of(double a) { return -a; }
-__device__ __forceinline__ float fma_of(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double fma_of(double a, double b, double c) { return fma(a, b, c); }
 // multiply by SIGN * i
 template <int SIGN, class T> __device__ __forceinline__ T mul_i(T a) {
     T r;
@@ -216,57 +218,6 @@ template <int N, int SIGN, class T> __device__ __forceinline__ void fft_inplace(
     for (int k = 0; k < N; ++k) y[k] = x[slot_of<N>(k)];
     #pragma unroll
     for (int k = 0; k < N; ++k) x[k] = y[k];
-}
-
-// The same transform by decimation in time.  Fewer operations, but a longer chain from input to output
-// and more live registers: faster in the cluster kernels, which have registers to spare (k_fused at
-// N = 32 302 -> 290 us, N = 24 34.6 -> 33.6, N = 16 in batches 1960 -> 1918), slower in k_col32
-// (92 -> 95) and in the planes of bz_lines.cu (29 -> 44), which spill.
-// Input order of the recursion: slot i of the working array holds x[dit_source<N>(i)].
-template <int N> __host__ __device__ constexpr int dit_source(int i) {
-    if constexpr (N % 2 != 0) return i;
-    else return i < N / 2 ? 2 * dit_source<N / 2>(i) : 2 * dit_source<N / 2>(i - N / 2) + 1;
-}
-
-// b <- a - w b, a <- a + w b, w = exp(SIGN 2 pi i k / N): the sum by two fused multiply-adds a
-// component and the difference as 2 a - sum, six operations against eight for a product and two
-// additions.  (A 32-point line takes 388 FP32 operations this way; 432 by fft_inplace.)
-template <int N, int SIGN, class T> __device__ __forceinline__ void bfly_tw(T &a, T &b, int k) {
-    if (k == 0) { bfly2<SIGN>(a, b); return; }
-    if (4 * k == N) {
-        b = mul_i<SIGN>(b);
-        bfly2<SIGN>(a, b);
-        return;
-    }
-    const T w = tw_entry((const T *)nullptr, tw_off<N>() + k);
-    const auto wi = SIGN < 0 ? neg_of(w.y) : w.y;
-    T u;
-    u.x = fma_of(w.x, b.x, fma_of(-wi, b.y, a.x));
-    u.y = fma_of(w.x, b.y, fma_of(wi, b.x, a.y));
-    b.x = fma_of(a.x, 2, -u.x);
-    b.y = fma_of(a.y, 2, -u.y);
-    a = u;
-}
-
-// In-place decimation in time on x[0 .. N), inputs in dit_source order, outputs in natural order.
-template <int N, int SIGN, class T> __device__ __forceinline__ void dit(T *x) {
-    if constexpr (N == 3) {
-        bfly3<SIGN>(x[0], x[1], x[2]);
-    } else if constexpr (N > 1) {
-        dit<N / 2, SIGN>(x);
-        dit<N / 2, SIGN>(x + N / 2);
-        #pragma unroll
-        for (int k = 0; k < N / 2; ++k) bfly_tw<N, SIGN>(x[k], x[k + N / 2], k);
-    }
-}
-
-template <int N, int SIGN, class T> __device__ __forceinline__ void fft_dit(T (&x)[N]) {
-    T y[N];
-    #pragma unroll
-    for (int i = 0; i < N; ++i) y[i] = x[dit_source<N>(i)];
-    dit<N, SIGN>(y);
-    #pragma unroll
-    for (int i = 0; i < N; ++i) x[i] = y[i];
 }
 
 }  // namespace bz

@@ -41,7 +41,8 @@ template <int N, int C_, bool R_ = false> struct FK {
     // stores of 8 bytes a thread for fhat, for h, and three times for the staged weights, beside the 128
     // of the exchanges.  251 instances of P = 512, one stage: 1910 us -> 1715 (32 of P = 192: 108 -> 98);
     // with fhat read from L1 1844, with the weights staged 1845, with the sums in registers 1745.
-    // Three CTAs an SM (80 registers, h in shared memory): 1740, so it is not short of warps.
+    // Three CTAs an SM (80 registers, h in shared memory): 1740, so it is not short of warps.  (Taken with an FFT since
+    // dropped for its rounding; the one in use adds 2.8%.)
     static constexpr bool TM = N == 16 && C_ == 1;
     static constexpr int HC = R_ ? N : 2 * N;               // tensor-memory columns: h, then sums, then fhat
     static constexpr int ACC0 = HC, F0 = HC + 2 * N, COLS = F0 + 2 * N, ALLOC = 256;   // two warps share a lane
@@ -86,13 +87,13 @@ __device__ __forceinline__ void phase_a(const float2 *__restrict__ fin, const fl
         #pragma unroll
         for (int i = 0; i < N; ++i) x[i] = f[i * N + lane];
     }
-    fft_dit<N, +1>(x);                                    // k2 -> j2
+    fft_inplace<N, +1>(x);                                    // k2 -> j2
     #pragma unroll
     for (int i = 0; i < N; ++i) my[i * LD + lane] = x[i];
     __syncthreads();
     #pragma unroll
     for (int j = 0; j < N; ++j) x[j] = my[lane * LD + j];
-    fft_dit<N, +1>(x);                                    // k3 -> j3 (row j2 = lane)
+    fft_inplace<N, +1>(x);                                    // k3 -> j3 (row j2 = lane)
     #pragma unroll
     for (int j = 0; j < N; ++j) my[lane * LD + j] = x[j];
 }
@@ -113,13 +114,13 @@ __device__ __forceinline__ void phase_a_pair(const float2 *__restrict__ fin, con
         const float2 u = cmul(ta, tws[N + i]), v = cmul(tb, tws[4 * N + i]);
         x[i] = cmul(TM ? x[i] : f[i * N + lane], make_float2(u.x - v.y, u.y + v.x));       // u + i v
     }
-    fft_dit<N, +1>(x);                                    // k2 -> j2
+    fft_inplace<N, +1>(x);                                    // k2 -> j2
     #pragma unroll
     for (int i = 0; i < N; ++i) my[i * LD + lane] = x[i];
     __syncthreads();
     #pragma unroll
     for (int j = 0; j < N; ++j) x[j] = my[lane * LD + j];
-    fft_dit<N, +1>(x);                                    // k3 -> j3 (row j2 = lane)
+    fft_inplace<N, +1>(x);                                    // k3 -> j3 (row j2 = lane)
     #pragma unroll
     for (int j = 0; j < N; ++j) my[lane * LD + j] = x[j];
 }
@@ -242,7 +243,7 @@ k_fused(ItemArgs a) {
             float2 x[N];
             #pragma unroll
             for (int k = 0; k < N; ++k) x[k] = ld_pencil(k);
-            fft_dit<N, +1>(x);                            // k1 -> j1
+            fft_inplace<N, +1>(x);                            // k1 -> j1
             if constexpr (K::TM) keep_h<N, REAL>(tl, x);
             else
             #pragma unroll
@@ -313,7 +314,7 @@ k_fused(ItemArgs a) {
             float2 x[N];
             #pragma unroll
             for (int k = 0; k < N; ++k) x[k] = ld_pencil(k);
-            fft_dit<N, +1>(x);                            // k1 -> j1
+            fft_inplace<N, +1>(x);                            // k1 -> j1
             if constexpr (K::TM && REAL) {
                 float hv[16];
                 t_ld16(tl, hv);
@@ -340,7 +341,7 @@ k_fused(ItemArgs a) {
                 #pragma unroll
                 for (int j = 0; j < N; ++j) x[j] = cmul(x[j], shs[((size_t)pid * N + j) * N + lane]);
             }
-            fft_dit<N, -1>(x);                            // j1 -> k1
+            fft_inplace<N, -1>(x);                            // j1 -> k1
             #pragma unroll
             for (int k = 0; k < N; ++k) st_pencil(k, x[k]);
             float2 ar[K::TM ? N : 1];                         // TM: the weights, a phase ahead
@@ -353,14 +354,14 @@ k_fused(ItemArgs a) {
             // C: rows over j3, then column k3 = lane over j2, times alpha, accumulate
             #pragma unroll
             for (int j = 0; j < N; ++j) x[j] = my[lane * LD + j];
-            fft_dit<N, -1>(x);                            // j3 -> k3 (row j2 = lane)
+            fft_inplace<N, -1>(x);                            // j3 -> k3 (row j2 = lane)
             #pragma unroll
             for (int j = 0; j < N; ++j) my[lane * LD + j] = x[j];
             cp_async_wait_1();                                // alpha tile (the next twiddles may pend)
             __syncthreads();
             #pragma unroll
             for (int i = 0; i < N; ++i) x[i] = my[i * LD + lane];
-            fft_dit<N, -1>(x);                            // j2 -> k2
+            fft_inplace<N, -1>(x);                            // j2 -> k2
             if constexpr (K::TM) {
                 #pragma unroll
                 for (int g = 0; g < 2; ++g) {
