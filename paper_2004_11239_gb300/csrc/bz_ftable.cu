@@ -87,7 +87,7 @@ struct TableArgs {
 // largest z, or from the l where that holds for this z), normalised by sum (2l + 1) j_l^2 = 1 with
 // the sign of j_0 = sin z / z or j_1.  One thread per row.
 // Double-float form (dblf): entries as (hi, lo) float2, and ahead of them kRowHead with part I in the same
-// variables, x = z c, y^2 = z^2 (1 - c^2): w0 + w1 c^2 + i w2 c.
+// variables, x = z c, y^2 = z^2 (1 - c^2): w0 + w1 c^2 + i w2 c; and z.
 constexpr int kRowHead = 4;
 struct CoefArgs {
     int i0, ni, nkk, stride, lmax, dblf;
@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(64) k_legendre_coef(CoefArgs a) {
         w[0] = pair(-0.5 * M_PI * z * z * a.A2);
         w[1] = pair(-2.0 * M_PI * z * z * (0.5 * a.A1 - 0.25 * a.A2));
         w[2] = pair(2.0 * M_PI * z * a.A0);
-        w[3] = make_float2(0.f, 0.f);
+        w[3] = pair(z);
     }
     if (!(z > 0.0)) {                                     // k = 0: F = 0
         a.cut[row] = 0;
@@ -227,7 +227,10 @@ __global__ void __launch_bounds__(128) ftable_kernel(TableArgs a) {
     for (int u = 0; u < np; ++u) {
         const double *tp = a.term + 5 * (size_t)(p0 + u);
         const double aa = M_PI * tp[0] / (2.0 * a.L);
-        const double x = aa * kap[u], y2 = aa * aa * fmax((double)kk - kap[u] * kap[u], 0.0);
+        // x with the clamped cos chi: a point longer than 1 (a caller's rule, unit to a few digits) shifts it against
+        // the j_l(a |k|), by a phase of z times the excess
+        const double x = 0.5 * aa * c2[u] * (kk > 0 ? sqrt((double)kk) : 0.0);
+        const double y2 = aa * aa * fmax((double)kk - kap[u] * kap[u], 0.0);
         double sx, cx;
         sincos(x, &sx, &cx);
         const double sc = tp[4] * a.inv_n3;
@@ -289,11 +292,16 @@ __global__ void __launch_bounds__(128) ftable_ff_kernel(TableArgs a) {
     const int cut = in_k || in_m ? a.cut[row] : 0;
     const ff rk = ld(a.rk[kk]), zero = {0.f, 0.f};
     ff ch[kLegTerms], c2[kLegTerms], q0[kLegTerms], q1[kLegTerms], sr[kLegTerms], si[kLegTerms];
+    float over[kLegTerms];                                // cos chi beyond 1 (a point longer than 1)
     #pragma unroll
     for (int u = 0; u < kLegTerms; ++u) {
         const float2 *tq = a.tq + 4 * (size_t)(p0 + (u < np ? u : 0));
         const ff f1 = {(float)k1, 0.f}, f2 = {(float)k2, 0.f}, f3 = {(float)k3, 0.f};
         ch[u] = fmul(fadd(fdot<1>(ld(tq[0]), f1, ld(tq[1]), f2), fmul(ld(tq[2]), f3)), rk);   // cos chi
+        const float one = ch[u].h < 0.f ? -1.f : 1.f;
+        over[u] = (ch[u].h - one) + ch[u].l;
+        if (over[u] * one > 0.f) ch[u] = {one, 0.f};
+        else over[u] = 0.f;
         c2[u] = {2.f * ch[u].h, 2.f * ch[u].l};
         q0[u] = {1.f, 0.f};
         q1[u] = c2[u];
@@ -315,7 +323,12 @@ __global__ void __launch_bounds__(128) ftable_ff_kernel(TableArgs a) {
     for (int u = 0; u < kLegTerms; ++u) {
         if (u >= np) break;
         const float4 *ph = a.ph + (size_t)(p0 + u) * 3 * N;
-        const ffc e = mul(mul(unpack(ph[i1]), unpack(ph[N + i2])), unpack(ph[2 * N + i3]));
+        ffc e = mul(mul(unpack(ph[i1]), unpack(ph[N + i2])), unpack(ph[2 * N + i3]));
+        if (over[u] != 0.f) {                             // the phase of the clamped cos chi: back by z over
+            float sn, cs;
+            sincosf(rw[3].x * over[u], &sn, &cs);
+            e = mul(e, {{cs, 0.f}, {-sn, 0.f}});
+        }
         ffc F = mul(e, {sr[u], si[u]});
         F.x = fadd(F.x, fadd(w0, fmul(w1, fmul(ch[u], ch[u]))));
         F.y = fadd(F.y, fmul(w2, ch[u]));
