@@ -97,13 +97,12 @@ enum { BZ_CONV_CIRCULAR = 0, BZ_CONV_PADDED = 1 };
  * FUSED where it applies. */
 enum { BZ_PIPE_AUTO = 0, BZ_PIPE_FUSED = 1, BZ_PIPE_CHUNKED = 2 };
 
-/* Precision of h = IFFT(fhat) on the fused pipeline.  FP32 transforms leave a noise floor of
+/* Precision of h = IFFT(fhat) on the fused pipeline and in 2D.  FP32 transforms leave a noise floor of
  * about eps max|h| over the grid, which the product h g_p turns into error where g_p is large
  * and h small; forming h in extended precision (from the caller's FP64 coefficients) removes that
- * half of the rounding error, at the cost of one or two short launches per collide.  BZ_H_FP64
- * computes in double-float arithmetic (pairs of FP32, about 47 bits): the stored FP32 h has the
- * error of its rounding, as with FP64 arithmetic.  FP32 forms h inside the fused kernel.
- * AUTO = FP64. */
+ * half of the rounding error, at the cost of one or two short launches per collide.  AUTO
+ * computes in double-float arithmetic (pairs of FP32, about 47 bits), BZ_H_FP64 in FP64; the stored FP32 h
+ * has the error of its rounding either way.  BZ_H_FP32 forms h inside the fused kernel; 2D and split-BF16 plans take it as AUTO. */
 enum { BZ_H_AUTO = 0, BZ_H_FP64 = 1, BZ_H_FP32 = 2 };
 
 /* Data of the operator (Sec. 2: f is a real distribution function, so fhat is Hermitian).

@@ -179,7 +179,7 @@ template <int N> bz_status run_n(Plan &pl, int p0, int p1, cudaStream_t st, int 
     const int nt = p1 - p0, most = pl.fused_G * D::SLOTS, nslots = nt < most ? nt : most;
     const int ctas = (nslots + D::SLOTS - 1) / D::SLOTS;
     tm_begin(pl, st);
-    const bz_status hs = hff_launch_2d(N, pl.src, pl.src_dtype, pl.h, pl.fcopy, st);
+    const bz_status hs = hff_launch_2d(N, pl.h_fp64, pl.src, pl.src_dtype, pl.h, pl.fcopy, st);
     if (hs != BZ_OK) return hs;
     tm_end(pl, st, TK_OTHER);
     tm_begin(pl, st);

@@ -213,7 +213,9 @@ bz_status create(bz_plan **out, const bz_plan_desc *d) {
     if (!(d->theta0 == 0.0 || (d->theta0 >= pl.eps && d->theta0 < M_PI))) { delete h; return BZ_ERR_ARG; }
     pl.theta0 = d->theta0;
     if (d->h_precision < BZ_H_AUTO || d->h_precision > BZ_H_FP32) { delete h; return BZ_ERR_ARG; }
-    pl.h_fp64 = d->h_precision != BZ_H_FP32 || d->precision == BZ_PREC_BF16X3;   // BF16X3 reads h formed in FP64
+    pl.h_fp64 = d->h_precision == BZ_H_FP64 ? bz::HFF_FP64
+                : d->h_precision == BZ_H_AUTO || d->precision == BZ_PREC_BF16X3 ? bz::HFF_PAIRS   // (BF16X3 reads an h beyond FP32)
+                : bz::HFF_FP32;
     cudaGetDevice(&pl.device);
     bz_status s = bz::build_terms(pl, d->sphere_xyz, d->sphere_w);
     if (s == BZ_OK) s = bz::build_kernel_constants(pl);

@@ -679,7 +679,7 @@ bz_status bz_batch_collide(bz_batch *batch, int count, const int *slots, const v
     if (!B.pl->real && !B.pl->cube32)
         k_batch_load<<<grid_for(B), 256, 0, st>>>(fhat, dtype, B.slots_dev, B.count_dev, n3, B.fin);
     if (B.pl->h_fp64) {                                   // (the real-data form's inputs come from the first pass)
-        s = hff_launch(B.pl->N, fhat, dtype, B.slots_dev, B.count_dev, B.capacity, B.scr64, B.h, st, B.fsym,
+        s = hff_launch(B.pl->N, B.pl->h_fp64, fhat, dtype, B.slots_dev, B.count_dev, B.capacity, B.scr64, B.h, st, B.fsym,
                        one_sm, B.pl->cube32 ? B.fin : nullptr);
         if (s != BZ_OK) return s;
     }
@@ -717,7 +717,7 @@ bz_status bz_batch_step_rk(bz_batch *batch, int count, const int *slots, void *f
         bz_status cs = BZ_OK;
         for (int stage = 1; stage <= 4 && cs == BZ_OK; ++stage) {
             if (B.pl->h_fp64)
-                cs = hff_launch(B.pl->N, B.fin64, BZ_C128, B.slots_dev, B.count_dev, B.capacity, B.scr64, B.h,
+                cs = hff_launch(B.pl->N, B.pl->h_fp64, B.fin64, BZ_C128, B.slots_dev, B.count_dev, B.capacity, B.scr64, B.h,
                                 B.cap_stream, B.fsym, B.pl->col32 || B.pl->cube32,
                                 B.pl->cube32 ? B.fin : nullptr);
             if (cs == BZ_OK) cs = launch_fused(*B.pl, item_args(B), B.cap_stream);

@@ -49,7 +49,7 @@ void fill(const bz::Plan &pl, Header &h) {
     h.f[F_PREC] = pl.precision;
     h.f[F_DATA] = pl.real ? BZ_DATA_REAL : BZ_DATA_COMPLEX;
     h.f[F_CONV] = pl.Nin ? BZ_CONV_PADDED : BZ_CONV_CIRCULAR;
-    h.f[F_HPREC] = pl.h_fp64 ? BZ_H_FP64 : BZ_H_FP32;
+    h.f[F_HPREC] = pl.h_fp64 == bz::HFF_FP64 ? BZ_H_FP64 : pl.h_fp64 ? BZ_H_AUTO : BZ_H_FP32;
     // 2D plans have one pipeline and split-BF16 plans one cluster size: left to the plan
     h.f[F_PIPE] = pl.dim == 2 ? BZ_PIPE_AUTO : (pl.use_fused ? BZ_PIPE_FUSED : BZ_PIPE_CHUNKED);
     h.f[F_CLUSTER] = pl.use_fused && pl.dim == 3 && pl.precision == BZ_PREC_FP32 && !pl.col32 && !pl.cube32 ? pl.fused_C : 0;   // 0: one term per SM
@@ -153,6 +153,9 @@ bz_status bz_checkpoint_read(const bz_plan *plan, const char *path, void *fhat, 
     Header h, mine;
     bool ok = read_header(fp, h);
     fill(pl, mine);
+    // (an h beyond FP32, asked for or not, was written as BZ_H_FP64 by earlier versions)
+    for (Header *p : {&h, &mine})
+        if (p->f[F_HPREC] == BZ_H_AUTO) p->f[F_HPREC] = BZ_H_FP64;
     // the same operator: every parameter of the terms and the kernel (the pipeline choices
     // may differ; they change only the rounding)
     ok = ok && std::memcmp(h.f, mine.f, sizeof(int32_t) * F_PIPE) == 0 &&

@@ -561,7 +561,7 @@ static bz_status load_input(Plan &pl, const void *fhat, int dtype, cudaStream_t 
     if (pl.real) return BZ_OK;
     if (dtype == BZ_C64) {
         pl.f32 = (const float2 *)fhat;
-    } else if (pl.dim == 2 || (pl.use_fused && (pl.h_fp64 || pl.precision == BZ_PREC_BF16X3))) {
+    } else if (pl.dim == 2 || (pl.use_fused && pl.h_fp64)) {
         pl.fcopy = pl.fin;
     } else {
         k_c128_to_c64<<<(n3 + 255) / 256, 256, 0, st>>>((const double2 *)fhat, pl.fin, n3);
@@ -664,8 +664,8 @@ bz_status run_noalloc(const Plan &pl, const void *fhat, void *Qhat, int dtype, u
         k_c128_to_c64<<<(n3 + 255) / 256, 256, 0, st>>>((const double2 *)fhat, fin, n3);
     }
     if (h64) {
-        // as bz_collide on this plan: h from the caller's coefficients in FP64, stored FP32
-        const bz_status s = hff_launch(N, fhat, dtype, nullptr, nullptr, 1, scr64, h, st);
+        // as bz_collide on this plan: h from the caller's coefficients beyond FP32, stored FP32
+        const bz_status s = hff_launch(N, pl.h_fp64, fhat, dtype, nullptr, nullptr, 1, scr64, h, st);
         if (s != BZ_OK) return s;
     } else {
         k_plane_inv<N><<<dim3(N / PPC, 1), Cfg<N>::THREADS, Cfg<N>::SMEM, st>>>(fin, pl.tw, S, 0, 0);

@@ -224,7 +224,7 @@ bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches
     a.nblk = nt > 0 ? (nt + a.TB - 1) / a.TB : 0;
     if (pl.h_fp64 || pl.precision == BZ_PREC_BF16X3) {
         tm_begin(pl, st);
-        s = hff_launch(pl.N, pl.src, pl.src_dtype, nullptr, nullptr, 1, pl.scr64,
+        s = hff_launch(pl.N, pl.h_fp64, pl.src, pl.src_dtype, nullptr, nullptr, 1, pl.scr64,
                        pl.col32 || cube ? (float2 *)pl.hcol : pl.h, st,
                        pl.col32 ? pl.fcol : (pl.real ? pl.fsym : nullptr), pl.col32 || cube,
                        cube ? pl.fcol : pl.fcopy);

@@ -74,7 +74,7 @@ struct Plan {
     int fused_C = 0;                // CTAs per cluster
     int fused_G = 0;                // resident clusters (persistent grid)
     float fused_ms = 0.f;           // timed collide of the selected cluster size
-    int h_fp64 = 1;                 // fused path: h formed in double-float (1) or in FP32 in-kernel (0)
+    int h_fp64 = 1;                 // fused path: bits of the h pass, HFF_*; HFF_FP32 in the term kernel
     double2 *fin64 = nullptr;       // [N^3] FP64 stage input (RK4) for the h pass
     double2 *scr64 = nullptr;       // [N^3] scratch of the h pass (16 bytes per mode)
     const void *src = nullptr;      // FP64-capable source of h for the next fused collide
@@ -245,19 +245,21 @@ struct ItemArgs {
 int fused_candidates(int N, int *cs, int forced);
 cudaError_t fused_setup(int N, int C, int *G, bool real);
 bz_status launch_fused(const Plan &pl, const ItemArgs &a, cudaStream_t st);
-// bz_hff.cu: h[slot] = IFFT(f[slot]) in double-float arithmetic (about 47 bits), stored FP32, for the
-// active slots (N <= 32).  Kernel launches of one hff_launch:
+// bz_hff.cu: h[slot] = IFFT(f[slot]), stored FP32, for the active slots (N <= 32); formed in double-float
+// arithmetic (HFF_PAIRS: about 47 bits), in FP64 (where BZ_H_FP64 is asked for) or in FP32 (N = 32).  Kernel
+// launches of one hff_launch:
+enum { HFF_FP32 = 0, HFF_PAIRS = 1, HFF_FP64 = 2 };
 inline int hff_launches(int N) { return N <= 16 ? 1 : 2; }
 // fsym (BZ_DATA_REAL, N a power of two): transform the Hermitian, Nyquist-free part of f and
 // store that part in FP32 to fsym; col (N = 32): in the layouts of k_col32 (fsym [k3 < 16][k1][k2], h packed
 // floats [j3][j1][j2]; the same stride of N^3 float2 per slot) or, without fsym, of k_cube32 (fcopy
 // [k3][k1][k2], h [j3][j1][j2]).  fcopy (complex data): f in FP32.  scr: 16 N^3 bytes per slot
 // (N = 24, 32).
-bz_status hff_launch(int N, const void *f, int dtype, const int *slots, const int *count_dev, int count,
+bz_status hff_launch(int N, int bits, const void *f, int dtype, const int *slots, const int *count_dev, int count,
                      double2 *scr, float2 *h, cudaStream_t st, float2 *fsym = nullptr, bool col = false,
                      float2 *fcopy = nullptr);
 // fcopy (complex data, c128): where f goes in FP32, or null
-bz_status hff_launch_2d(int N, const void *f, int dtype, float2 *h, float2 *fcopy, cudaStream_t st);
+bz_status hff_launch_2d(int N, int bits, const void *f, int dtype, float2 *h, float2 *fcopy, cudaStream_t st);
 bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches, const Sink &sink);
 // bz_real.cu (BZ_DATA_REAL): the pair table from alpha (after ftable_build); pl.fsym from a
 // c64 / c128 array

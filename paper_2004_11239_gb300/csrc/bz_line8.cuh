@@ -1,5 +1,5 @@
 // Transforms of N = 8 R points over 8 lanes, R points each, in double-float (ffc: pairs of FP32, about 47
-// significant bits) or FP64 (cd) arithmetic.
+// significant bits), FP64 (cd) or FP32 (cf) arithmetic.
 //
 // x[l + 8 m] in lane l -> X[r + R q] in the lane of q = bitrev(l): an R-point transform over m in
 // registers, the twiddle W_N^(l r), and an 8-point transform over the lanes (radix 2 by shuffles).
@@ -44,6 +44,7 @@ constexpr RootTableD make_rootsd() {
 static __device__ const RootTableD g_rootsd = make_rootsd();
 
 struct cd { double x, y; };
+struct cf { float x, y; };
 
 // exp(+2 pi i j / N)
 template <int N, class C> __device__ __forceinline__ C root(int j) {
@@ -52,7 +53,8 @@ template <int N, class C> __device__ __forceinline__ C root(int j) {
         return {v.x, v.y};
     } else {
         const float4 v = __ldg((const float4 *)g_roots.v + (j % N) * (192 / N));
-        return {{v.x, v.y}, {v.z, v.w}};
+        if constexpr (std::is_same<C, cf>::value) return {v.x, v.z};
+        else return {{v.x, v.y}, {v.z, v.w}};
     }
 }
 
@@ -96,9 +98,23 @@ __device__ __forceinline__ cd times_i(cd a) { return {-a.y, a.x}; }
 __device__ __forceinline__ cd half(cd a) { return {0.5 * a.x, 0.5 * a.y}; }
 __device__ __forceinline__ cd conj(cd a) { return {a.x, -a.y}; }
 __device__ __forceinline__ cd scale(cd a, double s) { return {a.x * s, a.y * s}; }
+__device__ __forceinline__ cf add(cf a, cf b) { return {a.x + b.x, a.y + b.y}; }
+__device__ __forceinline__ cf neg(cf a) { return {-a.x, -a.y}; }
+__device__ __forceinline__ cf sub(cf a, cf b) { return {a.x - b.x, a.y - b.y}; }
+__device__ __forceinline__ cf mul(cf a, cf w) { return {fmaf(a.x, w.x, -a.y * w.y), fmaf(a.x, w.y, a.y * w.x)}; }
+__device__ __forceinline__ cf times_i(cf a) { return {-a.y, a.x}; }
+__device__ __forceinline__ cf half(cf a) { return {0.5f * a.x, 0.5f * a.y}; }
+__device__ __forceinline__ cf conj(cf a) { return {a.x, -a.y}; }
+__device__ __forceinline__ cf scale(cf a, float s) { return {a.x * s, a.y * s}; }
 __device__ __forceinline__ float4 pack(ffc a) { return make_float4(a.x.h, a.x.l, a.y.h, a.y.l); }
 __device__ __forceinline__ ffc unpack(float4 v) { return {{v.x, v.y}, {v.z, v.w}}; }
 __device__ __forceinline__ float2 round2(ffc a) { return make_float2(a.x.h, a.y.h); }   // |lo| <= ulp(hi) / 2
+__device__ __forceinline__ double2 pack(cd a) { return make_double2(a.x, a.y); }
+__device__ __forceinline__ cd unpack(double2 v) { return {v.x, v.y}; }
+__device__ __forceinline__ float2 round2(cd a) { return make_float2((float)a.x, (float)a.y); }
+__device__ __forceinline__ float2 pack(cf a) { return make_float2(a.x, a.y); }
+__device__ __forceinline__ cf unpack(float2 v) { return {v.x, v.y}; }
+__device__ __forceinline__ float2 round2(cf a) { return make_float2(a.x, a.y); }
 
 // A double as hi + lo by its bits (no FP64 instruction): hi the leading 24 bits of the mantissa, lo the
 // other 29.  Below the FP32 range 0, above it and for Inf / NaN the FP32 infinity or NaN.
@@ -151,6 +167,9 @@ template <class C, int R> __device__ __forceinline__ void dft_reg(C (&v)[R]) {
 __device__ __forceinline__ ffc lane_xor(ffc a, int m) {
     return {{__shfl_xor_sync(0xffffffffu, a.x.h, m), __shfl_xor_sync(0xffffffffu, a.x.l, m)},
             {__shfl_xor_sync(0xffffffffu, a.y.h, m), __shfl_xor_sync(0xffffffffu, a.y.l, m)}};
+}
+__device__ __forceinline__ cf lane_xor(cf a, int m) {
+    return {__shfl_xor_sync(0xffffffffu, a.x, m), __shfl_xor_sync(0xffffffffu, a.y, m)};
 }
 __device__ __forceinline__ cd lane_xor(cd a, int m) {
     return {__shfl_xor_sync(0xffffffffu, a.x, m), __shfl_xor_sync(0xffffffffu, a.y, m)};

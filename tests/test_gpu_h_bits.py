@@ -1,0 +1,56 @@
+"""The arithmetic of h = IFFT(fhat): double-float by default, FP64 where BZ_H_FP64 asks for it (FP32 stores both).
+
+The default has to round as FP64 does: a stored value can differ only where some 45 bits leave its rounding open, by one
+FP32 ulp of a few values, far below 2^-24 of max |Q|; with low parts lost every value would be off by about
+1e-7 max |h|, which moves Q by some 1e-6 on data that the grid does not resolve.  And FP64 has to be FP64: a sum of
+1 + 2^-24 + 2^-52 lies above the middle between two FP32 numbers in 53 bits and on it in 47."""
+import numpy as np
+import pytest
+
+import bz_inputs as bi
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+L = 10.0
+FORMS = [(3, 8, 0), (3, 16, 0), (3, 16, 1), (3, 24, 0), (3, 32, 0), (3, 32, 1), (2, 8, 0), (2, 16, 0), (2, 32, 0), (2, 64, 0)]
+
+
+def _collides(dim, N, data, f):
+    import paper_2004_11239_gb300 as bz
+    out = []
+    for h in (bz.BZ_H_AUTO, bz.BZ_H_FP64):
+        if dim == 2:
+            plan = bz.bz_plan_create_ex(N, L, bi.R_from_L(L), 0.0, 0.0, 2, 12, kernel=bz.BZ_KERNEL_B2, dim=2, h_precision=h)
+        else:
+            plan = bz.bz_plan_create_ex(N, L, bi.R_from_L(L), 0.0, 0.5, 2, 12, data=data, h_precision=h)
+        q = torch.empty_like(f)
+        bz.bz_collide(plan, f, q)
+        out.append(q)
+        plan.close()
+    return out
+
+
+@pytest.mark.parametrize("dim,N,data", FORMS)
+@pytest.mark.parametrize("dtype", [torch.complex64, torch.complex128])
+def test_default_rounds_as_fp64(dim, N, data, dtype):
+    if dim == 3:
+        f = bi.random_mixture(N, L, seed=63)
+    else:
+        rng = np.random.default_rng(63)
+        f = (rng.standard_normal((N, N)) + 1j * rng.standard_normal((N, N))) * 10.0 ** rng.uniform(-9, 0, (N, N))
+    q, ref = _collides(dim, N, data, torch.from_numpy(f).cuda().to(dtype))
+    assert float((q - ref).abs().max() / ref.abs().max()) <= 2.0 ** -24
+
+
+@pytest.mark.parametrize("dim,N,data", FORMS)
+def test_fp64_is_fp64(dim, N, data):
+    f = np.zeros((N,) * dim, complex)
+    eps = 2.0 ** -24 + 2.0 ** -52
+    f[(0,) * dim] = 1.0
+    if data:                                   # Hermitian: the two modes add up to eps where their phase is 1
+        f[(1,) + (0,) * (dim - 1)] = f[(N - 1,) + (0,) * (dim - 1)] = eps / 2
+    else:
+        f[(1,) + (0,) * (dim - 1)] = eps
+    q, ref = _collides(dim, N, data, torch.from_numpy(f).cuda())
+    assert not torch.equal(q, ref)
