@@ -102,7 +102,8 @@ enum { BZ_PIPE_AUTO = 0, BZ_PIPE_FUSED = 1, BZ_PIPE_CHUNKED = 2 };
  * and h small; forming h in extended precision (from the caller's FP64 coefficients) removes that
  * half of the rounding error, at the cost of one or two short launches per collide.  AUTO
  * computes in double-float arithmetic (pairs of FP32, about 47 bits), BZ_H_FP64 in FP64; the stored FP32 h
- * has the error of its rounding either way.  BZ_H_FP32 forms h inside the fused kernel; 2D and split-BF16 plans take it as AUTO. */
+ * has the error of its rounding either way.  BZ_H_FP32 forms h inside the fused kernel or, at N = 32 with
+ * real data, in one pass before it; 2D and split-BF16 plans take it as AUTO. */
 enum { BZ_H_AUTO = 0, BZ_H_FP64 = 1, BZ_H_FP32 = 2 };
 
 /* Data of the operator (Sec. 2: f is a real distribution function, so fhat is Hermitian).

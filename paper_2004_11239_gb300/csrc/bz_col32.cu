@@ -310,16 +310,6 @@ __global__ void __launch_bounds__(256) k_col_table(const float2 *__restrict__ al
     }
 }
 
-// FP32 h (BZ_H_FP32): the kernel's inputs from the natural-order Hermitian part and h.
-__global__ void k_col_inputs(const float2 *__restrict__ fs, const float2 *__restrict__ h, float2 *__restrict__ fcol,
-                             float *__restrict__ hcol) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;                         // [i1][i2][i3]
-    if (e >= CN * C2) return;
-    const int i3 = e % CN, i12 = e / CN;
-    if (i3 < CW) fcol[i3 * C2 + i12] = fs[e];
-    hcol[i3 * C2 + i12] = h[e].x;
-}
-
 // Kahan-compensated FP32 sum (as the other reductions).
 struct KahanC {
     float sr = 0.f, si = 0.f, cr = 0.f, ci = 0.f;
@@ -403,12 +393,6 @@ bz_status col32_table(Plan &pl) {
     }
     BZ_CUDA_TRY(cudaGetLastError());
     BZ_CUDA_TRY(cudaDeviceSynchronize());
-    return BZ_OK;
-}
-
-bz_status col32_inputs(Plan &pl, cudaStream_t st) {
-    k_col_inputs<<<CN * C2 / 256, 256, 0, st>>>(pl.fsym, pl.h, pl.fcol, pl.hcol);
-    BZ_CUDA_TRY(cudaGetLastError());
     return BZ_OK;
 }
 

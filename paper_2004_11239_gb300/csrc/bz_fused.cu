@@ -204,7 +204,7 @@ bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches
     }
     if (pl.real) {
         if ((p0 | p1) & 1) return BZ_ERR_ARG;
-        if (!(pl.h_fp64 || pl.precision == BZ_PREC_BF16X3)) {
+        if (!pl.h_fp64 && !pl.col32) {
             // h formed in FP32 in the kernel from the symmetrised copy (the h pass writes it otherwise)
             tm_begin(pl, st);
             s = sym_input(pl, pl.src, pl.src_dtype, st);
@@ -222,7 +222,7 @@ bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches
     const int nt = a.p1 - a.p0, G = few ? pl.few_G : pl.fused_G;
     a.TB = nt > 0 ? (nt + G - 1) / G : 1;
     a.nblk = nt > 0 ? (nt + a.TB - 1) / a.TB : 0;
-    if (pl.h_fp64 || pl.precision == BZ_PREC_BF16X3) {
+    if (pl.h_fp64 || pl.col32) {
         tm_begin(pl, st);
         s = hff_launch(pl.N, pl.h_fp64, pl.src, pl.src_dtype, nullptr, nullptr, 1, pl.scr64,
                        pl.col32 || cube ? (float2 *)pl.hcol : pl.h, st,
@@ -231,15 +231,14 @@ bz_status collide_fused(Plan &pl, int p0, int p1, cudaStream_t st, int *launches
         if (s != BZ_OK) return s;
         tm_end(pl, st, TK_OTHER);
         nl += hff_launches(pl.N);
-    } else if (pl.pair3 || pl.col32) {
-        // these kernels read h: formed in FP32 from the symmetrised input by one plane pass
-        // and one pencil pass of the chunked pipeline
+    } else if (pl.pair3) {
+        // this kernel reads h: formed in FP32 from the symmetrised input by one plane pass and one pencil
+        // pass of the chunked pipeline
         tm_begin(pl, st);
         s = h_fp32(pl, pl.fsym, st);
-        if (s == BZ_OK && pl.col32) s = col32_inputs(pl, st);
         if (s != BZ_OK) return s;
         tm_end(pl, st, TK_OTHER);
-        nl += pl.col32 ? 3 : 2;
+        nl += 2;
     } else {
         a.hg = nullptr;                                   // h formed in FP32 in the item prologue
     }

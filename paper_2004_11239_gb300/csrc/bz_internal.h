@@ -74,7 +74,7 @@ struct Plan {
     int fused_C = 0;                // CTAs per cluster
     int fused_G = 0;                // resident clusters (persistent grid)
     float fused_ms = 0.f;           // timed collide of the selected cluster size
-    int h_fp64 = 1;                 // fused path: bits of the h pass, HFF_*; HFF_FP32 in the term kernel
+    int h_fp64 = 1;                 // fused path: bits of the h pass, HFF_*; HFF_FP32 in the term kernel but for k_col32
     double2 *fin64 = nullptr;       // [N^3] FP64 stage input (RK4) for the h pass
     double2 *scr64 = nullptr;       // [N^3] scratch of the h pass (16 bytes per mode)
     const void *src = nullptr;      // FP64-capable source of h for the next fused collide
@@ -274,13 +274,12 @@ bz_status sym_output(Plan &pl, cudaStream_t st, const Sink &sink);
 cudaError_t pair3_setup(int *G);
 bz_status launch_pair3(const Plan &pl, const ItemArgs &a, cudaStream_t st);
 
-// bz_col32.cu (BZ_DATA_REAL, N = 32): one CTA per SM; items count terms.  The table from pl.alpha;
-// inputs from pl.fsym and pl.h (FP32 h); sink <- the sum of nblk items
+// bz_col32.cu (BZ_DATA_REAL, N = 32): one CTA per SM; items count terms.  The table from pl.alpha; sink <- the
+// sum of nblk items
 constexpr size_t kCol32Part = (size_t)18 * 32 * 32;     // float2 per item's sums
 cudaError_t col32_setup(int *G);
 bz_status launch_col32(const Plan &pl, const ItemArgs &a, cudaStream_t st);
 bz_status col32_table(Plan &pl);
-bz_status col32_inputs(Plan &pl, cudaStream_t st);
 bz_status reduce_col(Plan &pl, int nblk, cudaStream_t st, const Sink &sink);
 
 // bz_batch.cu: terms per item of a batch of one-term-per-SM items; asked <= 0: chosen

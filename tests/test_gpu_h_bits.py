@@ -54,3 +54,21 @@ def test_fp64_is_fp64(dim, N, data):
         f[(1,) + (0,) * (dim - 1)] = eps
     q, ref = _collides(dim, N, data, torch.from_numpy(f).cuda())
     assert not torch.equal(q, ref)
+
+
+@pytest.mark.parametrize("dtype", [torch.complex64, torch.complex128])
+def test_fp32_h_of_real_data(dtype):
+    """BZ_H_FP32 of real data at N = 32 takes the launches of the other arithmetics (h and the kernel's inputs in two) and
+    stays within 2.5e-5 of max |Q| of them on data that the grid does not resolve."""
+    import paper_2004_11239_gb300 as bz
+    f = torch.from_numpy(bi.random_mixture(32, L, seed=63)).cuda().to(dtype)
+    out = []
+    for h in (bz.BZ_H_AUTO, bz.BZ_H_FP32):
+        plan = bz.bz_plan_create_ex(32, L, bi.R_from_L(L), -1.0, 0.5, 2, 12, data=bz.BZ_DATA_REAL, h_precision=h)
+        q = torch.empty_like(f)
+        bz.bz_collide(plan, f, q)
+        assert bz.bz_plan_last_launches(plan) == 4
+        out.append(q)
+        plan.close()
+    err = float((out[0] - out[1]).abs().max() / out[0].abs().max())
+    assert 0 < err <= 2.5e-5, err
