@@ -79,10 +79,19 @@ std::vector<float2> make_twiddles(const bz::Plan &pl) {
 
 // The plans of k_col32 and k_cube32: one CTA per SM, nothing to select.  tuned_ms is one timed collide of a zero field.
 bz_status setup_one_sm(bz::Plan &pl) {
+    const size_t n3 = bz::modes(pl), field = n3 * sizeof(float2);
+    pl.col32 = pl.real;
+    pl.cube32 = !pl.real;
     int G = 0;
     if ((pl.col32 ? bz::col32_setup(&G) : bz::cube32_setup(&G)) != cudaSuccess || G <= 0) return BZ_ERR_CUDA;
-    const size_t part = (size_t)G * (pl.col32 ? bz::kCol32Part : bz::modes(pl)) * sizeof(float2);
-    if (dmalloc(&pl.part, part) != BZ_OK) return BZ_ERR_OOM;
+    const size_t part = (size_t)G * (pl.col32 ? bz::kCol32Part : n3) * sizeof(float2);
+    if (dmalloc(&pl.acol, (size_t)pl.P * (pl.col32 ? bz::kCol32Part * sizeof(float2) : field)) != BZ_OK ||
+        dmalloc(&pl.fcol, field) != BZ_OK || dmalloc(&pl.hcol, field) != BZ_OK ||
+        (pl.real && dmalloc(&pl.fsym, field) != BZ_OK) || dmalloc(&pl.fin64, n3 * sizeof(double2)) != BZ_OK ||
+        dmalloc(&pl.scr64, n3 * sizeof(double2)) != BZ_OK || dmalloc(&pl.part, part) != BZ_OK)
+        return BZ_ERR_OOM;
+    if ((pl.col32 ? bz::col32_table(pl) : bz::cube32_table(pl)) != BZ_OK) return BZ_ERR_CUDA;
+    pl.ws_bytes += (pl.real ? 3 : 2) * field + 2 * n3 * sizeof(double2);
     pl.use_fused = 1; pl.fused_C = 1; pl.fused_G = G;
     // (the clusters' sums go where the items' do, which are more)
     if (pl.cube32 && (bz::fused_setup(32, 8, &pl.few_G, false) != cudaSuccess || pl.few_G > G)) {
@@ -107,6 +116,16 @@ bz_status setup_one_sm(bz::Plan &pl) {
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     return s;
+}
+
+// Undoes what a setup_one_sm without enough memory did.
+void drop_one_sm(bz::Plan &pl) {
+    cudaGetLastError();
+    cudaFree(pl.acol); cudaFree(pl.fcol); cudaFree(pl.hcol); cudaFree(pl.fsym);
+    cudaFree(pl.fin64); cudaFree(pl.scr64); cudaFree(pl.part);
+    pl.acol = nullptr; pl.fcol = nullptr; pl.hcol = nullptr; pl.fsym = nullptr;
+    pl.fin64 = nullptr; pl.scr64 = nullptr; pl.part = nullptr;
+    pl.col32 = 0; pl.cube32 = 0;
 }
 
 // Times one full collide of a zero field for each compiled cluster size (or only `forced`)
@@ -263,24 +282,18 @@ bz_status create(bz_plan **out, const bz_plan_desc *d) {
         return BZ_ERR_CUDA;
     }
     s = bz::ftable_build(pl);
-    // real data at N = 32: k_col32, unless a cluster size or a pair kernel is asked for.  RK4 at
-    // P = 1024 took 191 us a collide with the faster of k_fused and k_pair3 (timed here until then).
-    pl.col32 = pl.real && N == 32 && d->pipeline != BZ_PIPE_CHUNKED && d->cluster <= 0 && d->ctas_per_sm <= 0;
-    if (s == BZ_OK && pl.col32) {
-        if ((s = dmalloc(&pl.acol, (size_t)pl.P * bz::kCol32Part * sizeof(float2))) == BZ_OK &&
-            (s = dmalloc(&pl.fcol, field)) == BZ_OK && (s = dmalloc(&pl.hcol, n3 * sizeof(float))) == BZ_OK &&
-            (s = dmalloc(&pl.fsym, field)) == BZ_OK)
-            s = bz::col32_table(pl);
-        pl.ws_bytes += 2 * field + n3 * sizeof(float);
-    }
-    // complex data at N = 32: k_cube32 likewise (FP32 form, h beyond FP32)
-    pl.cube32 = !pl.real && dim == 3 && N == 32 && pl.precision == BZ_PREC_FP32 && pl.h_fp64 &&
-                d->pipeline != BZ_PIPE_CHUNKED && d->cluster <= 0 && d->ctas_per_sm <= 0;
-    if (s == BZ_OK && pl.cube32) {
-        if ((s = dmalloc(&pl.acol, (size_t)pl.P * field)) == BZ_OK && (s = dmalloc(&pl.fcol, field)) == BZ_OK &&
-            (s = dmalloc(&pl.hcol, field)) == BZ_OK)
-            s = bz::cube32_table(pl);
-        pl.ws_bytes += 2 * field;
+    // N = 32 on one SM a term, unless a cluster size or a pair kernel is asked for: k_col32 for real data (RK4 at
+    // P = 1024 took 191 us a collide with the faster of k_fused and k_pair3, 123 with it), k_cube32 for complex
+    // data (FP32 form, h beyond FP32).  They hold the weights a second time, in their order; without
+    // the memory for it the plan takes the cluster kernels.
+    const bool one_sm = dim == 3 && N == 32 && pl.precision == BZ_PREC_FP32 && (pl.real || pl.h_fp64) &&
+                        d->pipeline != BZ_PIPE_CHUNKED && d->cluster <= 0 && d->ctas_per_sm <= 0;
+    if (s == BZ_OK && one_sm) {
+        s = setup_one_sm(pl);
+        if (s == BZ_ERR_OOM) {
+            drop_one_sm(pl);
+            s = BZ_OK;
+        }
     }
     if (s == BZ_OK && pl.real && !pl.col32) {
         // term pairs (2q, 2q + 1) share a radial node (M even) and one pair of transforms
@@ -314,20 +327,11 @@ bz_status create(bz_plan **out, const bz_plan_desc *d) {
     }
     // pipeline: the fused cluster kernel where it applies (cluster size timed on this
     // device, fastest kept), else the chunked kernels
-    if (d->pipeline != BZ_PIPE_CHUNKED && N <= 32) {
+    if (d->pipeline != BZ_PIPE_CHUNKED && N <= 32 && !pl.use_fused) {
         if (dmalloc(&pl.fin64, n3 * sizeof(double2)) == BZ_OK && dmalloc(&pl.scr64, n3 * sizeof(double2)) == BZ_OK) {
             pl.ws_bytes += 2 * n3 * sizeof(double2);
-            if (pl.col32 || pl.cube32) s = setup_one_sm(pl);
-            else if (select_fused(pl, d->cluster, d->ctas_per_sm) != BZ_OK) cudaGetLastError();
-        } else if (pl.col32 || pl.cube32) {
-            s = BZ_ERR_OOM;
+            if (select_fused(pl, d->cluster, d->ctas_per_sm) != BZ_OK) cudaGetLastError();
         }
-    }
-    if (s != BZ_OK) {                         // these plans have no other pipeline's tables
-        cudaGetLastError();
-        free_plan(pl);
-        delete h;
-        return s;
     }
     if ((d->pipeline == BZ_PIPE_FUSED || pl.precision == BZ_PREC_BF16X3) && !pl.use_fused) {
         free_plan(pl);
