@@ -11,6 +11,7 @@
 // h = IFFT(fhat) is formed once per call by plane_inv without twiddles plus an
 // inverse-only pencil pass.  Inverse transforms are unnormalised; alpha carries N^-3.
 #include <algorithm>
+#include <cstdint>
 #include <cstdio>
 
 #include "bz_fft.cuh"
@@ -555,6 +556,11 @@ static bz_status load_input(Plan &pl, const void *fhat, int dtype, cudaStream_t 
         pl.src_dtype = BZ_C128;
         if (launches) *launches += 1;
         return BZ_OK;
+    }
+    if (dtype == BZ_C64 && (uintptr_t)fhat % sizeof(float2)) {
+        // an array of floats at an odd place: the kernels read pairs, so it is copied
+        BZ_CUDA_TRY(cudaMemcpyAsync(pl.fin, fhat, (size_t)n3 * sizeof(float2), cudaMemcpyDeviceToDevice, st));
+        fhat = pl.fin;
     }
     pl.src = fhat;
     pl.src_dtype = dtype;
