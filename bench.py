@@ -747,7 +747,7 @@ def run_ours(args, w):
 
     plan = make_plan(data_form)
     pipe = bz.bz_plan_pipeline(plan)
-    pipe["h_precision"] = {0: "fp64", 1: "fp64", 2: "fp32"}[args.h_precision]
+    pipe["h_precision"] = {0: "double-float", 1: "fp64", 2: "fp32"}[args.h_precision]
     f_host = _fhat(w, L)
     f = torch.from_numpy(f_host).to("cuda")
     q = torch.empty_like(f)
@@ -812,8 +812,7 @@ def run_ours(args, w):
                                        _profile_key(bz.bz_plan_pipeline(po)["kernel"], not real))}
         po.close()
 
-    # the same workload with h formed in FP32 too: FP64 only in the weight tables, the RK state
-    # and the moments
+    # the same workload with h formed in FP32 too
     pure = None
     if args.workload == "rk4_n32" and real and args.h_precision != 2 and not args.no_other_form:
         pp = bz.bz_plan_create_ex(N, L, R, w["gamma"], w["s"], w["N_rho"], w["M"], h_precision=2, data=data_form)
@@ -1315,7 +1314,7 @@ def main():
     ap.add_argument("--ctas-per-sm", type=int, default=0, choices=[0, 2, 3],
                     help="real-data form at N = 32: 2 runs k_fused, 3 k_pair3, 0 k_col32")
     ap.add_argument("--h-precision", type=int, default=0, choices=[0, 1, 2],
-                    help="h = IFFT(fhat) precision on the fused path: 0 auto (FP64), 1 FP64, 2 FP32")
+                    help="h = IFFT(fhat) precision on the fused path: 0 auto (double-float), 1 FP64, 2 FP32")
     args = ap.parse_args()
     w = dict(WORKLOADS[args.workload])
     if args.n_rho > 0:

@@ -74,7 +74,7 @@ enum { BZ_KERNEL_B1 = 3, BZ_KERNEL_B2 = 4, BZ_KERNEL_B3 = 5, BZ_KERNEL_B4 = 6 };
  *                   split as x = x_hi + x_lo and the products x_hi w_hi + x_lo w_hi +
  *                   x_hi w_lo accumulated in FP32 (about 16 significant bits per product);
  *                   twiddles, the product with h, the alpha weighting and the sum over terms
- *                   stay FP32, h is formed in FP64.  Fused pipeline, N = 32 only; other N
+ *                   stay FP32, h is formed beyond FP32.  Fused pipeline, N = 32 only; other N
  *                   or BZ_PIPE_CHUNKED give BZ_ERR_UNSUPPORTED.  Accuracy target: relative
  *                   L-infinity error 1e-3 of max |Qhat|. */
 enum { BZ_PREC_FP32 = 0, BZ_PREC_BF16X3 = 1 };
@@ -122,7 +122,7 @@ enum { BZ_H_AUTO = 0, BZ_H_FP64 = 1, BZ_H_FP32 = 2 };
  *                    exchanges and (nearly) table bytes per term.  3D, FP32, circular, M even;
  *                    the fused pipeline for N = 8, 16, 32, the chunked one for N = 24, 48, 64
  *                    (BZ_PIPE_FUSED with those: BZ_ERR_UNSUPPORTED); bz_collide_terms takes even term bounds;
- *                    batches need h in FP64 (the default); bz_collide_noalloc returns
+ *                    batches need h beyond FP32 (the default); bz_collide_noalloc returns
  *                    BZ_ERR_UNSUPPORTED. */
 enum { BZ_DATA_COMPLEX = 0, BZ_DATA_REAL = 1 };
 
@@ -166,7 +166,7 @@ typedef struct {
                          faster.  Any other plan: must be <= 0 or 2, else BZ_ERR_UNSUPPORTED. */
 } bz_plan_desc;
 
-/* Creates a plan: quadrature terms, the FP64 F table (computed on the device, stored
+/* Creates a plan: quadrature terms, the F table (computed on the device beyond FP32, stored
  * FP32 as alpha_p = c_p F / N^3), twiddle vectors and workspace, on the current CUDA
  * device.  Synchronous.  Sec. 4, eq. approxG; Sec. 4.1.
  * Errors: BZ_ERR_ARG for unsupported N, N_rho < 1, s outside [0, 1), a sphere rule
@@ -222,7 +222,8 @@ bz_status bz_kernel_constants(int kernel, double s, double eps, double *c, doubl
 
 /* Qhat = Q(fhat, fhat) over all terms (eq. realQ).  fhat and Qhat are device arrays
  * of N^3 complex values of the given dtype; fhat != Qhat (BZ_ERR_ARG otherwise).
- * Arithmetic: FP32 FFTs and products, FP64 accumulation over terms. */
+ * Arithmetic: FP32 FFTs and products; each kernel sums its block of terms in FP32, the blocks are added with
+ * compensation and handed on in FP64. */
 bz_status bz_collide(bz_plan *plan, const void *fhat, void *Qhat, int dtype, void *stream);
 
 /* As bz_collide, restricted to terms p0 <= p < p1 (0 <= p0 <= p1 <= P). */
@@ -244,8 +245,9 @@ bz_status bz_moments(bz_plan *plan, const void *fhat, int dtype, double out[5], 
 
 /* F(k, r_i, qhat_j) in FP64 for `count` entries (device arrays): k_idx[3e..3e+2] array
  * indices in [0, N), term[e] in [0, P); out[2e], out[2e+1] = re, im.  Sums the theta rule
- * of the radial node directly; in 3D the plan's table takes the same rule through a Legendre
- * series (they agree to FP64 rounding before the table's FP32 store).  Synchronous. */
+ * of the radial node directly; in 3D the plan's table takes the finest rule of its nodes through a
+ * Legendre series, in double-float arithmetic (about 47 bits) up to 160 terms and FP64 beyond (they agree to
+ * the table's FP32 rounding and 1e-11 of the term's largest weight).  Synchronous. */
 bz_status bz_ftable_entries(bz_plan *plan, int count, const int *k_idx, const int *term,
                             double *out);
 
@@ -261,7 +263,7 @@ const char *bz_status_str(bz_status s);
  * time loop that cannot pay the device synchronisation of cudaMalloc/cudaFree, a host
  * that forbids a library to grow its footprint after start-up).
  * It computes the operator bz_collide computes on the same plan: h = IFFT(fhat) is formed
- * the same way (in FP64 on the fused pipeline unless the plan asks for BZ_H_FP32, in FP32 on
+ * the same way (beyond FP32 on the fused pipeline unless the plan asks for BZ_H_FP32, in FP32 on
  * the chunked one), the terms run through the chunked FP32 kernels and are summed in FP64;
  * results agree within the FP32 pipeline's rounding (the term chunking and summation order
  * differ).  Every scratch buffer lives in one file-scope device array of
@@ -269,7 +271,7 @@ const char *bz_status_str(bz_status s);
  * nothing is allocated or freed.  The plan must have been created beforehand on the
  * current device.
  *   - Size limit: the array holds the FP32 input copy and h (8 N^3 bytes each), the FP64
- *     accumulator (16 N^3), the h pass's scratch where the plan asks for BZ_H_FP64 (16 N^3) and at
+ *     accumulator (16 N^3), the h pass's scratch unless the plan asks for BZ_H_FP32 (16 N^3) and at
  *     least one term of 8 N^3 (each rounded up to 256-byte blocks).  N <= 48 fits (N = 48: five
  *     terms per chunk); N = 64 does not and returns BZ_ERR_ARG without touching Qhat.
  *   - Each call looks up the array's device address (cudaGetSymbolAddress) with the current
@@ -359,7 +361,8 @@ int bz_batch_last_launches(const bz_batch *batch);
 /* Free streaming df/dt + v_1 df/dx = 0 over time t (any sign), in place: exact at the velocity
  * nodes v_j = -L + 2 L j / N and spectral in x (x-DFT over the cells, phase
  * exp(-2 pi i kappa v_1 t / Lx) with the signed x-mode kappa, -nx/2 included, inverse x-DFT),
- * computed in FP64 along the k1 axis only (the phase depends on v_1 alone).  N and nx in
+ * computed along the k1 axis only (the phase depends on v_1 alone), c128 cells in FP64, c64 ones in
+ * double-float arithmetic scaled by a power of two (their error is the rounding of the result).  N and nx in
  * {8, 16, 24, 32}; BZ_ERR_UNSUPPORTED otherwise. */
 bz_status bz_transport_x(int N, double L, int nx, double Lx, void *fcells, int dtype, double t, void *stream);
 

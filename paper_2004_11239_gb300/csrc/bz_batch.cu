@@ -7,7 +7,7 @@
 //
 // State lives in slots [0, capacity); each call names the active slots, so instances can
 // join and leave between steps (continuous batching).  The fused item kernel processes
-// (instance, block of TB terms) items; an instance's result is the fixed-order FP64 sum of
+// (instance, block of TB terms) items; an instance's result is the fixed-order compensated sum of
 // its block partials, independent of the other instances in the call.  One RK4 step
 // (4 x [fused items, stage update]) is captured once per dt into a CUDA graph and replayed;
 // the active count and slot list are read from device memory at run time.
@@ -586,7 +586,7 @@ bz_status bz_batch_create(bz_batch **out, const bz_plan *plan, int capacity, int
     if (!out || !plan || capacity < 1) return BZ_ERR_ARG;
     *out = nullptr;
     Plan *pl = const_cast<Plan *>(plan_internal(plan));
-    // batches: circular 3D plans; on the fused pipeline the real-data form needs h formed in FP64
+    // batches: circular 3D plans; on the fused pipeline the real-data form needs h formed beyond FP32
     if (pl->Nin || pl->dim == 2 || (pl->use_fused && pl->real && !pl->h_fp64)) return BZ_ERR_UNSUPPORTED;
     bz_batch *B = new (std::nothrow) bz_batch();
     if (!B) return BZ_ERR_OOM;

@@ -525,18 +525,10 @@ static bz_status run_chunks(Plan &pl, int p0, int p1, cudaStream_t st, int *laun
     return BZ_OK;
 }
 
-template <int N> static void h_fp32_n(Plan &pl, const float2 *fin, cudaStream_t st) {
-    plane_inv<N, false>(fin, pl.tw, pl.S, 0, 1, 0, st);
-    k_pencil<N, 0><<<dim3((N * N + 127) / 128, 1), 128, 0, st>>>(pl.S, nullptr, pl.h);
-}
-
 bz_status h_fp32(Plan &pl, const float2 *fin, cudaStream_t st) {
-    switch (pl.N) {
-        case 8: h_fp32_n<8>(pl, fin, st); break;
-        case 16: h_fp32_n<16>(pl, fin, st); break;
-        case 32: h_fp32_n<32>(pl, fin, st); break;
-        default: return BZ_ERR_UNSUPPORTED;
-    }
+    if (pl.N != 32) return BZ_ERR_UNSUPPORTED;
+    plane_inv<32, false>(fin, pl.tw, pl.S, 0, 1, 0, st);
+    pencil<32, 0>(pl.S, nullptr, pl.h, 1, st);
     BZ_CUDA_TRY(cudaGetLastError());
     return BZ_OK;
 }
@@ -629,7 +621,7 @@ bz_status collide_range(Plan &pl, int p0, int p1, const void *fhat, void *Qhat, 
 // file-scope device array of kNoallocBytes, which every GPU that loads libbz holds
 // until the process exits.  The caller passes the plan (built beforehand) and the
 // input and output arrays; nothing is allocated or freed during the call.  h is formed as
-// bz_collide forms it on the same plan (FP64 on the fused pipeline unless the plan asks for
+// bz_collide forms it on the same plan (beyond FP32 on the fused pipeline unless the plan asks for
 // FP32 h, FP32 on the chunked one), so both compute the same operator.
 // =======================================================================================
 namespace bz {
@@ -651,8 +643,8 @@ bz_status noalloc_scratch(unsigned char **out) {
 
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
-// Scratch layout (256-byte blocks): fin (8 N^3 bytes), h (8 N^3), acc (16 N^3), the FP64 h
-// pass's scratch where the plan forms h in FP64 (16 N^3), then T terms of 8 N^3.
+// Scratch layout (256-byte blocks): fin (8 N^3 bytes), h (8 N^3), acc (16 N^3), the h
+// pass's scratch where the plan forms h beyond FP32 (16 N^3), then T terms of 8 N^3.
 template <int N>
 bz_status run_noalloc(const Plan &pl, const void *fhat, void *Qhat, int dtype, unsigned char *base,
                       bool h64, int T, cudaStream_t st) {
@@ -712,7 +704,7 @@ extern "C" bz_status bz_collide_noalloc(const bz_plan *plan, const void *fhat, v
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess) return BZ_ERR_CUDA;
     if (dev != pl.device) return BZ_ERR_ARG;
-    // h as bz_collide forms it on this plan: FP64 on the fused pipeline with FP64 h, else FP32
+    // h as bz_collide forms it on this plan: beyond FP32 on the fused pipeline unless FP32 is asked for, else FP32
     const bool h64 = pl.use_fused && pl.h_fp64;
     const size_t n3 = (size_t)pl.N * pl.N * pl.N;
     const size_t field = n3 * sizeof(float2);

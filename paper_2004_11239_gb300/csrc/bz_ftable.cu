@@ -1,4 +1,4 @@
-// FP64 weight table F(k, r_i, qhat_j) on the GPU (Sec. 2.1 eq. FF, Sec. 4.1 split, 3D).
+// Weight table F(k, r_i, qhat_j) on the GPU (Sec. 2.1 eq. FF, Sec. 4.1 split, 3D).
 //
 // With a = pi r / (2L), kappa = k.qhat, kperp = |k - kappa qhat|, x = a kappa, y = a kperp
 // and g(t) = sin(t) b(cos t), the phi integral of eq. FF3D1 is exact (2 pi J0), so
@@ -18,8 +18,11 @@
 //       mu_l = 2 pi sum_n W_n (P_l(cos t_n) - 1).
 //     The rule enters through the mu_l only (one short sum per l on the host), j_l(z) depends on
 //     (r_i, |k|^2) only (k_legendre_coef, one row per radial node and |k|^2), and an entry is a
-//     Legendre series of about z + 25 terms of three FP64 operations, against a few hundred rule
-//     nodes of some hundred operations each.
+//     Legendre series of about z + 25 terms of three operations (in double-float arithmetic up to 160
+//     terms, in FP64 beyond), against a few hundred rule nodes of some hundred operations each.  The
+//     mu_l come from the finest rule of the plan's nodes.  Measured over N = 8 .. 64, three
+//     potentials and gammas: the FP32 table has the error against 64 bits that the direct FP64 sums gave
+//     it, in the 2-norm, the largest entry and entry by entry.
 #include <cmath>
 #include <cstring>
 #include <vector>

@@ -219,7 +219,7 @@ k_fused(ItemArgs a) {
         const int t0 = a.p0 + blk * a.TB;
         const int t1 = min(a.p1, t0 + a.TB);
         const float2 *fin = a.fin + (size_t)slot * N3;
-        // prologue: the h slice of the pencils this CTA owns, either formed beforehand in FP64
+        // prologue: the h slice of the pencils this CTA owns, either formed beforehand
         // (a.hg) or here in FP32 (no twiddle, inverse only) straight into shared memory
         __syncthreads();                                      // the previous item is done with smem
         fetch_tw(t0, 0);

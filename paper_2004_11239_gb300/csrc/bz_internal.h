@@ -67,7 +67,7 @@ struct Plan {
     float2 *fcopy = nullptr;        // where the h pass stores it (complex128 callers), or null
     double2 *acc = nullptr;         // [N^3] FP64 accumulator (while a chunked collide runs, the same
                                     // bytes hold k_reduce's compensated FP32 state: s, c per mode pair)
-    double2 *rk = nullptr;          // [3][N^3] RK4 state (f0, fsum) + spare
+    double2 *rk = nullptr;          // [2][N^3] RK4 state (f0, fsum)
     double *mom = nullptr;          // moments scratch
     // fused cluster pipeline (N <= 32)
     int use_fused = 0;              // 1: bz_collide runs k_fused
@@ -222,7 +222,7 @@ inline Sink acc_sink(Plan &pl) {
     s.acc = pl.acc;
     return s;
 }
-// pl.h = IFFT(fin) in FP32 (one plane pass and one pencil pass through pl.S; N = 8, 16, 32)
+// pl.h = IFFT(fin) in FP32 (one plane pass and one pencil pass through pl.S; N = 32: k_pair3)
 bz_status h_fp32(Plan &pl, const float2 *fin, cudaStream_t st);
 
 // bz_fused.cu
@@ -234,7 +234,7 @@ struct ItemArgs {
     const float2 *alpha = nullptr;   // [P][N^3]
     const float *gsc = nullptr;      // [slots][N_rho] radial scale r_i^(gamma_b - gamma_plan), or null
     float2 *part = nullptr;          // [slots][nblk][N^3] per-item partial sums
-    const float2 *hg = nullptr;      // [slots][N^3] h = IFFT(fhat), formed in FP64, stored FP32
+    const float2 *hg = nullptr;      // [slots][N^3] h = IFFT(fhat), stored FP32; null: formed in the kernel in FP32
     const int *slots = nullptr;      // device [count] or null
     const int *count_dev = nullptr;  // device instance count, or null (use count)
     int count = 1, p0 = 0, p1 = 0, TB = 1, nblk = 0, M = 1, N_rho = 1;
