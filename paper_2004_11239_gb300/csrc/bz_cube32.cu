@@ -15,7 +15,7 @@
 // The sums of column w stay in tensor memory (64 words a thread, as the waiting half: all of it), those of
 // column w + 16 in the item's place of the partial sums, which is in L2.  Input [k3][k1][k2], h and its product
 // [j3][j1][j2], table and sums [k3][k1][k2].
-// Measured at P = 1024: 179 us, k_fused (8-CTA clusters) 290.  A term takes 52 k clocks, some 28 k of them issue
+// Measured at P = 1024: 179 us, k_fused (8-CTA clusters) 302.  A term takes 52 k clocks, some 28 k of them issue
 // slots; bound as k_col32 by issue, the block barriers (four a term) and L2 latency (1 MB a term: fhat, h,
 // weights and the second column's sums).
 #include "bz_cluster.cuh"
