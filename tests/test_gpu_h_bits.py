@@ -72,3 +72,25 @@ def test_fp32_h_of_real_data(dtype):
         plan.close()
     err = float((out[0] - out[1]).abs().max() / out[0].abs().max())
     assert 0 < err <= 2.5e-5, err
+
+
+@pytest.mark.parametrize("data", [0, 1])
+@pytest.mark.parametrize("dtype", [torch.complex64, torch.complex128])
+def test_fp64_on_one_sm_kernels_and_batches(data, dtype):
+    """At N = 32 with enough terms for k_cube32 (its layouts of fhat and h), and of two slots of a batch."""
+    import paper_2004_11239_gb300 as bz
+    f = torch.stack([torch.from_numpy(bi.random_mixture(32, L, seed=s)) for s in (63, 64, 65)]).cuda().to(dtype)
+    out = []
+    for h in (bz.BZ_H_AUTO, bz.BZ_H_FP64):
+        plan = bz.bz_plan_create_ex(32, L, bi.R_from_L(L), 0.0, 0.5, 4, 12, data=data, h_precision=h)
+        one, q = torch.empty_like(f[0]), torch.zeros_like(f)
+        bz.bz_collide(plan, f[0].clone(), one)
+        batch = bz.bz_batch_create(plan, 3, 0)
+        bz.bz_batch_collide(batch, [2, 0], f, q)
+        batch.close()
+        plan.close()
+        out.append((one, q))
+    for a, b in zip(*out):
+        assert float((a - b).abs().max() / b.abs().max()) <= 2.0 ** -24
+    assert not out[1][1][1].any() and out[1][1][2].any()
+    assert float((out[1][0] - out[1][1][0]).abs().max() / out[1][0].abs().max()) <= 1e-6
